@@ -220,6 +220,9 @@ cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint
                               int nr, int lpad, int64_t nkeys, char* tab, int prec, cudaStream_t st);
 cudaError_t launch_sketch_sp(const Plan& P, int item, const void* X, int64_t first, int64_t count, void* ws,
                              cudaStream_t st);
+bool use_strip_kernel(const Plan& P, int item, int64_t count);
+cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t first, int64_t count, void* ws,
+                                cudaStream_t st);
 bool sp_batched_eligible(const Plan& P, size_t* smem_out, int* lpad_out, int t3max = 4);
 cudaError_t launch_sketch_sp_batched(const Plan& P, const void* const* X, const BatchCfg& cfg, void* ws,
                                      cudaStream_t st);

@@ -1498,6 +1498,7 @@ cudaError_t launch_sketch_mixed(const Plan& P, int item, const void* X, int64_t 
     if (e != cudaErrorNotSupported) return e;
   }
   if (use_sp_kernel(P, item, count)) return launch_sketch_sp(P, item, X, first, count, ws, st);
+  if (use_strip_kernel(P, item, count)) return launch_sketch_strip(P, item, X, first, count, ws, st);
   return launch_sketch_mma(P, item, X, first, count, ws, st);
 }
 
