@@ -3,9 +3,11 @@
 //
 // The cores are contracted into a left interface L_{d*} (N_{d*} x r_{d*}) and a
 // right interface Rt_{d*+1} (r_{d*} x M_{d*}); then X~ = L_{d*} Rt_{d*+1} seen as
-// the middle unfolding, one thread per entry (FP64).
+// the middle unfolding: digit arithmetic on the tensor cores for larger FP32 data
+// (expand.cuh), else one thread per entry (FP64).
 #include <algorithm>
 
+#include "expand.cuh"
 #include "internal.cuh"
 
 namespace tts {
@@ -210,6 +212,41 @@ cudaError_t build_interfaces(const Plan& P, int item, const double* cores, void*
   return cudaGetLastError();
 }
 
+namespace {
+
+template <int P, int KS, int UT, int NTL, int MODE>
+cudaError_t run_expand(expand::ExpandArgs a, cudaStream_t st) {
+  a.nub = (a.Nm + UT - 1) / UT;
+  // columns per CTA: about eight CTAs per SM, whole staging steps
+  const int64_t want = std::max<int64_t>(1, 8LL * device_sm_count() / a.nub);
+  a.vlen = ((a.Mm + want - 1) / want + expand::kVT - 1) / expand::kVT * expand::kVT;
+  const int64_t ctas = a.nub * ((a.Mm + a.vlen - 1) / a.vlen);
+  constexpr int LD = 16 * std::max(KS, 1) + 8, PA = KS ? P : (P + 1) / 2;
+  const size_t smem = 2ul * (P * UT + PA * expand::kVT) * LD + sizeof(int) * (2 * UT + expand::kVT);
+  auto k = expand::expand_kernel<P, KS, UT, NTL, MODE>;
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  count_launch();
+  k<<<(unsigned)ctas, expand::kThreads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+template <int P, int NTL, int MODE>
+cudaError_t run_expand_ks(const expand::ExpandArgs& a, cudaStream_t st) {
+  if (a.rp <= 8) return run_expand<P, 0, 256, NTL, MODE>(a, st);
+  switch ((a.rp + 15) / 16) {
+    case 1: return run_expand<P, 1, 256, NTL, MODE>(a, st);
+    case 2: return run_expand<P, 2, 128, NTL, MODE>(a, st);
+    case 3: return run_expand<P, 3, 128, NTL, MODE>(a, st);
+    default: return run_expand<P, 4, 128, NTL, MODE>(a, st);
+  }
+}
+
+}  // namespace
+
 cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, void* Xt, int x_f64,
                                const void* Xcmp, int cmp_f64, double* out2, void* ws,
                                cudaStream_t st) {
@@ -223,6 +260,26 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
   double* W = (double*)ws;
   const int ds = it.ds;
   const int64_t Nm = it.N[ds], Mm = it.N[it.d] / it.N[ds];
+  // Digit arithmetic (expand.cuh) for FP32 data from 3 2^18 entries on, with both
+  // interfaces at least as long as a staging step.  Measured (whole call, us, FP64
+  // kernel -> digit kernel): below the line 64^3 rank 2: 8 -> 11, 9^6 rank 8: 23 ->
+  // 26; above it 1000 x 1000 rank 3: 12.8 -> 12.2, 100^3 rank 10: 28 -> 17, 128^3
+  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 4750 (3.6 TB/s
+  // of the output; the epilogue and the digit products share the issue slots);
+  // error sums 24^6 rank 10: 4590 -> 859.
+  if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && Nm * Mm >= (3 << 18)) {
+    expand::ExpandArgs a;
+    a.L = W + it.off_L[ds];
+    a.Rt = W + it.off_Rt[ds + 1];
+    a.Nm = Nm;
+    a.Mm = Mm;
+    a.rp = it.rpad[ds];
+    a.out = (float*)Xt;
+    a.X = (const float*)Xcmp;
+    a.out2 = out2;
+    a.vec = Nm % 4 == 0 && ((uintptr_t)(Xt ? Xt : Xcmp) & 15) == 0 ? 1 : 0;
+    return Xt ? run_expand_ks<5, 4, 0>(a, st) : run_expand_ks<7, 2, 1>(a, st);
+  }
   count_launch();
   dense_kernel<<<grid_for(Nm * Mm), kThreads, 0, st>>>(W + it.off_L[ds], W + it.off_Rt[ds + 1], Nm, Mm,
                                                        it.rpad[ds], Xt, x_f64, Xcmp, cmp_f64, out2);
