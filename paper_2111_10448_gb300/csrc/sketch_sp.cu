@@ -572,7 +572,11 @@ __global__ void __launch_bounds__(Prec<FMT>::kThreads, 1) sketch_sp_kernel(const
 
 // Batched form: persistent CTAs take `chunk` consecutive units (item, block)
 // of the largest-first unit sequence at a time; row slots are flushed after
-// every unit, the others when the item or the kL block changes.
+// every unit, the others when the item or the kL block changes.  LPAD = 0: a
+// batch with items of both padded widths, each served at its own (512 tensors
+// with ranks 2..16 and p = 5: a call takes 32 ms, 113 ms on the 64 x 32 tile
+// kernel, which took such batches before).
+
 template <int LPAD, int FMT>
 __global__ void __launch_bounds__(Prec<FMT>::kThreads, 1) sketch_sp_batched_kernel(const BatchLaunch b) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -589,6 +593,12 @@ __global__ void __launch_bounds__(Prec<FMT>::kThreads, 1) sketch_sp_batched_kern
   float* acc = reinterpret_cast<float*>(smraw + Prec<FMT>::kWarps * Prec<FMT>::kWarpBytes);
   sp_zero<FMT>(smraw, acc, 0);
   int cur = -1;
+  auto lpad = [&]() { return LPAD ? LPAD : g.ell <= 16 ? 16 : 32; };
+  auto flush = [&](bool long_class, int64_t bL, int64_t bR) {
+    if constexpr (LPAD != 0) sp_flush<LPAD, FMT>(g, g.sk, acc, long_class, bL, bR);
+    else if (g.ell <= 16) sp_flush<16, FMT>(g, g.sk, acc, long_class, bL, bR);
+    else sp_flush<32, FMT>(g, g.sk, acc, long_class, bL, bR);
+  };
   int64_t cur_bL = -1;
   int age = 0;
   for (;;) {
@@ -617,7 +627,7 @@ __global__ void __launch_bounds__(Prec<FMT>::kThreads, 1) sketch_sp_batched_kern
       // while the item and the kL block stay the same, for at most
       // kColFlushBlocks units
       if (cur >= 0 && (it_idx != cur || lu / g.tilesR != cur_bL || age == kColFlushBlocks)) {
-        sp_flush<LPAD, FMT>(g, g.sk, acc, true, cur_bL, 0);
+        flush(true, cur_bL, 0);
         __syncthreads();
         age = 0;
         cur_bL = -1;
@@ -633,20 +643,23 @@ __global__ void __launch_bounds__(Prec<FMT>::kThreads, 1) sketch_sp_batched_kern
         }
         __syncthreads();
         // slots of this item start at zero (every unit is flushed completely)
-        for (int i = threadIdx.x; i < g.nslots * LPAD * g.ldo; i += Prec<FMT>::kThreads) acc[i] = 0.0f;
+        for (int i = threadIdx.x; i < g.nslots * lpad() * g.ldo; i += Prec<FMT>::kThreads) acc[i] = 0.0f;
         __syncthreads();
         cur = it_idx;
       }
       const int64_t bL = lu / g.tilesR, bR = lu - bL * g.tilesR;
       cur_bL = bL;
       ++age;
-      sp_block<LPAD, FMT, false>(g, g.sk, smraw, acc, bL, bR);  // batched plans refuse Khatri-Rao
+      // batched plans refuse Khatri-Rao
+      if constexpr (LPAD != 0) sp_block<LPAD, FMT, false>(g, g.sk, smraw, acc, bL, bR);
+      else if (g.ell <= 16) sp_block<16, FMT, false>(g, g.sk, smraw, acc, bL, bR);
+      else sp_block<32, FMT, false>(g, g.sk, smraw, acc, bL, bR);
       __syncthreads();
-      sp_flush<LPAD, FMT>(g, g.sk, acc, false, bL, bR);
+      flush(false, bL, bR);
       __syncthreads();
     }
   }
-  if (cur >= 0 && cur_bL >= 0) sp_flush<LPAD, FMT>(g, g.sk, acc, true, cur_bL, 0);
+  if (cur >= 0 && cur_bL >= 0) flush(true, cur_bL, 0);
 }
 
 // Batched tables: blockIdx.y = item; its staged sketches one after another.
@@ -796,12 +809,13 @@ cudaError_t launch_sketch_sp(const Plan& P, int item, const void* X, int64_t fir
   return cudaGetLastError();
 }
 
-// Batched form: every item must fit the small-plane kernel with the same
-// padded width (the tables and tiles of a launch share it).
+// Batched form: every item must fit the small-plane kernel (*lpad_out = 0 when
+// their padded widths differ).
 bool sp_batched_eligible(const Plan& P, size_t* smem_out, int* lpad_out, int t3max) {
   const int n = plan_num_items(&P);
   size_t smem = 0;
   int lpad = 0;
+  bool mixed = false;
   for (int i = 0; i < n; ++i) {
     const DevItem& it = plan_items_host(&P)[i];
     if (it.prec != plan_items_host(&P)[0].prec) return false;
@@ -809,12 +823,12 @@ bool sp_batched_eligible(const Plan& P, size_t* smem_out, int* lpad_out, int t3m
     size_t need = 0;
     if (!sp::plan_sp(P, i, it.n[it.d - 1], &g, &need, t3max)) return false;
     const int lp = g.ell <= 16 ? 16 : 32;
-    if (lpad && lp != lpad) return false;
+    mixed = mixed || (lpad && lp != lpad);
     lpad = lp;
     smem = std::max(smem, need);
   }
   if (smem_out) *smem_out = smem;
-  if (lpad_out) *lpad_out = lpad;
+  if (lpad_out) *lpad_out = mixed ? 0 : lpad;
   return n > 0 && n <= kMaxBatchItems;
 }
 
@@ -832,15 +846,18 @@ cudaError_t launch_sketch_sp_batched(const Plan& P, const void* const* X, const 
   b.t3max = t3max;
   for (int i = 0; i < nitems; ++i) b.X[i] = X[i];
   using KernelFn = void (*)(const BatchLaunch);
-  const KernelFn kernels[3][2] = {
-      {sp::sketch_sp_batched_kernel<16, sp::kFmtBF16>, sp::sketch_sp_batched_kernel<32, sp::kFmtBF16>},
-      {sp::sketch_sp_batched_kernel<16, sp::kFmtTF32>, sp::sketch_sp_batched_kernel<32, sp::kFmtTF32>},
-      {sp::sketch_sp_batched_kernel<16, sp::kFmtFP16>, sp::sketch_sp_batched_kernel<32, sp::kFmtFP16>}};
+  const KernelFn kernels[3][3] = {
+      {sp::sketch_sp_batched_kernel<16, sp::kFmtBF16>, sp::sketch_sp_batched_kernel<32, sp::kFmtBF16>,
+       sp::sketch_sp_batched_kernel<0, sp::kFmtBF16>},
+      {sp::sketch_sp_batched_kernel<16, sp::kFmtTF32>, sp::sketch_sp_batched_kernel<32, sp::kFmtTF32>,
+       sp::sketch_sp_batched_kernel<0, sp::kFmtTF32>},
+      {sp::sketch_sp_batched_kernel<16, sp::kFmtFP16>, sp::sketch_sp_batched_kernel<32, sp::kFmtFP16>,
+       sp::sketch_sp_batched_kernel<0, sp::kFmtFP16>}};
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaSuccess;
     for (int f = 0; f < 3; ++f)
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < 3; ++i)
         if (e == cudaSuccess)
           e = cudaFuncSetAttribute(kernels[f][i], cudaFuncAttributeMaxDynamicSharedMemorySize, sp::kMaxSmem);
     if (e != cudaSuccess) {
@@ -857,7 +874,7 @@ cudaError_t launch_sketch_sp_batched(const Plan& P, const void* const* X, const 
   count_launch();
   const int nsm = device_sm_count();
   const int threads = fmt == sp::kFmtTF32 ? sp::Prec<sp::kFmtTF32>::kThreads : sp::Prec<sp::kFmtBF16>::kThreads;
-  kernels[fmt][lpad == 16 ? 0 : 1]<<<nsm, threads, smem, st>>>(b);
+  kernels[fmt][lpad == 16 ? 0 : lpad == 32 ? 1 : 2]<<<nsm, threads, smem, st>>>(b);
   return cudaGetLastError();
 }
 
