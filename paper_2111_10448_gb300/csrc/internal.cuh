@@ -131,10 +131,9 @@ struct DevItem {
   int64_t off_bbar;         // adjoint of B
   int64_t off_rr[TT_MAXD + 1];    // leading r x r block of the basis R factor (rpad x rpad)
   int64_t off_small;        // 4 x TT_MAXL^2 doubles of backward scratch (single-item plans)
-  int diff;                 // TT_FLAG_DIFF: full interface chain reserved
-  int64_t off_Lall[TT_MAXD + 1];  // left interfaces L_k, k = 1..d-1 (N_k x rpad_k)
-  int64_t off_Rall[TT_MAXD + 2];  // right interfaces Rt_k, k = 2..d (rpad_{k-1} x M_{k-1})
-  int64_t off_Y;            // max_k N_k x rpad_k
+  int diff;                 // TT_FLAG_DIFF: the reconstruction's adjoint has its workspace
+  int64_t off_Z[TT_MAXD + 1];     // Z_k, k = 1..ds (N_k x rpad_k): dX with the cores past k absorbed
+  int64_t off_Wd[TT_MAXD + 1];    // W_k, k = ds..d-1 (rpad_k x M_k): dX with the cores up to k absorbed
   int64_t off_tctab;        // plane kernel: staged test-matrix blocks shared by many planes
   int64_t tctab_doubles;    // its size (0 when the plane kernel cannot serve the item)
   int64_t off_sptab;        // small-plane kernel: staged test-matrix rows of the sketches

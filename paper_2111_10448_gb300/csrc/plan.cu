@@ -450,11 +450,8 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   it.diff = (q.flags & TT_FLAG_DIFF) ? 1 : 0;
   it.short_chains = (q.flags & TT_FLAG_SHORT_CHAINS) ? 1 : 0;
   if (it.diff) {
-    int64_t ymax = 1;
-    for (int k = 1; k < d; ++k) it.off_Lall[k] = ws.take(it.N[k] * it.rpad[k]);
-    for (int k = 2; k <= d; ++k) it.off_Rall[k] = ws.take((int64_t)it.rpad[k - 1] * (it.N[d] / it.N[k - 1]));
-    for (int k = 1; k <= d; ++k) ymax = std::max<int64_t>(ymax, it.N[k] * it.rpad[k]);
-    it.off_Y = ws.take(ymax);
+    for (int k = 1; k <= ds; ++k) it.off_Z[k] = ws.take(it.N[k] * it.rpad[k]);
+    for (int k = ds; k < d; ++k) it.off_Wd[k] = ws.take((int64_t)it.rpad[k] * (it.N[d] / it.N[k]));
   }
   P.items.push_back(it);
   return TT_OK;

@@ -150,6 +150,108 @@ __global__ void __launch_bounds__(128) ygram_kernel(const void* dX, int dx_f64, 
   }
 }
 
+// W(c, v) += sum_u L(u, c) dX(u + Nk v)   (L: Nk x rp; W: rp x Mk).  A warp takes V
+// columns v and uc rows u, its lanes the rows: RP V sums per lane, folded over the
+// lanes by a halving butterfly that leaves sum j on lane j (mod 32), one FP64
+// atomic each.  Like ygram_kernel it is bound by the FP64 pipe: one FMA per entry
+// and rank.
+template <int RP, int V>
+__global__ void __launch_bounds__(128) wgram_kernel(const void* dX, int dx_f64, int64_t Nk, int64_t Mk, const double* L,
+                                                    int rp, double* W, int64_t uc) {
+  constexpr int NS = RP * V;
+  const int lane = threadIdx.x & 31;
+  const int64_t nvg = (Mk + V - 1) / V, nuc = (Nk + uc - 1) / uc;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t job = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); job < nvg * nuc; job += nwarps) {
+    const int64_t v0 = (job % nvg) * V, u0 = (job / nvg) * uc, u1 = imin64(Nk, u0 + uc);
+    double acc[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) acc[j] = 0.0;
+    for (int64_t u = u0 + lane; u < u1; u += 32) {
+      double x[V];
+#pragma unroll
+      for (int q = 0; q < V; ++q) {
+        const int64_t e = u + Nk * imin64(v0 + q, Mk - 1);   // a column past the end is dropped below
+        x[q] = dx_f64 ? __ldg((const double*)dX + e) : (double)__ldg((const float*)dX + e);
+      }
+#pragma unroll
+      for (int c = 0; c < RP; ++c) {
+        const double l = __ldg(L + u + Nk * min(c, rp - 1));
+#pragma unroll
+        for (int q = 0; q < V; ++q) acc[q * RP + c] = fma(l, x[q], acc[q * RP + c]);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < NS; b += 32) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+          const double keep = up ? acc[b + j + o] : acc[b + j], send = up ? acc[b + j] : acc[b + j + o];
+          acc[b + j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      }
+      const int j = b + lane, c = j % RP;
+      const int64_t v = v0 + j / RP;
+      if (c < rp && v < Mk) atomicAdd(W + c + (int64_t)rp * v, acc[b]);
+    }
+  }
+}
+
+// Z_{k-1}(u, a) = sum_{i, c} Z_k(u + N_{k-1} i, c) G_k(a, i, c): one warp per entry,
+// the lanes over (i, c).
+__global__ void zdown_kernel(const double* Z, int64_t Np, int64_t nk, int rpc, const double* G, int rpa, double* Zo) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5), Nk = Np * nk, len = nk * rpc;
+  for (int64_t job = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); job < Np * rpa; job += nwarps) {
+    const int64_t u = job % Np;
+    const int a = (int)(job / Np);
+    double acc = 0.0;
+    for (int64_t j = lane; j < len; j += 32) {
+      const int64_t i = j % nk, c = j / nk;
+      acc = fma(Z[u + Np * i + Nk * c], G[a + (int64_t)rpa * j], acc);   // j = i + n_k c
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) Zo[u + Np * a] = acc;
+  }
+}
+
+// W_k(c, v) = sum_{a, i} G_k(a, i, c) W_{k-1}(a, i + n_k v): one warp per entry, the
+// lanes over (a, i).
+__global__ void wup_kernel(const double* Wp, int rpa, int64_t nk, int64_t Mk, const double* G, int rpc, double* Wo) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5), len = (int64_t)rpa * nk;
+  for (int64_t job = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); job < Mk * rpc; job += nwarps) {
+    const int c = (int)(job % rpc);
+    const int64_t v = job / rpc;
+    double acc = 0.0;
+    for (int64_t j = lane; j < len; j += 32) acc = fma(G[j + len * c], Wp[j + len * v], acc);
+    acc = warp_sum(acc);
+    if (lane == 0) Wo[c + (int64_t)rpc * v] = acc;
+  }
+}
+
+// dG_k(a, i, c) = sum_v W_{k-1}(a, i + n_k v) Rt_{k+1}(c, v) (Rt = null: one v, 1): one
+// warp per entry, the lanes over v.
+__global__ void dcore_right_kernel(const double* Wp, int rpa, int64_t nk, int64_t Mk, const double* Rt, int rpc,
+                                   double* dG) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5), len = (int64_t)rpa * nk;
+  for (int64_t job = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); job < len * rpc; job += nwarps) {
+    const int64_t ai = job % len;
+    const int c = (int)(job / len);
+    double acc = 0.0;
+    if (Rt == nullptr) {
+      if (lane == 0) dG[job] = Wp[ai];
+      continue;
+    }
+    for (int64_t v = lane; v < Mk; v += 32) acc = fma(Wp[ai + len * v], Rt[c + (int64_t)rpc * v], acc);
+    acc = warp_sum(acc);
+    if (lane == 0) dG[job] = acc;
+  }
+}
+
 // dG_k(a, i, c) = sum_u L_{k-1}(u, a) Y_k(u + N_{k-1} i, c);  L_0 = [1].
 // dG is zeroed first; a warp takes one entry and one chunk of u (lanes split
 // the chunk) and adds its sum with an atomic.
@@ -288,62 +390,92 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
 
 // Adjoint of the reconstruction: for every core k,
 //   dG_k(a, i, c) = sum_{u, v} L_{k-1}(u, a) dX(u + N_{k-1} i + N_k v) Rt_{k+1}(c, v)
-// with the left / right interfaces of the train (all of them: TT_FLAG_DIFF).
+// with the left / right interfaces of the train.  dX is contracted twice, at the
+// middle: Z_ds = dX Rt_{ds+1}^T for the cores up to ds, W_ds = L_ds^T dX for the
+// others; from there the cores absorb one mode at a time (Z_{k-1} from Z_k and G_k,
+// W_k from W_{k-1} and G_k), so only these two products see every entry (2 N r
+// FMAs).  One contraction per core (d N r FMAs, and the interfaces of length
+// N_{d-1}) took 4.5 ms for 32^5 of rank 8; this takes 1.2 ms, 1.1 of them FP64-pipe
+// time of the two products.
 cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* cores, const void* dXt,
                                         int dx_f64, double* dcores, void* ws, cudaStream_t st) {
   const DevItem& it = plan_items_host(&P)[item];
   double* W = (double*)ws;
-  const int d = it.d;
-  for (int k = 1; k < d; ++k) {
-    const double* Lp = k == 1 ? nullptr : W + it.off_Lall[k - 1];
-    count_launch();
-    iface_left_kernel<<<grid_for(it.N[k] * it.rpad[k]), kThreads, 0, st>>>(
-        Lp, it.N[k - 1], it.rpad[k - 1], cores + it.core_off[k], it.n[k - 1], it.rpad[k], W + it.off_Lall[k]);
-  }
-  for (int k = d; k >= 2; --k) {
-    const double* Rn = k == d ? nullptr : W + it.off_Rall[k + 1];
-    const int64_t Mn = it.N[d] / it.N[k];
-    count_launch();
-    iface_right_kernel<<<grid_for((int64_t)it.rpad[k - 1] * it.n[k - 1] * Mn), kThreads, 0, st>>>(
-        Rn, Mn, it.rpad[k], cores + it.core_off[k], it.n[k - 1], it.rpad[k - 1], W + it.off_Rall[k]);
-  }
+  const int d = it.d, ds = it.ds;
+  cudaError_t e = build_interfaces(P, item, cores, ws, st);
+  if (e != cudaSuccess) return e;
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(ygram_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         4 * 64 * 32 * (int)sizeof(double));
+    e = cudaFuncSetAttribute(ygram_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             4 * 64 * 32 * (int)sizeof(double));
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  for (int k = 1; k <= d; ++k) {
-    const int64_t Nk = it.N[k], Mk = it.N[d] / it.N[k];
-    const int rpk = it.rpad[k];
-    cudaError_t e = cudaMemsetAsync(W + it.off_Y, 0, sizeof(double) * Nk * rpk, st);
+  const int64_t Nm = it.N[ds], Mm = it.N[d] / Nm;
+  const int rp = it.rpad[ds];
+  const int64_t sms = device_sm_count();
+  {  // Z_ds = dX Rt_{ds+1}^T; v chunks sized so that about 32k warp jobs cover the entries
+    double* Z = W + it.off_Z[ds];
+    e = cudaMemsetAsync(Z, 0, sizeof(double) * Nm * rp, st);
     if (e != cudaSuccess) return e;
-    // v chunks sized so that about 32k warp jobs cover the entries
-    const int64_t vc = std::max<int64_t>(16, (Nk * Mk) / (32LL * 32768));
-    const int64_t nrb = (Nk + 31) / 32, nvg = ((Mk + vc - 1) / vc + 3) / 4;
-    const int g = (int)std::max<int64_t>(1, std::min<int64_t>(nrb * nvg, 16LL * device_sm_count()));
-    const double* Rt = k == d ? nullptr : W + it.off_Rall[k + 1];
+    const int64_t vc = std::max<int64_t>(16, (Nm * Mm) / (32LL * 32768));
+    const int64_t nrb = (Nm + 31) / 32, nvg = ((Mm + vc - 1) / vc + 3) / 4;
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>(nrb * nvg, 16 * sms));
+    const double* Rt = W + it.off_Rt[ds + 1];
     count_launch();
-    if (rpk <= 8)
-      ygram_kernel<8><<<g, 128, 4 * 8 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nk, Mk, Rt, rpk, W + it.off_Y, vc);
-    else if (rpk <= 16)
-      ygram_kernel<16><<<g, 128, 4 * 16 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nk, Mk, Rt, rpk, W + it.off_Y, vc);
-    else if (rpk <= 32)
-      ygram_kernel<32><<<g, 128, 4 * 32 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nk, Mk, Rt, rpk, W + it.off_Y, vc);
+    if (rp <= 8)
+      ygram_kernel<8><<<g, 128, 4 * 8 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+    else if (rp <= 16)
+      ygram_kernel<16><<<g, 128, 4 * 16 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+    else if (rp <= 32)
+      ygram_kernel<32><<<g, 128, 4 * 32 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
     else
-      ygram_kernel<64><<<g, 128, 4 * 64 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nk, Mk, Rt, rpk, W + it.off_Y, vc);
-    e = cudaGetLastError();
+      ygram_kernel<64><<<g, 128, 4 * 64 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+  }
+  {  // W_ds = L_ds^T dX; row chunks likewise
+    double* Wd = W + it.off_Wd[ds];
+    e = cudaMemsetAsync(Wd, 0, sizeof(double) * Mm * rp, st);
     if (e != cudaSuccess) return e;
-    const int64_t nout = (int64_t)it.rpad[k - 1] * it.n[k - 1] * rpk;
+    const int V = rp <= 8 ? 4 : rp <= 16 ? 2 : 1;
+    const int64_t nvg = (Mm + V - 1) / V;
+    const int64_t want = std::max<int64_t>(1, 64 * sms / nvg);
+    const int64_t uc = std::max<int64_t>(256, (Nm + want - 1) / want);
+    const int64_t jobs = nvg * ((Nm + uc - 1) / uc);
+    const int g = (int)std::max<int64_t>(1, std::min<int64_t>((jobs + 3) / 4, 16 * sms));
+    const double* L = W + it.off_L[ds];
+    count_launch();
+    if (rp <= 8) wgram_kernel<8, 4><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+    else if (rp <= 16) wgram_kernel<16, 2><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+    else if (rp <= 32) wgram_kernel<32, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+    else wgram_kernel<64, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+  }
+  for (int k = ds; k >= 1; --k) {
+    const int64_t Np = it.N[k - 1], nk = it.n[k - 1];
+    const int rpa = it.rpad[k - 1], rpc = it.rpad[k];
+    const int64_t nout = (int64_t)rpa * nk * rpc;
     e = cudaMemsetAsync(dcores + it.core_off[k], 0, sizeof(double) * nout, st);
     if (e != cudaSuccess) return e;
-    const int64_t Np = it.N[k - 1];
     const int64_t uc = std::max<int64_t>(256, (nout * Np) / 32768);
     count_launch();
     dcore_kernel<<<grid_for(nout * ((Np + uc - 1) / uc) * 32), kThreads, 0, st>>>(
-        k == 1 ? nullptr : W + it.off_Lall[k - 1], Np, it.rpad[k - 1], W + it.off_Y, it.n[k - 1], rpk,
-        dcores + it.core_off[k], uc);
+        k == 1 ? nullptr : W + it.off_L[k - 1], Np, rpa, W + it.off_Z[k], nk, rpc, dcores + it.core_off[k], uc);
+    if (k > 1) {
+      count_launch();
+      zdown_kernel<<<grid_for(Np * rpa * 32), kThreads, 0, st>>>(W + it.off_Z[k], Np, nk, rpc, cores + it.core_off[k],
+                                                                rpa, W + it.off_Z[k - 1]);
+    }
+  }
+  for (int k = ds + 1; k <= d; ++k) {
+    const int64_t nk = it.n[k - 1], Mk = it.N[d] / it.N[k];
+    const int rpa = it.rpad[k - 1], rpc = it.rpad[k];
+    count_launch();
+    dcore_right_kernel<<<grid_for((int64_t)rpa * nk * rpc * 32), kThreads, 0, st>>>(
+        W + it.off_Wd[k - 1], rpa, nk, Mk, k == d ? nullptr : W + it.off_Rt[k + 1], rpc, dcores + it.core_off[k]);
+    if (k < d) {
+      count_launch();
+      wup_kernel<<<grid_for(Mk * rpc * 32), kThreads, 0, st>>>(W + it.off_Wd[k - 1], rpa, nk, Mk,
+                                                              cores + it.core_off[k], rpc, W + it.off_Wd[k]);
+    }
   }
   return cudaGetLastError();
 }
