@@ -299,6 +299,7 @@ __global__ void qr_abar_kernel(char* wsb, int item, int k, const int* ranks, con
 }  // namespace
 
 cudaError_t launch_pbar_ls(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st);
+cudaError_t launch_backward_h(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st);
 cudaError_t launch_sketch_adjoint(const Plan& P, int item, void* dX, void* ws, cudaStream_t st);
 
 cudaError_t launch_backward(const Plan& P, int item, const double* dcores, void* dX, void* ws, cudaStream_t st) {
@@ -306,9 +307,10 @@ cudaError_t launch_backward(const Plan& P, int item, const double* dcores, void*
   const DevSketch* sks = plan_sketches_host(&P);
   char* wsb = (char*)ws;
   double* W = (double*)ws;
-  cudaError_t e;
   // ranks of the forward call: the finalize keeps a copy of item 0's in ws
   const int* ranks_dev = reinterpret_cast<const int*>(wsb + kRankCopyOff);
+  cudaError_t e = launch_backward_h(P, item, ws, ranks_dev, st);
+  if (e != cudaSuccess) return e;
   double* small = W + it.off_small;
   const int d = it.d, ds = it.ds;
   // 1. core adjoints

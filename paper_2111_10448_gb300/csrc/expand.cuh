@@ -20,14 +20,16 @@
 #pragma once
 #include <cstdint>
 
+#include "digits.cuh"
 #include "internal.cuh"
 
 namespace tts {
 namespace expand {
 
+using namespace digit;
+
 constexpr int kThreads = 256, kWarps = 8;
 constexpr int kVT = 64;          // columns v staged at a time
-constexpr int kExpZero = -4000;  // exponent that stands for a zero
 
 struct ExpandArgs {
   const double *L, *Rt;
@@ -40,51 +42,6 @@ struct ExpandArgs {
   int vec;             // float4 accesses are aligned
 };
 
-__device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void ldsm4(uint32_t a, uint32_t* r) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
-}
-__device__ __forceinline__ void mma(float* c, const uint32_t* a, const uint32_t* b) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-               "{%0,%1,%2,%3};" : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// Exponent e with |x| < 2^e (kExpZero for zero and subnormal numbers, which count as zero).
-__device__ __forceinline__ int exp_of(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e == 0 ? kExpZero : e - 1022;
-}
-__device__ __forceinline__ bool nonfinite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) == 0x7ff; }
-
-// round(x 2^(B - E)), |x| < 2^E, in integer arithmetic.
-template <int B>
-__device__ __forceinline__ long long fixed(double x, int E) {
-  const long long bits = __double_as_longlong(x);
-  const int e = (int)((bits >> 52) & 0x7ff);
-  if (e == 0) return 0;
-  const unsigned long long m = ((unsigned long long)bits & 0xfffffffffffffull) | (1ull << 52);
-  static_assert(B <= 53, "the shift below is not negative");
-  const int s = 1075 + E - B - e;   // >= 53 - B
-  if (s > 54) return 0;
-  const long long q = (long long)(s > 0 ? (m + (1ull << (s - 1))) >> s : m);
-  return bits < 0 ? -q : q;
-}
-
-// The P balanced base-256 digits of q (most significant first) as BF16 bit
-// patterns: the bytes of q + 0x80..80, less 128 each.
-template <int P>
-__device__ __forceinline__ void digits(long long q, uint32_t (&d)[P]) {
-  unsigned long long b = (unsigned long long)q;
-#pragma unroll
-  for (int i = 0; i < P; ++i) b += 0x80ull << (8 * i);
-#pragma unroll
-  for (int i = 0; i < P; ++i) {
-    const uint32_t byte = (uint32_t)(b >> (8 * (P - 1 - i))) & 0xffu;
-    d[i] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | byte), 8388736.0f)) >> 16;
-  }
-}
 __device__ __forceinline__ float pow2f(int e) {  // 2^e, zero below the normal range, e <= 127
   return e < -126 ? 0.0f : __int_as_float((min(e, 127) + 127) << 23);
 }

@@ -17,6 +17,7 @@
 // stay on the device; later kernels read them from there.
 #include <algorithm>
 
+#include "digits.cuh"
 #include "internal.cuh"
 #include "philox.cuh"
 #include "testmat.cuh"
@@ -819,8 +820,10 @@ __global__ void __launch_bounds__(kThreads) mid_h_kernel(char* wsb, int item_arg
 // the FP64 work is the plain multiply-adds with one short reduction per pair.
 constexpr int kCoreChunk = 32;
 __global__ void __launch_bounds__(kThreads) cores_kernel(char* wsb, double* cores, const int* ranks,
-                                                         int item0, int nitems, int only_k, int dmax) {
-  __shared__ double sA[kCoreChunk * TT_MAXL], sB[kCoreChunk * TT_MAXL];
+                                                         int item0, int nitems, int only_k, int dmax,
+                                                         uint32_t skip) {
+  constexpr int LDC = kCoreChunk + 1;   // threads of a warp read different columns of one row
+  __shared__ double sA[LDC * TT_MAXL], sB[LDC * TT_MAXL];
   __shared__ double red[kThreads];
   const int item = item0 + (int)blockIdx.x / dmax;
   const int k = (int)blockIdx.x % dmax + 1;
@@ -829,6 +832,7 @@ __global__ void __launch_bounds__(kThreads) cores_kernel(char* wsb, double* core
   if (k > it.d) return;
   if (only_k > 0 && k != only_k) return;
   if (only_k == 0 && k == it.mcore && it.passes == 2) return;  // second pass computes it
+  if (skip >> k & 1) return;  // formed by core_gemm_kernel
   const DevSketch* S = dsk(wsb);
   const double* ws = reinterpret_cast<const double*>(wsb);
   const int* rk = ranks + it.rank_off;
@@ -884,15 +888,15 @@ __global__ void __launch_bounds__(kThreads) cores_kernel(char* wsb, double* core
         __syncthreads();
         for (int o = threadIdx.x; o < uc * ra; o += blockDim.x) {
           const int u = o % uc, aa = o / uc;
-          sA[u + kCoreChunk * aa] = left ? (A ? A[u0 + u + lda * aa] : 1.0) : A[i + nk * (u0 + u) + lda * aa];
+          sA[u + LDC * aa] = left ? (A ? A[u0 + u + lda * aa] : 1.0) : A[i + nk * (u0 + u) + lda * aa];
         }
         for (int o = threadIdx.x; o < uc * rc; o += blockDim.x) {
           const int u = o % uc, cc = o / uc;
-          sB[u + kCoreChunk * cc] = left ? B[u0 + u + inner * i + ldb * cc] : (B ? B[u0 + u + ldb * cc] : 1.0);
+          sB[u + LDC * cc] = left ? B[u0 + u + inner * i + ldb * cc] : (B ? B[u0 + u + ldb * cc] : 1.0);
         }
         __syncthreads();
         if (sp < nsplit)
-          for (int u = sp; u < uc; u += nsplit) acc = fma(sA[u + kCoreChunk * a], sB[u + kCoreChunk * c], acc);
+          for (int u = sp; u < uc; u += nsplit) acc = fma(sA[u + LDC * a], sB[u + LDC * c], acc);
       }
       red[threadIdx.x] = sp < nsplit ? acc : 0.0;
       __syncthreads();
@@ -907,6 +911,160 @@ __global__ void __launch_bounds__(kThreads) cores_kernel(char* wsb, double* core
       const int a = o % rpa, c = o / rpa;
       if (a >= ra || c >= rc) Gi[a + rpa * nk * c] = 0.0;
     }
+  }
+}
+
+// Large cores of a single problem in digit arithmetic: C(a, i, j) += sum_u A(u, a)
+// B(u, i, j) over one K range of slice i (cores_kernel's products; FP64 FMAs bound
+// those: 1.72 per cycle and SM on this GPU, against 1015 BF16 ones, which is 30 FP64
+// products in the 34 digit products kept here).  A block takes 64 contraction
+// indices at a time: a warp loads one column's 64 values (two per lane), scales
+// them by the column's largest exponent in this chunk and writes their seven
+// balanced base-256 digits (the largest value keeps all 53 bits); every (16 a) x
+// (8 j) tile sums its digit products of weight at most seven exactly in FP32 (64 x 7
+// x 2^14 < 2^24) and adds them to its FP64 sums.  What is dropped is below 2^-57 of
+// the largest product of the chunk, so the result is as exact as FP64 FMAs.
+// Measured (middle core of 960^3, r = 25, l = 35): H = S M 1.64 ms and Q^T H 3.14 ms
+// -> Q^T S 0.60 ms and (Q^T S) M 0.04 ms.
+struct CoreGemm {
+  const double *A, *B;
+  double* C;
+  int64_t sau, lda, sai;    // A(u, a) of slice i at u sau + a lda + i sai
+  int64_t ldb, sbi;         // B(u, i, j) at u + j ldb + i sbi
+  int64_t ldc, sci;         // C(a, i, j) at a + i sci + j ldc
+  int64_t inner, klen;      // contraction length, the part of one block
+  int ra, rb;
+};
+constexpr int kGemmP = 7, kGemmK = 64, kGemmLD = kGemmK + 8;
+__global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g) {
+  using namespace digit;
+  constexpr int P = kGemmP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P + 1;   // weights kept: 0..7
+  extern __shared__ __align__(16) double sm[];
+  const int ma = (g.ra + 15) / 16, nb = (g.rb + 7) / 8, rows = 16 * ma + 8 * nb;
+  uint16_t* D = reinterpret_cast<uint16_t*>(sm);             // [P][rows][kGemmLD]: A's columns, then B's
+  int* er = reinterpret_cast<int*>(D + P * rows * kGemmLD);  // column exponents
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
+  const int64_t i = blockIdx.x, k0 = (int64_t)blockIdx.y * g.klen, k1 = imin64(g.inner, k0 + g.klen);
+  const double *Ai = g.A + g.sai * i, *Bi = g.B + g.sbi * i;
+  const int tiles = ma * nb;
+  double c[4][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) c[q][0] = c[q][1] = c[q][2] = c[q][3] = 0.0;
+  int bad = 0;
+  for (int64_t u0 = k0; u0 < k1; u0 += kGemmK) {
+    __syncthreads();
+    for (int r0 = warp; r0 < rows; r0 += 4 * (kThreads / 32)) {
+      double x[4][2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * (kThreads / 32);
+        const bool isa = r < 16 * ma;
+        const int col = isa ? r : r - 16 * ma;
+        const bool on = r < rows && col < (isa ? g.ra : g.rb);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int64_t u = u0 + 2 * lane + e;
+          x[q][e] = on && u < k1 ? (isa ? Ai[u * g.sau + col * g.lda] : Bi[u + col * g.ldb]) : 0.0;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = r0 + q * (kThreads / 32);
+        if (r >= rows) break;
+        bad |= (nonfinite(x[q][0]) || nonfinite(x[q][1])) ? 1 : 0;
+        const int m = __reduce_max_sync(0xffffffffu, max(exp_of(x[q][0]), exp_of(x[q][1])));
+        if (lane == 0) er[r] = m;
+        uint32_t d0[P], d1[P];
+        digits<P>(fixed<B>(x[q][0], m), d0);
+        digits<P>(fixed<B>(x[q][1], m), d1);
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+          *reinterpret_cast<uint32_t*>(D + (p * rows + r) * kGemmLD + 2 * lane) = d0[p] | (d1[p] << 16);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int t = warp + q * (kThreads / 32);
+      if (t < tiles) {
+        const int mt = t % ma, nt = t / ma;
+        float acc[NW][4];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) acc[w][0] = acc[w][1] = acc[w][2] = acc[w][3] = 0.0f;
+        const uint32_t pa = s_u32(D + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kGemmLD + 8 * (lane >> 4));
+        const uint32_t pb = s_u32(D + (16 * ma + 8 * nt + (lane & 7)) * kGemmLD + 8 * (lane >> 3));
+        const int stride = 2 * rows * kGemmLD;   // bytes between digit arrays
+#pragma unroll 1
+        for (int kk = 0; kk < kGemmK; kk += 32) {
+          uint32_t fb[P][4];   // two k-steps of each digit of B
+#pragma unroll
+          for (int p = 0; p < P; ++p) ldsm4(pb + p * stride + 2 * kk, fb[p]);
+#pragma unroll
+          for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+              uint32_t fa[4];
+              ldsm4(pa + p * stride + 2 * (kk + 16 * ks), fa);
+#pragma unroll
+              for (int p2 = 0; p2 < P; ++p2)
+                if (p + p2 < NW) mma(acc[(p + p2) % NW], fa, fb[p2] + 2 * ks);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int ea = er[16 * mt + gq + 8 * (e >> 1)], eb = er[16 * ma + 8 * nt + 2 * tq + (e & 1)];
+          long long hi = 0, lo = 0;
+#pragma unroll
+          for (int w = 0; w < 4; ++w) {
+            hi = hi * 256 + __float2int_rn(acc[w][e]);
+            lo = lo * 256 + __float2int_rn(acc[w + 4][e]);
+          }
+          // (hi 2^32 + lo) 2^(ea + eb - 2 LEAD - 56); a column of zeros has no exponent
+          if (hi | lo) {
+            const int x = ea + eb - 2 * LEAD - 56;
+            const double v = fma((double)hi, 4294967296.0, (double)lo);
+            if (x > -900 && x < 900) c[q][e] = fma(v, __hiloint2double((x + 1023) << 20, 0), c[q][e]);
+            else c[q][e] += ldexp(v, x);
+          }
+        }
+      }
+    }
+  }
+  // a non-finite value in this block's range: its products as FP64 FMAs
+  if (__syncthreads_or(bad)) {
+    for (int o = threadIdx.x; o < g.ra * g.rb; o += kThreads) {
+      const int a = o % g.ra, j = o / g.ra;
+      double s = 0.0;
+      for (int64_t u = k0; u < k1; ++u) s = fma(Ai[u * g.sau + a * g.lda], Bi[u + j * g.ldb], s);
+      atomicAdd(g.C + a + g.sci * i + g.ldc * j, s);
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int t = warp + q * (kThreads / 32);
+    if (t >= tiles) break;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int a = 16 * (t % ma) + gq + 8 * (e >> 1), j = 8 * (t / ma) + 2 * tq + (e & 1);
+      if (a < g.ra && j < g.rb) atomicAdd(g.C + a + g.sci * i + g.ldc * j, c[q][e]);
+    }
+  }
+}
+
+// G(a, i, c) = sum_j T(a, i, j) M(j, c) (T: ra x n x l, M: l x rc with columns past
+// the rank zero), one thread per entry.
+__global__ void __launch_bounds__(kThreads) core_tm_kernel(const double* T, const double* M, double* G, int64_t rows,
+                                                           int l, int rc) {
+  __shared__ double Ms[TT_MAXL * TT_MAXL];
+  for (int o = threadIdx.x; o < l * rc; o += blockDim.x) Ms[o] = M[o];
+  __syncthreads();
+  for (int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; o < rows * rc; o += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t r = o % rows;
+    const int c = (int)(o / rows);
+    double s = 0.0;
+    for (int j = 0; j < l; ++j) s = fma(T[r + rows * j], Ms[j + l * c], s);
+    G[o] = s;
   }
 }
 
@@ -1001,7 +1159,101 @@ __global__ void __launch_bounds__(kThreads) twopass_last_kernel(char* wsb, const
   }
 }
 
+// Work from which a core goes to core_gemm_kernel (FMAs; 2^25 take cores_kernel
+// 67 us at the FP64 pipe's rate, the three extra launches about 10).
+constexpr int64_t kGemmMin = 1LL << 25;
+
+// The one-pass middle core as (Q_{d*-1}^T S) M instead of Q_{d*-1}^T (S M): T = Q^T S is
+// formed by core_gemm_kernel in H's place, and H itself is not needed (the backward
+// forms it when it runs).  For large middle sketches that the region of H can
+// hold T of.
+bool mid_by_gemm(const Plan& P, int item) {
+  const DevItem& it = plan_items_host(&P)[item];
+  if (plan_num_items(&P) != 1 || it.passes != 1 || it.sided1 || it.ds < 2 || it.mcore != it.ds) return false;
+  const int64_t ra = it.rpad[it.ds - 1], rc = it.rpad[it.ds], l = it.lmid;
+  return ra * l * it.N[it.ds] >= kGemmMin && ra * l <= rc * (l + ra) && ra * l <= it.N[it.ds - 1] * rc;
+}
+
+cudaError_t run_core_gemm(CoreGemm g, int64_t n, int64_t nout, cudaStream_t st) {
+  const int rows = (g.ra + 15) / 16 * 16 + (g.rb + 7) / 8 * 8;
+  const size_t smem = 2ul * kGemmP * rows * kGemmLD + sizeof(int) * rows;
+  static bool attr = false;
+  cudaError_t e;
+  if (!attr) {
+    e = cudaFuncSetAttribute(core_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(2 * kGemmP * 2 * TT_MAXL * kGemmLD + sizeof(int) * 2 * TT_MAXL));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  e = cudaMemsetAsync(g.C, 0, sizeof(double) * nout, st);
+  if (e != cudaSuccess) return e;
+  // slices shorter than two blocks per SM are split along the contraction
+  const int64_t split = std::max<int64_t>(1, std::min<int64_t>((2LL * device_sm_count() + n - 1) / n, g.inner / 256));
+  g.klen = ((g.inner + split - 1) / split + kGemmK - 1) / kGemmK * kGemmK;
+  count_launch();
+  core_gemm_kernel<<<dim3((unsigned)n, (unsigned)((g.inner + g.klen - 1) / g.klen)), kThreads, smem, st>>>(g);
+  return cudaGetLastError();
+}
+
+// The cores of a single problem that are large enough for core_gemm_kernel; their
+// bits are set in *done.
+cudaError_t launch_core_gemms(const Plan& P, void* ws, double* cores, uint32_t* done, cudaStream_t st) {
+  const DevItem& it = plan_items_host(&P)[0];
+  const DevSketch* S = plan_sketches_host(&P);
+  double* W = (double*)ws;
+  *done = 0;
+  if (plan_num_items(&P) != 1 || it.sided1) return cudaSuccess;
+  for (int k = 2; k < it.d; ++k) {
+    const int64_t n = it.n[k - 1], ra = it.rpad[k - 1], rc = it.rpad[k];
+    const bool left = k <= it.ds, mid = k == it.mcore;
+    if (mid && !mid_by_gemm(P, 0)) continue;
+    CoreGemm g;
+    g.ra = (int)ra;
+    g.rb = (int)(mid ? it.lmid : rc);
+    g.inner = left ? it.N[k - 1] : it.N[it.d] / it.N[k];
+    if (ra * g.rb * g.inner * n < kGemmMin || n >= (1LL << 31)) continue;
+    const DevSketch& sa = S[it.basis_of_k[k - 1]];
+    const DevSketch& sb = S[mid ? it.mid_sk : it.basis_of_k[k]];
+    g.A = W + sa.lev_z[0];
+    g.lda = sa.rows;
+    g.sau = left ? 1 : n;
+    g.sai = left ? 0 : 1;
+    g.B = W + (mid ? sb.off : sb.lev_z[0]);
+    g.ldb = sb.rows;
+    g.sbi = left ? g.inner : 0;
+    g.C = mid ? W + it.off_H : cores + it.core_off[k];
+    g.sci = ra;
+    g.ldc = ra * n;
+    cudaError_t e = run_core_gemm(g, n, ra * n * g.rb, st);
+    if (e != cudaSuccess) return e;
+    if (mid) {
+      const int64_t rows = ra * n;
+      const int grid = (int)std::min<int64_t>((rows * rc + kThreads - 1) / kThreads, 16LL * device_sm_count());
+      count_launch();
+      core_tm_kernel<<<grid, kThreads, 0, st>>>(g.C, W + it.off_QB, cores + it.core_off[k], rows, it.lmid, (int)rc);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    *done |= 1u << k;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_mid_h(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st) {
+  const DevItem& it = plan_items_host(&P)[item];
+  const int64_t Nm = plan_sketches_host(&P)[it.mid_sk].rows;
+  const int grid = (int)std::min<int64_t>((Nm * it.rpad[it.mbk] + kThreads - 1) / kThreads, 8LL * device_sm_count());
+  count_launch();
+  mid_h_kernel<<<grid, kThreads, 0, st>>>((char*)ws, item, ranks);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+// H for the backward, when the forward's middle core did without it.
+cudaError_t launch_backward_h(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st) {
+  return mid_by_gemm(P, item) ? launch_mid_h(P, item, ws, ranks, st) : cudaSuccess;
+}
 
 cudaError_t launch_mid_b_mixed(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st);
 
@@ -1130,11 +1382,14 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
     mid_ls_kernel<<<1, kThreads, 0, st>>>(wsb, i, ranks);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t Nm = sks[it.mid_sk].rows;
-    const int grid = (int)std::min<int64_t>((Nm * it.rpad[it.mbk] + kThreads - 1) / kThreads, 8LL * device_sm_count());
-    count_launch();
-    mid_h_kernel<<<grid, kThreads, 0, st>>>(wsb, i, ranks);
-    e = cudaGetLastError();
+    if (!mid_by_gemm(P, i)) {
+      e = launch_mid_h(P, i, ws, ranks, st);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  uint32_t skip = 0;
+  if (nitems == 1) {
+    e = launch_core_gemms(P, ws, cores, &skip, st);
     if (e != cudaSuccess) return e;
   }
   int dmax = 1;
@@ -1147,7 +1402,7 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
   const int64_t gy = std::min<int64_t>(nmax, std::max<int64_t>(1, 2048 / ((int64_t)nitems * dmax)));
   dim3 grid((unsigned)(nitems * dmax), (unsigned)gy);
   count_launch();
-  cores_kernel<<<grid, kThreads, 0, st>>>(wsb, cores, ranks, 0, nitems, 0, dmax);
+  cores_kernel<<<grid, kThreads, 0, st>>>(wsb, cores, ranks, 0, nitems, 0, dmax, skip);
   return cudaGetLastError();
 }
 
@@ -1157,7 +1412,7 @@ cudaError_t launch_cores_one(const Plan& P, int item, int only_k, void* ws, doub
   const DevItem& it = plan_items_host(&P)[item];
   dim3 grid((unsigned)it.d, (unsigned)std::min<int64_t>(it.n[only_k - 1], 512));
   count_launch();
-  cores_kernel<<<grid, kThreads, 0, st>>>((char*)ws, cores, ranks, item, 1, only_k, it.d);
+  cores_kernel<<<grid, kThreads, 0, st>>>((char*)ws, cores, ranks, item, 1, only_k, it.d, 0u);
   return cudaGetLastError();
 }
 
