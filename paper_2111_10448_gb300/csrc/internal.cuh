@@ -15,6 +15,8 @@
 // for k = d-1 the row sketch has whi = 0: these two collect every plane.)
 #pragma once
 #include <cstdint>
+#include <vector>
+
 #include <cuda_runtime.h>
 #include "../../include/ttsketch.h"
 #include <nvtx3/nvToolsExt.h>
@@ -72,6 +74,8 @@ struct DevSketch {
   int64_t off_piv;     // pivots (width ints, stored as int in a double slot area)
   int64_t gen_tab;     // generic tile kernel: byte offset (in the item's table area) of
                        // this sketch's staged test-matrix rows, -1: regenerated per tile
+  int64_t st_tab;      // strip kernel: byte offset (from the workspace base) of its staged rows
+                       // in the backward's scratch, -1: drawn per tile
   int64_t sp_tab;      // small-plane kernel: byte offset of this sketch's staged
                        // test-matrix rows (BF16), -1 when it is generated per plane
   // ---- Khatri-Rao test matrix (TT_FLAG_KR; kr_nm = 0: dense Gaussian).  The
@@ -219,6 +223,28 @@ cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint
                               int nr, int lpad, int64_t nkeys, char* tab, int prec, cudaStream_t st);
 cudaError_t launch_sketch_sp(const Plan& P, int item, const void* X, int64_t first, int64_t count, void* ws,
                              cudaStream_t st);
+// Column octets and bytes of a staged test-matrix row of the strip kernel, for sketches
+// of width at most l.  16-bit rows are an odd number of 16-byte chunks, so that the
+// eight row addresses of an ldmatrix fall on distinct banks; TF32 rows are 8 or 24
+// words past a multiple of 32, so that the four k rows of a fragment load do.
+__host__ __device__ constexpr int strip_nt(int l) { return l <= 16 ? 2 : l <= 48 ? (l + 7) / 8 : 8; }
+__host__ __device__ constexpr int strip_row_bytes(bool tf32, int nt) {
+  return tf32 ? (nt * 8 + ((nt & 1) ? 0 : 8)) * 4 : (nt | 1) * 16;
+}
+// Batched strip launch: every tensor's arguments and first unit, in the visiting
+// order of the plan (uploaded with the plan tables).
+struct StripBatchPlan {
+  std::vector<unsigned char> args;
+  std::vector<uint32_t> prefix;
+  int nt = 2;
+  size_t smem = 0;
+};
+bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatchPlan* out);
+cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, int64_t off_prefix,
+                                        const void* const* X, void* ws, cudaStream_t st);
+bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args, int64_t* off_prefix);
+// The staged rows (st_tab) of every item of a batched plan, lpad elements a row.
+cudaError_t launch_rows_table_batched(char* wsb, int nitems, int lpad, cudaStream_t st);
 bool use_strip_kernel(const Plan& P, int item, int64_t count);
 cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t first, int64_t count, void* ws,
                                 cudaStream_t st);

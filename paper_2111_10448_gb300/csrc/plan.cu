@@ -41,6 +41,9 @@ struct Plan {
   const void* stream_ws = nullptr;   // workspace of the streaming decomposition begun last
   const void* forward_ws = nullptr;  // workspace of the last completed forward call
   BatchCfg bcfg{64, 4, 4};  // batched sketch launch shape (tt_plan_autotune)
+  StripBatchPlan strip;              // batched strip launch (strip_ok)
+  bool strip_ok = false;
+  int64_t off_strip_args = 0, off_strip_prefix = 0;  // byte offsets of its tables in the workspace
 };
 
 static constexpr int64_t kTableOff = 256;  // bytes
@@ -433,6 +436,7 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   for (int k = 1; k <= ds; ++k) it.off_L[k] = ws.take(it.N[k] * it.rpad[k]);
   for (int k = ds + 1; k <= d; ++k) it.off_Rt[k] = ws.take((int64_t)it.rpad[k - 1] * (it.N[d] / it.N[k - 1]));
   // backward scratch
+  it.off_bar = ws.top;
   for (int si = it.sk0; si < it.sk0 + it.nsk; ++si) {
     const DevSketch& s = P.sketches[si];
     it.off_sbar[si - it.sk0] = ws.take(s.rows * s.width);
@@ -445,6 +449,40 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   if (q.passes == 1) {
     it.off_hbar = ws.take(it.N[ds] * it.rpad[ds]);
     it.off_bbar = ws.take((int64_t)it.rpad[ds] * it.lmid);
+  }
+  // Staged test-matrix rows of the strip kernel: the rows of each sketch that are
+  // staged more than once (a column-side row, key w / wdiv and i_d, by wdiv planes
+  // times the strips of i_1; a row-side row, key w % wdiv and i_1, by W / wdiv planes
+  // times the tiles of i_d), in the kernel's row format, for the whole last mode or
+  // n_1.  They live for one accumulate, in the backward's scratch (free until the
+  // backward runs), smallest tables first as far as that reaches; the other rows
+  // are drawn per tile.  Reading a staged row costs less than drawing it even when
+  // it comes from HBM (an 80-byte row 3.5 cycles of an SM's share of the bandwidth,
+  // its seven column quads 13 cycles at 0.52 quads a cycle).
+  {
+    const bool ok = (op16 || q.prec == TT_PREC_TF32) && q.x_dtype == TT_F32 && it.tctab_doubles == 0 &&
+                    (single || it.sptab_doubles > 0);
+    const int64_t tilesA = (q.n[0] + 127) / 128, tilesB = (q.n[d - 1] + 63) / 64;
+    int lmax = 1;
+    for (int si = it.sk0; si < it.sk0 + it.nsk; ++si) lmax = std::max(lmax, P.sketches[si].width);
+    // (a batched launch uses the row format of its widest tensor, at most 32 columns)
+    const int64_t row = strip_row_bytes(q.prec == TT_PREC_TF32, strip_nt(single ? lmax : std::max(lmax, 32)));
+    std::vector<std::pair<int64_t, int>> want;
+    for (int si = it.sk0; si < it.sk0 + it.nsk; ++si) {
+      DevSketch& s = P.sketches[si];
+      s.st_tab = -1;
+      // a mode-by-mode Khatri-Rao sketch reads one factor row per tile row: nothing to stage
+      if (!ok || s.kr_mbm) continue;
+      if (s.type == SK_COL && s.wdiv * tilesA >= 2) want.emplace_back((it.W / s.wdiv) * q.n[d - 1] * row, si);
+      if (s.type == SK_ROW && (it.W / s.wdiv) * tilesB >= 2) want.emplace_back(s.wdiv * q.n[0] * row, si);
+    }
+    std::sort(want.begin(), want.end());
+    int64_t at = (it.off_bar * 8 + 255) / 256 * 256;
+    for (const auto& w : want) {
+      if (at + w.first > ws.top * 8) break;
+      P.sketches[w.second].st_tab = at;
+      at += (w.first + 255) / 256 * 256;
+    }
   }
   if (single) it.off_small = ws.take(4LL * TT_MAXL * TT_MAXL);
   it.diff = (q.flags & TT_FLAG_DIFF) ? 1 : 0;
@@ -493,6 +531,13 @@ static void build_blob(Plan& P) {
   off += align_up((int64_t)(sizeof(int64_t) * (order.size() + 1)), 64);
   t.off_bcounter = off;
   off += 64;
+  P.strip_ok = P.items.size() > 1 && strip_plan_batched(P, order, &P.strip);
+  if (P.strip_ok) {
+    P.off_strip_args = off;
+    off += align_up((int64_t)P.strip.args.size(), 64);
+    P.off_strip_prefix = off;
+    off += align_up((int64_t)(sizeof(uint32_t) * P.strip.prefix.size()), 64);
+  }
   P.blob.assign((size_t)(off - kTableOff), 0);
   auto put = [&](int64_t at, const void* src, size_t n) {
     if (n) std::memcpy(P.blob.data() + (at - kTableOff), src, n);
@@ -502,6 +547,10 @@ static void build_blob(Plan& P) {
   put(t.off_sketches, P.sketches.data(), sizeof(DevSketch) * P.sketches.size());
   for (int L = 0; L < kMaxLev; ++L) put(t.off_tasks[L], P.tasks[L].data(), sizeof(Task) * P.tasks[L].size());
   put(t.off_border, order.data(), sizeof(int) * order.size());
+  if (P.strip_ok) {
+    put(P.off_strip_args, P.strip.args.data(), P.strip.args.size());
+    put(P.off_strip_prefix, P.strip.prefix.data(), sizeof(uint32_t) * P.strip.prefix.size());
+  }
 }
 
 static tt_status build_all(Plan& P, const tt_problem* probs, int count, int64_t base_doubles) {
@@ -626,6 +675,12 @@ int device_sm_count() {
 // The staged tables of the slab kernel that do not depend on the slab are
 // generated by the first accumulate of a decomposition and reused by the
 // others (begin / tt_pstt2 clear the flag).
+bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args, int64_t* off_prefix) {
+  *bp = &P.strip;
+  *off_args = P.off_strip_args;
+  *off_prefix = P.off_strip_prefix;
+  return P.strip_ok;
+}
 bool& plan_stream_tables(Plan& P) { return P.stream_tables; }
 int& plan_pending_folds(Plan& P) { return P.pending_folds; }
 

@@ -685,6 +685,27 @@ __global__ void sp_table_batched_kernel(char* wsb) {
   }
 }
 
+// Staged rows of the batched strip kernel: blockIdx.y = item, the sketches that
+// have a table (st_tab) one after another, lpad elements a row.
+__global__ void rows_table_batched_kernel(char* wsb, int lpad) {
+  const DevTables& T = *reinterpret_cast<const DevTables*>(wsb + kTableOffB);
+  const DevItem& it = reinterpret_cast<const DevItem*>(wsb + T.off_items)[blockIdx.y];
+  const DevSketch* sks = reinterpret_cast<const DevSketch*>(wsb + T.off_sketches);
+  for (int si = 0; si < it.nsk; ++si) {
+    const DevSketch& d = sks[it.sk0 + si];
+    if (d.st_tab < 0) continue;
+    SpSk k;
+    k.hstride = d.hstride;
+    k.col = d.type == SK_COL ? 1 : 0;
+    k.sid = d.stream_id;
+    k.kr = -1;  // batched plans draw dense test matrices
+    const int nr = k.col ? (int)it.n[it.d - 1] : (int)it.n[0];
+    sp_table_fill(wsb, k, it.seed, 0, it.n[0], nr, d.width, lpad, k.col ? it.W / d.wdiv : d.wdiv,
+                  wsb + d.st_tab, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+                  (int64_t)gridDim.x * blockDim.x, it.prec);
+  }
+}
+
 // Unit prefix of the batched form (largest items first); resets the work
 // counter and the status word.
 __global__ void __launch_bounds__(1024) sp_batch_prep_kernel(char* wsb, int t3max) {
@@ -748,6 +769,12 @@ cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 16LL * device_sm_count()));
   count_launch();
   sp::sp_table_kernel<<<blocks, 256, 0, st>>>(wsb, k, seed, first, n1, nr, d.width, lpad, nkeys, tab, prec);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rows_table_batched(char* wsb, int nitems, int lpad, cudaStream_t st) {
+  count_launch();
+  sp::rows_table_batched_kernel<<<dim3(16, (unsigned)nitems), 256, 0, st>>>(wsb, lpad);
   return cudaGetLastError();
 }
 

@@ -47,21 +47,28 @@ namespace {
 
 constexpr int kSmemTwo = 111 * 1024;   // dynamic shared memory of a CTA, two per SM
 constexpr int kSmemOne = 224 * 1024;   // one per SM
+constexpr int64_t kBatchUnit = 1 << 17;  // entries of a batched unit, about
 
-uint32_t recip20(int d) { return ((1u << 20) + (uint32_t)d - 1u) / (uint32_t)d; }
-
-int nt_instance(int nt) { return nt <= 2 ? 2 : nt <= 6 ? nt : 8; }
+int strip_octets(const Plan& P, int item) {
+  const DevItem& it = plan_items_host(&P)[item];
+  const DevSketch* sks = plan_sketches_host(&P);
+  int lmax = 1;
+  for (int s = 0; s < it.nsk; ++s) lmax = std::max(lmax, sks[it.sk0 + s].width);
+  return strip_nt(lmax);
+}
 
 // Fills the launch arguments when the kernel serves this call.
+// nt_batch: column octets of a batched launch (0: a launch of its own), whose
+// units are sized by entries, since other tensors fill the SMs beside it.
 bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt_out, int* nt_out, size_t* smem,
-                int64_t* units) {
+                int64_t* units, int nt_batch = 0) {
   const DevItem& it = plan_items_host(&P)[item];
   if (it.x_f64 || (it.prec != TT_PREC_BF16 && it.prec != TT_PREC_TF32 && it.prec != TT_PREC_FP16)) return false;
   const int fmt = it.prec == TT_PREC_TF32 ? kFmtTF32 : it.prec == TT_PREC_FP16 ? kFmtFP16 : kFmtBF16;
   const DevSketch* sks = plan_sketches_host(&P);
   StripArgs g;
   memset(&g, 0, sizeof(g));
-  int lmax = 1;
+  bool kr = false;
   for (int s = 0; s < it.nsk; ++s) {
     const DevSketch& d = sks[it.sk0 + s];
     StSk k;
@@ -69,15 +76,16 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
     k.rows = d.rows;
     k.off = d.off;
     k.hstride = d.hstride;
-    k.tab = d.gen_tab >= 0 && it.gentab_doubles > 0 ? it.off_gentab * 8 + d.gen_tab : -1;
+    k.tab = d.st_tab;
     if (d.wdiv >= (1LL << 31)) return false;
     k.wdiv = (uint32_t)d.wdiv;
     k.width = d.width;
-    k.lpad = (d.width + 15) / 16 * 16;
+    k.nq = (d.width + 3) / 4;
+    k.inv_nq = 1.0f / (float)k.nq;
     k.sid = d.stream_id;
     k.kr = d.kr_nm ? it.sk0 + s : -1;
     k.mbm = d.kr_nm && d.kr_mbm ? 1 : 0;
-    lmax = std::max(lmax, d.width);
+    kr = kr || d.kr_nm;
     if (d.type == SK_COL) {
       if (g.ncol == kMaxCol) return false;
       g.col[g.ncol++] = k;
@@ -92,7 +100,21 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
   if (it.n[0] >= (1LL << 31) || count < 1 || count >= (1LL << 31) || it.W >= (1LL << 31) ||
       WR * ((count + tbmax - 1) / tbmax) >= (1LL << 31))
     return false;
-  const int nt = nt_instance((lmax + 7) / 8);
+  const int nt = nt_batch ? nt_batch : strip_octets(P, item);
+  const int64_t nrh = it.d - 1 > it.ds ? it.n[it.d - 2] : 1, sR = WR / nrh, q2 = it.ds >= 2 ? it.n[1] : 1;
+  for (int s = 0; s < g.ncol; ++s) g.tabs |= g.col[s].tab >= 0 ? 1u << s : 0u;
+  for (int r = 0; r < g.nrow; ++r) g.tabs |= g.row[r].tab >= 0 ? 1u << (kMaxCol + r) : 0u;
+  for (int s = 0; s < g.ncol; ++s) {
+    const int64_t w = g.col[s].wdiv;
+    if (w != 1 && w != q2 && w != WL) return false;
+    g.col[s].kind = w == WL ? 2 : w == 1 ? 0 : 1;
+    g.col[s].mulr = WL / w;
+  }
+  for (int r = 0; r < g.nrow; ++r) {
+    const int64_t q = g.row[r].wdiv / WL;
+    if (q != 1 && q != sR && q != WR) return false;
+    g.row[r].kind = q == WR ? 2 : q == 1 ? 0 : 1;
+  }
   g.n1 = it.n[0];
   g.cnt = count;
   g.Nd1 = it.N[it.d - 1];
@@ -100,68 +122,108 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
   g.xscale = fmt == kFmtFP16 ? it.xscale : 1.0f;
   g.WL = (uint32_t)WL;
   g.WR = (uint32_t)WR;
-  g.q2 = it.ds >= 2 ? (uint32_t)it.n[1] : 1u;
+  g.q2 = (uint32_t)q2;
   g.q3 = it.ds >= 3 ? (uint32_t)it.n[2] : 1u;
+  g.nrh = (uint32_t)nrh;
+  g.sR = (uint32_t)sR;
   // strips and tiles of even size, rounded to m-tiles
   g.nA = (int)((g.n1 + kMaxTA - 1) / kMaxTA);
-  g.TA = (int)(((g.n1 + g.nA - 1) / g.nA + 15) / 16 * 16);
-  g.nA = (int)((g.n1 + g.TA - 1) / g.TA);
+  g.n1p = (int)(((g.n1 + g.nA - 1) / g.nA + 15) / 16 * 16);
+  g.nA = (int)((g.n1 + g.n1p - 1) / g.n1p);
   g.nB = (int)((count + tbmax - 1) / tbmax);
-  g.TB = (int)(((count + g.nB - 1) / g.nB + 15) / 16 * 16);
-  g.nB = (int)((count + g.TB - 1) / g.TB);
-  g.ngt = (uint32_t)(WR * g.nB);
-  const int E = esz(fmt), mtB = g.TB / 16, mtA = g.TA / 16;
-  int off = g.TB * (g.TA + 8) * E;
-  g.off_xl = off;
-  off *= 2;
-  g.off_raw = off;
-  off += g.TB * (g.TA + 4) * 4;
-  for (int s = 0; s < g.ncol; ++s) {
-    g.col[s].soff = off;
-    off += g.TB * ldg_bytes(fmt, nt);
+  g.ndp = (int)(((count + g.nB - 1) / g.nB + 15) / 16 * 16);
+  g.nB = (int)((count + g.ndp - 1) / g.ndp);
+  const int E = esz(fmt), ldg = ldg_bytes(fmt, nt);
+  const int ncs = nt_batch || g.ncol > 2 ? 3 : 2;
+  // shared memory before the row sums, and one column tile's row sums
+  auto layout = [&](int PL, int PR, int* per) {
+    g.PL = PL;
+    g.PR = PR;
+    g.TA = PL * g.n1p;
+    g.TB = PR * g.ndp;
+    int off = g.TB * (g.TA + 8) * E;
+    g.off_xl = off;
+    off *= 2;
+    g.off_raw = off;
+    const int run = PL > 1 ? PL * (int)g.n1 : g.n1p;
+    g.rawld = (run + 3) / 4 * 4 + 4;
+    off += PR * (int)std::min<int64_t>(count, g.ndp) * g.rawld * 4;
+    g.off_g = off;
+    for (int s = 0; s < g.ncol; ++s) {
+      g.col[s].per = PL > 1 && g.col[s].wdiv == 1 ? 1 : 0;
+      g.col[s].soff = off;
+      off += (g.col[s].per ? PL : 1) * g.TB * ldg;
+    }
+    for (int r = 0; r < g.nrow; ++r) {
+      g.row[r].per = PR > 1 && g.row[r].wdiv == (uint32_t)it.W ? 1 : 0;
+      g.row[r].soff = off;
+      off += (g.row[r].per ? PR : 1) * g.TA * ldg;
+    }
+    g.off_scale = off;
+    off += 8 * nt * (int)sizeof(float);
+    g.off_acc = (off + 15) / 16 * 16;
+    *per = g.nrow * (g.TB / 16) * nt * 512;
+    return g.off_acc;
+  };
+  // Small planes are grouped into tiles (dense test matrices only: a mode-by-mode
+  // sketch is scaled per plane): the largest tile that leaves two CTAs an SM.
+  const bool regs_two = ncs * nt <= 12;
+  int PL = 1, PR = 1, per = 0;
+  if (!kr && (g.nA == 1 || g.nB == 1)) {
+    int64_t best = 0;
+    const int pl_max = g.nA == 1 ? (int)std::min<int64_t>(kMaxTA / g.n1p, g.q2) : 1;
+    const int pr_max = g.nB == 1 ? (int)std::min<int64_t>(std::max<int64_t>(1, tbmax / g.ndp), g.nrh) : 1;
+    for (int pl = 1; pl <= pl_max; ++pl)
+      for (int pr = 1; pr <= pr_max; ++pr) {
+        if (layout(pl, pr, &per) + per > (regs_two ? kSmemTwo : kSmemOne)) continue;
+        const int64_t area = (int64_t)pl * pr;
+        if (area > best || (area == best && pl * g.n1p >= pr * g.ndp && PL * g.n1p < PR * g.ndp)) {
+          best = area;
+          PL = pl;
+          PR = pr;
+        }
+      }
   }
-  for (int r = 0; r < g.nrow; ++r) {
-    g.row[r].soff = off;
-    off += g.TA * ldg_bytes(fmt, nt);
-  }
-  g.off_scale = off;
-  off += 8 * nt * (int)sizeof(float);
-  g.off_acc = off = (off + 15) / 16 * 16;
+  int off = layout(PL, PR, &per);
+  g.inv_pl = 1.0f / (float)PL;
+  g.npos = (uint32_t)((g.q2 + PL - 1) / PL * g.q3);
+  g.ngt = (uint32_t)(g.sR * ((g.nrh + PR - 1) / PR) * g.nB);
   // the row sums of a set of column tiles take the rest; fewer when the sets
   // alone would leave SMs without a unit
-  const int per = g.nrow * mtB * nt * 512;
+  const int mtA = g.TA / 16, mtB = g.TB / 16;
   const int slots = device_sm_count() * 2;
-  const bool two = (g.ncol <= 2 ? 2 : 3) * nt <= 12 && off + per <= kSmemTwo;
+  const bool two = regs_two && off + per <= kSmemTwo;
   int64_t ng = ((two ? kSmemTwo : kSmemOne) - off) / per;
   if (ng < 1) return false;
   ng = std::min<int64_t>(ng, g.ngt);
-  ng = std::min(ng, std::max<int64_t>(1, (int64_t)g.ngt * g.nA * WL / slots));
+  if (!nt_batch) ng = std::min(ng, std::max<int64_t>(1, (int64_t)g.ngt * g.nA * g.npos / slots));
   g.nGS = (int)((g.ngt + ng - 1) / ng);
   g.NG = (int)((g.ngt + g.nGS - 1) / g.nGS);
   g.nGS = (int)((g.ngt + g.NG - 1) / g.NG);
-  // kL ranges: about four units per CTA slot
+  // position ranges: about four units per CTA slot
   const int64_t base = (int64_t)g.nA * g.nGS;
-  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(WL, (4LL * slots + base - 1) / base));
-  g.CL = (uint32_t)((WL + want - 1) / want);
-  *units = base * ((WL + g.CL - 1) / g.CL);
+  const int64_t goal = nt_batch ? (it.N[it.d] + kBatchUnit - 1) / kBatchUnit : 4LL * slots;
+  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(g.npos, (goal + base - 1) / base));
+  g.CL = (uint32_t)((g.npos + want - 1) / want);
+  *units = base * ((g.npos + g.CL - 1) / g.CL);
   if (*units >= (1LL << 31)) return false;
-  g.inv_qpr = recip20(g.TA / 4);
   // row products (m-tile, sketch) to the least-loaded warp; a warp with an
   // m-tile of the strip starts with its column products
   int load[kWarps], cnt[kWarps];
   for (int w = 0; w < kWarps; ++w) {
     load[w] = w < mtA ? g.ncol * g.TB : 0;
     cnt[w] = 0;
-    memset(g.task[w], 255, kMaxTasks);
+    memset(g.task[w], 255, kWarpTasks);
   }
   for (int mt = 0; mt < mtB; ++mt)
     for (int r = 0; r < g.nrow; ++r) {
       int w = 0;
       for (int v = 1; v < kWarps; ++v)
-        if (load[v] < load[w]) w = v;
+        if (cnt[v] < kWarpTasks && (cnt[w] == kWarpTasks || load[v] < load[w])) w = v;
       g.task[w][cnt[w]++] = (uint8_t)(mt + 8 * r);
       load[w] += g.TA;
     }
+  g.item = item;
   *out = g;
   *fmt_out = fmt;
   *nt_out = nt;
@@ -193,18 +255,18 @@ cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t 
   g.wsb = (char*)ws;
   g.first = first;
   g.vec = it.n[0] % 4 == 0 && ((uintptr_t)X & 15) == 0 ? 1 : 0;
-  g.cpr = g.TA / 4 + (g.vec ? 0 : 1);
-  g.inv_cpr = strip::recip20(g.cpr);
+  g.cpr = g.rawld / 4;
   g.total = g.Nd1 * count;
   for (int s = 0; s < it.nsk; ++s) {
     const DevSketch& d = sks[it.sk0 + s];
-    if (d.gen_tab < 0 || it.gentab_doubles == 0) continue;
-    // stage the sketch's rows for this call: the slab's i_d (column side) or i_1 (row side)
+    if (d.st_tab < 0) continue;
+    // stage the sketch's rows for this call, in the kernel's own row format: the
+    // slab's i_d (column side) or i_1 (row side)
     const bool col = d.type == SK_COL;
+    const int lpad = strip::ldg_bytes(fmt, nt) / strip::esz(fmt);
     const cudaError_t e = launch_rows_table(d, it.sk0 + s, (const char*)ws, it.seed, first, it.n[0],
-                                            col ? (int)count : (int)it.n[0], (d.width + 15) / 16 * 16,
-                                            col ? it.W / d.wdiv : d.wdiv, (char*)ws + it.off_gentab * 8 + d.gen_tab,
-                                            it.prec, st);
+                                            col ? (int)count : (int)it.n[0], lpad, col ? it.W / d.wdiv : d.wdiv,
+                                            (char*)ws + d.st_tab, it.prec, st);
     if (e != cudaSuccess) return e;
   }
   const strip::KernelFn k = fmt == strip::kFmtTF32   ? strip::kernel_tf32(nt, g.ncol)
@@ -219,6 +281,71 @@ cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t 
   }
   count_launch();
   k<<<(unsigned)units, strip::kThreads, smem, st>>>(g);
+  return cudaGetLastError();
+}
+
+bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatchPlan* out) {
+  const int n = plan_num_items(&P);
+  out->args.clear();
+  out->prefix.assign(1, 0u);
+  out->nt = 2;
+  out->smem = 0;
+  if (n < 2 || n > kMaxBatchItems) return false;
+  for (int i = 0; i < n; ++i) {
+    const DevItem& it = plan_items_host(&P)[i];
+    if (it.prec != plan_items_host(&P)[0].prec || it.sptab_doubles == 0) return false;
+    out->nt = std::max(out->nt, strip::strip_octets(P, i));
+  }
+  if (out->nt > 4) return false;
+  out->args.resize((size_t)n * sizeof(strip::StripArgs));
+  int64_t units = 0;
+  for (int pos = 0; pos < n; ++pos) {
+    strip::StripArgs g;
+    int fmt, nt;
+    size_t smem;
+    int64_t u;
+    const DevItem& it = plan_items_host(&P)[order[(size_t)pos]];
+    if (!strip::plan_strip(P, order[(size_t)pos], it.n[it.d - 1], &g, &fmt, &nt, &smem, &u, out->nt)) return false;
+    if (smem > (size_t)strip::kSmemTwo) return false;
+    g.vec = it.n[0] % 4 == 0;
+    g.cpr = g.rawld / 4;
+    g.total = g.Nd1 * g.cnt;
+    std::memcpy(out->args.data() + (size_t)pos * sizeof(g), &g, sizeof(g));
+    out->smem = std::max(out->smem, smem);
+    units += u;
+    if (units >= (1LL << 31)) return false;
+    out->prefix.push_back((uint32_t)units);
+  }
+  return true;
+}
+
+cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, int64_t off_prefix,
+                                        const void* const* X, void* ws, cudaStream_t st) {
+  const int n = plan_num_items(&P);
+  const int prec = plan_items_host(&P)[0].prec;
+  const int fmt = prec == TT_PREC_TF32 ? strip::kFmtTF32 : prec == TT_PREC_FP16 ? strip::kFmtFP16 : strip::kFmtBF16;
+  cudaError_t e = cudaMemsetAsync((char*)ws + kStatusOff, 0, sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  const int lpad = strip::ldg_bytes(fmt, bp.nt) / strip::esz(fmt);
+  e = launch_rows_table_batched((char*)ws, n, lpad, st);
+  if (e != cudaSuccess) return e;
+  strip::StripBatch b;
+  b.wsb = (char*)ws;
+  b.off_args = off_args;
+  b.off_prefix = off_prefix;
+  b.nitems = n;
+  std::memcpy(b.X, X, sizeof(void*) * (size_t)n);
+  const strip::BatchFn k = fmt == strip::kFmtTF32   ? strip::batched_tf32(bp.nt)
+                           : fmt == strip::kFmtFP16 ? strip::batched_fp16(bp.nt)
+                                                    : strip::batched_bf16(bp.nt);
+  static bool attr_set[3][5] = {};
+  if (!attr_set[fmt][bp.nt]) {
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, strip::kSmemTwo);
+    if (e != cudaSuccess) return e;
+    attr_set[fmt][bp.nt] = true;
+  }
+  count_launch();
+  k<<<bp.prefix.back(), strip::kThreads, bp.smem, st>>>(b);
   return cudaGetLastError();
 }
 

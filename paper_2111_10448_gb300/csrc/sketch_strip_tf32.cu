@@ -5,5 +5,6 @@
 namespace tts {
 namespace strip {
 KernelFn kernel_tf32(int nt, int ncol) { return kernel_of<kFmtTF32>(nt, ncol); }
+BatchFn batched_tf32(int nt) { return batched_of<kFmtTF32>(nt); }
 }  // namespace strip
 }  // namespace tts

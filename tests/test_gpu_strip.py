@@ -92,3 +92,46 @@ def test_strip_aligned_equals_unaligned(prec):
     for g in got[1:]:
         for k in g:
             assert np.linalg.norm(g[k] - got[0][k]) <= 1e-6 * np.linalg.norm(got[0][k])
+
+
+GROUPED = [
+    # small planes: tiles of several kL (i_2) and kR (i_{d-1}) values, ragged at both ends
+    ([8, 3, 5, 9], 3, 5, [9]),
+    ([24, 5, 3, 24], 6, 5, [24]),
+    ([24, 7, 2, 5, 3, 23], 10, 10, [23]),         # d = 6, three sketches a side
+    ([9, 7, 5, 8, 6, 9], 4, 5, [4, 5]),           # slabs
+    ([16, 9, 3, 17, 32], 8, 9, [32]),
+    ([31, 4, 3, 30], 5, 6, [30]),                 # unaligned rows
+    ([32, 3, 32], 20, 10, [32]),                  # one kR value
+    ([12, 1, 9, 11], 4, 4, [11]),
+    ([1, 6, 5, 3], 2, 2, [3]),
+    ([20, 18], 6, 6, [18]),
+    ([10, 40, 12, 8], 5, 6, [1, 7]),
+    ([40, 5, 6, 7, 20], 9, 6, [20]),              # grouped along i_{d-1} and i_2, past the small-plane limit
+]
+
+
+@pytest.mark.parametrize("prec", ["tf32", "bf16", "fp16"])
+@pytest.mark.parametrize("dims,r,p,slabs", GROUPED)
+def test_strip_grouped_planes_match_oracle(dims, r, p, slabs, prec):
+    x = np.random.default_rng(6).standard_normal(int(np.prod(dims))).astype(np.float32)
+    s = _scale_of(x) if prec == "fp16" else 0
+    ranks = [1] + [r] * (len(dims) - 1) + [1]
+    t = TTSketch(dims, ranks=ranks, p=p, seed=4, x_dtype=torch.float32, prec=prec, x_scale_log2=s)
+    n = int(np.prod(dims[:-1]))
+    buf = to_dev(x)
+    t.begin()
+    a = 0
+    for c in slabs:
+        t.accumulate(buf[a * n:(a + c) * n], a, c)
+        a += c
+    sk = {k: v * 2.0 ** -s for k, v in sketch_dict(t).items()}
+    t.finalize()
+    o = OP.pstt2(_split(x, prec, s), dims, ranks=ranks, p=p, seed=4, passes=1, test_fmt=prec)
+    for name, ty in (("S", 0), ("R", 1)):
+        for k, S in o["sketch"][name].items():
+            G = sk[(ty, k)]
+            assert G.shape == S.shape
+            fro = np.linalg.norm(G - S) / np.linalg.norm(S)
+            mx = np.max(np.abs(G - S)) / np.max(np.abs(S))
+            assert fro <= 1e-4 and mx <= 2e-3, (name, k, fro, mx)
