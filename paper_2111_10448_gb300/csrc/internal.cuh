@@ -219,17 +219,22 @@ cudaError_t launch_sketch_slab(const Plan& P, int item, const void* X, int64_t f
 // j < lpad, at element (key nr + r) lpad + j of tab (BF16 or FP16, or FP32
 // rounded to TF32, by prec), rows as the sketch's test matrix numbers them for
 // the slab starting at `first` (column side) or for plane key (row side).
+// swizzle: 16-bit rows in the strip kernel's chunk order.
 cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint64_t seed, int64_t first, int64_t n1,
-                              int nr, int lpad, int64_t nkeys, char* tab, int prec, cudaStream_t st);
+                              int nr, int lpad, int64_t nkeys, char* tab, int prec, bool swizzle, cudaStream_t st);
 cudaError_t launch_sketch_sp(const Plan& P, int item, const void* X, int64_t first, int64_t count, void* ws,
                              cudaStream_t st);
 // Column octets and bytes of a staged test-matrix row of the strip kernel, for sketches
-// of width at most l.  16-bit rows are an odd number of 16-byte chunks, so that the
-// eight row addresses of an ldmatrix fall on distinct banks; TF32 rows are 8 or 24
-// words past a multiple of 32, so that the four k rows of a fragment load do.
+// of width at most l.  The eight row addresses of an ldmatrix have to fall on
+// distinct banks: 16-bit rows of an odd number of 16-byte chunks do, in the others
+// chunk c of row r lies at c ^ strip_swizzle(chunks, r).  TF32 rows are 8 or 24 words
+// past a multiple of 32, so that the four k rows of a fragment load do.
 __host__ __device__ constexpr int strip_nt(int l) { return l <= 16 ? 2 : l <= 48 ? (l + 7) / 8 : 8; }
 __host__ __device__ constexpr int strip_row_bytes(bool tf32, int nt) {
-  return tf32 ? (nt * 8 + ((nt & 1) ? 0 : 8)) * 4 : (nt | 1) * 16;
+  return tf32 ? (nt * 8 + ((nt & 1) ? 0 : 8)) * 4 : nt * 16;
+}
+__host__ __device__ constexpr int strip_swizzle(int chunks, int r) {
+  return (chunks & 1) ? 0 : (chunks & 2) ? (r >> 2) & 1 : chunks == 4 ? (r >> 1) & 3 : r & 7;
 }
 // Batched strip launch: every tensor's arguments and first unit, in the visiting
 // order of the plan (uploaded with the plan tables).

@@ -454,11 +454,11 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   // staged more than once (a column-side row, key w / wdiv and i_d, by wdiv planes
   // times the strips of i_1; a row-side row, key w % wdiv and i_1, by W / wdiv planes
   // times the tiles of i_d), in the kernel's row format, for the whole last mode or
-  // n_1.  They live for one accumulate, in the backward's scratch (free until the
-  // backward runs), smallest tables first as far as that reaches; the other rows
-  // are drawn per tile.  Reading a staged row costs less than drawing it even when
-  // it comes from HBM (an 80-byte row 3.5 cycles of an SM's share of the bandwidth,
-  // its seven column quads 13 cycles at 0.52 quads a cycle).
+  // n_1.  They live for one accumulate, in workspace that is free then: the backward's
+  // scratch and the other tile kernels' staging areas, largest table first; rows that
+  // find no room are drawn per tile.  Reading a staged row costs less than drawing it
+  // even when it comes from HBM (a 64-byte row 3 cycles of an SM's share of the
+  // bandwidth, its seven column quads 13 cycles at 0.52 quads a cycle).
   {
     const bool ok = (op16 || q.prec == TT_PREC_TF32) && q.x_dtype == TT_F32 && it.tctab_doubles == 0 &&
                     (single || it.sptab_doubles > 0);
@@ -476,13 +476,19 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
       if (s.type == SK_COL && s.wdiv * tilesA >= 2) want.emplace_back((it.W / s.wdiv) * q.n[d - 1] * row, si);
       if (s.type == SK_ROW && (it.W / s.wdiv) * tilesB >= 2) want.emplace_back(s.wdiv * q.n[0] * row, si);
     }
-    std::sort(want.begin(), want.end());
-    int64_t at = (it.off_bar * 8 + 255) / 256 * 256;
-    for (const auto& w : want) {
-      if (at + w.first > ws.top * 8) break;
-      P.sketches[w.second].st_tab = at;
-      at += (w.first + 255) / 256 * 256;
-    }
+    std::sort(want.begin(), want.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+    // (start, end) of the free regions, bytes
+    int64_t reg[3][2] = {{it.off_bar * 8, ws.top * 8},
+                         {it.off_gentab * 8, (it.off_gentab + it.gentab_doubles) * 8},
+                         {it.off_sptab * 8, (it.off_sptab + it.sptab_doubles) * 8}};
+    for (const auto& w : want)
+      for (auto& r : reg) {
+        const int64_t at = (r[0] + 255) / 256 * 256;
+        if (at + w.first > r[1]) continue;
+        P.sketches[w.second].st_tab = at;
+        r[0] = at + w.first;
+        break;
+      }
   }
   if (single) it.off_small = ws.take(4LL * TT_MAXL * TT_MAXL);
   it.diff = (q.flags & TT_FLAG_DIFF) ? 1 : 0;

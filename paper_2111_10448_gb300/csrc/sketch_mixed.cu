@@ -1367,7 +1367,7 @@ cudaError_t launch_sketch_mma(const Plan& P, int item, const void* X, int64_t fi
       cudaError_t e = launch_rows_table(d, it.sk0 + s, (const char*)ws, it.seed, first, a.n1,
                                         col ? (int)count : (int)a.n1, lpad,
                                         col ? it.W / d.wdiv : d.wdiv, (char*)ws + a.sk[s].tab,
-                                        it.prec, st);
+                                        it.prec, false, st);
       if (e != cudaSuccess) return e;
     }
   }

@@ -157,7 +157,8 @@ __device__ __forceinline__ uint32_t op16x2(bool f16, float lo, float hi) {
 // FP32 words), zero for j >= l.  Threads tid0, tid0 + nthr, ... of the caller
 // take the entries.
 __device__ void sp_table_fill(const char* wsb, const SpSk& s, uint64_t seed, int64_t first, int64_t n1, int nr,
-                              int ell, int lpad, int64_t nkeys, char* tab, int64_t tid0, int64_t nthr, int prec) {
+                              int ell, int lpad, int64_t nkeys, char* tab, int64_t tid0, int64_t nthr, int prec,
+                              bool swizzle = false) {
   const bool tf = prec == TT_PREC_TF32, f16 = prec == TT_PREC_FP16;
   const DevSketch* kr = kr_of(wsb, s.kr);
   const int qpr = lpad / 4;
@@ -178,15 +179,16 @@ __device__ void sp_table_fill(const char* wsb, const SpSk& s, uint64_t seed, int
     } else {
       const uint32_t lo = op16x2(f16, 4 * q < ell ? z.x : 0.f, 4 * q + 1 < ell ? z.y : 0.f);
       const uint32_t hi = op16x2(f16, 4 * q + 2 < ell ? z.z : 0.f, 4 * q + 3 < ell ? z.w : 0.f);
-      *reinterpret_cast<uint2*>(tab + el * 2) = make_uint2(lo, hi);
+      const int sw = swizzle ? (strip_swizzle(lpad / 8, r) ^ (q >> 1)) - (q >> 1) : 0;   // 16-byte chunks moved by
+      *reinterpret_cast<uint2*>(tab + el * 2 + 16 * sw) = make_uint2(lo, hi);
     }
   }
 }
 
 __global__ void sp_table_kernel(const char* wsb, SpSk s, uint64_t seed, int64_t first, int64_t n1, int nr, int ell,
-                                int lpad, int64_t nkeys, char* tab, int prec) {
+                                int lpad, int64_t nkeys, char* tab, int prec, bool swizzle) {
   sp_table_fill(wsb, s, seed, first, n1, nr, ell, lpad, nkeys, tab,
-                (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, prec);
+                (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x, prec, swizzle);
 }
 
 // Launch arguments of one item (the whole last mode when count = n_d), shared
@@ -702,7 +704,7 @@ __global__ void rows_table_batched_kernel(char* wsb, int lpad) {
     const int nr = k.col ? (int)it.n[it.d - 1] : (int)it.n[0];
     sp_table_fill(wsb, k, it.seed, 0, it.n[0], nr, d.width, lpad, k.col ? it.W / d.wdiv : d.wdiv,
                   wsb + d.st_tab, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
-                  (int64_t)gridDim.x * blockDim.x, it.prec);
+                  (int64_t)gridDim.x * blockDim.x, it.prec, true);
   }
 }
 
@@ -758,7 +760,7 @@ bool plan_sp(const Plan& P, int item, int64_t count, SpArgs* out, size_t* smem, 
 }  // namespace sp
 
 cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint64_t seed, int64_t first, int64_t n1,
-                              int nr, int lpad, int64_t nkeys, char* tab, int prec, cudaStream_t st) {
+                              int nr, int lpad, int64_t nkeys, char* tab, int prec, bool swizzle, cudaStream_t st) {
   sp::SpSk k;
   memset(&k, 0, sizeof(k));
   k.hstride = d.hstride;
@@ -768,7 +770,8 @@ cudaError_t launch_rows_table(const DevSketch& d, int gsk, const char* wsb, uint
   const int64_t total = nkeys * nr * (lpad / 4);
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 16LL * device_sm_count()));
   count_launch();
-  sp::sp_table_kernel<<<blocks, 256, 0, st>>>(wsb, k, seed, first, n1, nr, d.width, lpad, nkeys, tab, prec);
+  sp::sp_table_kernel<<<blocks, 256, 0, st>>>(wsb, k, seed, first, n1, nr, d.width, lpad, nkeys, tab, prec,
+                                             swizzle);
   return cudaGetLastError();
 }
 
@@ -824,7 +827,7 @@ cudaError_t launch_sketch_sp(const Plan& P, int item, const void* X, int64_t fir
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, 16LL * device_sm_count());
     count_launch();
     sp::sp_table_kernel<<<blocks, 256, 0, st>>>(g.wsb, k, g.seed, first, g.n1, nr, k.ell, lpad, nkeys,
-                                                g.wsb + g.tab0 + k.tab, it.prec);
+                                                g.wsb + g.tab0 + k.tab, it.prec, false);
   }
   const int64_t nblocks = g.tilesL * g.tilesR;
   const int grid = (int)std::min<int64_t>(nblocks, device_sm_count());

@@ -266,7 +266,7 @@ cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t 
     const int lpad = strip::ldg_bytes(fmt, nt) / strip::esz(fmt);
     const cudaError_t e = launch_rows_table(d, it.sk0 + s, (const char*)ws, it.seed, first, it.n[0],
                                             col ? (int)count : (int)it.n[0], lpad, col ? it.W / d.wdiv : d.wdiv,
-                                            (char*)ws + d.st_tab, it.prec, st);
+                                            (char*)ws + d.st_tab, it.prec, true, st);
     if (e != cudaSuccess) return e;
   }
   const strip::KernelFn k = fmt == strip::kFmtTF32   ? strip::kernel_tf32(nt, g.ncol)

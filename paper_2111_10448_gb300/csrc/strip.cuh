@@ -269,11 +269,10 @@ template <int FMT>
 __device__ __forceinline__ void put_quad(char* gs, int ldg, int r, int q, float4 z, int width) {
   const float z0 = 4 * q < width ? z.x : 0.f, z1 = 4 * q + 1 < width ? z.y : 0.f;
   const float z2 = 4 * q + 2 < width ? z.z : 0.f, z3 = 4 * q + 3 < width ? z.w : 0.f;
-  char* p = gs + r * ldg + 4 * esz(FMT) * q;
   if constexpr (FMT == kFmtTF32)
-    *reinterpret_cast<float4*>(p) = make_float4(round_tf32(z0), round_tf32(z1), round_tf32(z2), round_tf32(z3));
+    *reinterpret_cast<float4*>(gs + r * ldg + 16 * q) = make_float4(round_tf32(z0), round_tf32(z1), round_tf32(z2), round_tf32(z3));
   else
-    *reinterpret_cast<uint2*>(p) =
+    *reinterpret_cast<uint2*>(gs + r * ldg + 16 * ((q >> 1) ^ strip_swizzle(ldg / 16, r)) + 8 * (q & 1)) =
         make_uint2(tc::op16x2_bits<FMT == kFmtFP16>(z0, z1), tc::op16x2_bits<FMT == kFmtFP16>(z2, z3));
 }
 
@@ -354,10 +353,12 @@ __device__ __forceinline__ void step(float (*t)[4], const uint32_t* xh, const ui
   const int lane = threadIdx.x & 31;
   constexpr int LDG = ldg_bytes(FMT, NT);
   if constexpr (FMT != kFmtTF32) {
-    const uint32_t p = gs + (k0 + (lane & 7) + 8 * ((lane >> 3) & 1)) * LDG + 16 * (lane >> 4);
+    // chunk n + (lane >> 4) of row k0 + ..., swizzled: n even, so n + m = n ^ m
+    const uint32_t m = (uint32_t)((lane >> 4) ^ strip_swizzle(NT, lane & 7));
+    const uint32_t p = gs + (k0 + (lane & 7) + 8 * ((lane >> 3) & 1)) * LDG;
     uint32_t b[(NT + 1) / 2][4];
 #pragma unroll
-    for (int n = 0; n + 1 < NT; n += 2) ldsm4t(p + 16 * n, b[n / 2]);
+    for (int n = 0; n + 1 < NT; n += 2) ldsm4t(p + 16 * (m ^ (uint32_t)n), b[n / 2]);
     if constexpr (NT & 1) ldsm2t(gs + (k0 + (lane & 15)) * LDG + 16 * (NT - 1), b[NT / 2]);
 #pragma unroll
     for (int n = 0; n < NT; ++n) mma<FMT, FIRST>(t[n], xh, b[n / 2] + 2 * (n & 1));
