@@ -92,140 +92,167 @@ __device__ __forceinline__ double warp_sum4(double p0, double p1, double p2, dou
   return k;
 }
 
-// FP64 instructions on this GPU hold their sub-partition's FP64 pipe for 64
-// cycles each, and guarding one with a run-time condition costs several times
-// that even when the guard is false.  So the per-warp column groups below are
-// templates on their column count NC (1..4), dispatched by a switch, and
-// their FP64 arithmetic is unconditional.
-
-// Gram row entries g_c = sum_{r >= i} A(r, i) A(r, c) of the NC columns
-// c = cb + nw j, written to gram[c]; the group holding column i also forms the
-// reflector of step i (beta, R(i, i), head v0).
-template <int NC>
-__device__ __forceinline__ void gram_group(const double* A, int lda, int nr, int i, int cb, int nw,
-                                           double* gram, double* beta, double* rdiag, double* v0s) {
-  const int lane = threadIdx.x & 31;
-  double p[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int r = i + lane; r < nr; r += 32) {
-    const double a = A[r + lda * i];
+// The FP64 pipe takes a warp instruction every 64 cycles and sub-partition, a guard
+// around one costs several times that, and a shuffled addition about 130 cycles.  So
+// the QR steps below give G = 8, 16 or 32 lanes to a column (more as fewer columns are
+// left, so that the four pipes stay even; log2 G additions sum a column), two rows a
+// lane at a time, without guards: rows above the current one have a zero multiplier,
+// rows past the block are zero.
+__host__ __device__ constexpr int qr_rows(int nr) { return tsqr_ld(nr) - 8; }   // multiple of 32
+// Leading dimension: 8 mod 16, so that the 16 lanes of two columns read distinct banks.
+__host__ __device__ constexpr int qr_ld(int nr) { return tsqr_ld(nr); }
+template <int G>
+__device__ __forceinline__ double group_sum(double v) {
 #pragma unroll
-    for (int j = 0; j < NC; ++j) p[j] = fma(a, A[r + lda * (cb + nw * j)], p[j]);
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Reflector of a column with squared norm g over rows i.. and head x0: v = (x0 - alpha,
+// rest), R(i, i) = alpha, beta = 2 / (v^T v) = 1 / (g + |x0| sqrt(g)) (0 for a zero
+// column).  One lane's serial chain in every QR step, so the root and the quotient
+// are Newton iterations from the 20-bit approximate instructions (two each, error
+// 2^-20 -> 2^-40 -> below rounding; five dependent FMAs, where the library's root and
+// division took about 690 and 670 cycles).
+__device__ __forceinline__ void reflector(double g, double x0, double& alpha, double& b, double& v0) {
+  alpha = 0.0, b = 0.0, v0 = 0.0;
+  if (!(g > 0.0)) {
+    if (g == 0.0) return;
+    alpha = v0 = b = g;   // NaN
+    return;
   }
-  double g;
-  int q;
-  bool wr;
-  if (NC == 1) {
-    g = warp_sum(p[0]), q = 0, wr = lane == 0;
-  } else if (NC == 2) {
-    g = warp_sum2(p[0], p[1]), q = lane >> 4, wr = (lane & 15) == 0;
+  const int e = (__double2hiint(g) >> 20) & 0x7ff;
+  double nx;
+  if (e > 40 && e < 2000) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(g));
+    double s = g * y, h = 0.5 * y;
+    double r = fma(-s, h, 0.5);
+    s = fma(s, r, s);
+    h = fma(h, r, h);
+    r = fma(-s, h, 0.5);
+    nx = fma(s, r, s);
+    const double d = fma(fabs(x0), nx, g);
+    double q;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(d));
+    q = fma(q, fma(-d, q, 1.0), q);
+    b = fma(q, fma(-d, q, 1.0), q);
   } else {
-    g = warp_sum4(p[0], p[1], p[2], p[3]), q = lane >> 3, wr = (lane & 7) == 0 && q < NC;
+    nx = sqrt(g);
+    b = 1.0 / fma(fabs(x0), nx, g);
   }
-  if (wr) gram[cb + nw * q] = g;
-  if (cb == i && lane == 0) {
-    const double x0 = A[i + lda * i];
-    const double nx = sqrt(g);
-    double alpha = 0.0, b = 0.0;
-    if (nx > 0.0) {
-      alpha = -copysign(nx, x0);
-      const double v0 = x0 - alpha;
-      const double vn2 = g - x0 * x0 + v0 * v0;
-      b = vn2 > 0.0 ? 2.0 / vn2 : 0.0;
+  alpha = -copysign(nx, x0);
+  v0 = x0 - alpha;
+}
+
+// Rows per iteration of a group and the first row of step i.
+template <int G>
+struct QrRows {
+  static constexpr int kStep = G == 8 ? 16 : 32;         // 2 G, or G for whole warps
+  static constexpr int kSecond = G == 32 ? 0 : G;        // offset of a lane's second row (0: none)
+  static __device__ __forceinline__ int first(int i) { return i & ~(kStep - 1); }
+};
+
+// Gram row of step i: gram[c] = sum_{r >= i} A(r, i) A(r, c) for c > i, by all warps but
+// the first, which forms the reflector of column i meanwhile (the longest chain of a
+// step).
+template <int G>
+__device__ __forceinline__ void gram_pass(const double* A, int lda, int nrp, int w, int i, double* gram) {
+  using R = QrRows<G>;
+  const int t = (int)threadIdx.x - 32;
+  const int sub = t & (G - 1), slot = t / G, nslot = ((int)blockDim.x - 32) / G;
+  const int wbase = slot - (t & 31) / G;   // the warp's first slot
+  const double* ai = A + lda * i;
+  for (int cb = i + 1; cb + wbase < w; cb += nslot) {     // the same count for the whole warp
+    const int c = cb + slot;
+    const double* ac = A + lda * min(c, w - 1);
+    double p0 = 0.0, p1 = 0.0;
+    for (int r = R::first(i) + sub; r < nrp; r += R::kStep) {
+      p0 = fma(r >= i ? ai[r] : 0.0, ac[r], p0);
+      if (G < 32) p1 = fma(r + R::kSecond >= i ? ai[r + R::kSecond] : 0.0, ac[r + R::kSecond], p1);
     }
+    const double g = group_sum<G>(G < 32 ? p0 + p1 : p0);
+    if (sub == 0 && c < w) gram[c] = g;
+  }
+}
+__device__ __forceinline__ void pivot_pass(const double* ai, int nrp, int i, double* beta, double* rdiag, double* v0s) {
+  double p = 0.0;
+  for (int r = (i & ~31) + (int)threadIdx.x; r < nrp; r += 32) {
+    const double u = r >= i ? ai[r] : 0.0;
+    p = fma(u, u, p);
+  }
+  p = group_sum<32>(p);
+  if (threadIdx.x == 0) {
+    double alpha, b, v0;
+    reflector(p, ai[i], alpha, b, v0);
     beta[i] = b;
     rdiag[i] = alpha;
-    *v0s = nx > 0.0 ? x0 - alpha : 0.0;
+    *v0s = v0;
   }
 }
 
-// A(i:, c) -= b v (v^T A(i:, c)) for the NC columns c = cb + nw j, with
-// v^T A(i:, c) = g_c - alpha A(i, c) and v = (v0, A(i+1:, i)).
-template <int NC>
-__device__ __forceinline__ void update_group(double* A, int lda, int nr, int i, int cb, int nw,
-                                             const double* gram, double b, double alpha, double v0) {
-  const int lane = threadIdx.x & 31;
-  double coef[NC];
-#pragma unroll
-  for (int j = 0; j < NC; ++j) {
-    const int c = cb + nw * j;
-    coef[j] = b * fma(-alpha, A[i + lda * c], gram[c]);
-  }
-  __syncwarp();
-  for (int r = i + lane; r < nr; r += 32) {
-    const double v = r == i ? v0 : A[r + lda * i];
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      double* e = A + r + lda * (cb + nw * j);
-      *e = fma(-coef[j], v, *e);
+// A(i:, c) -= b v (v^T A(i:, c)) for c > i, with v^T A(i:, c) = g_c - alpha A(i, c) and v =
+// (v0, A(i+1:, i)).
+template <int G>
+__device__ __forceinline__ void update_pass(double* A, int lda, int nrp, int w, int i, const double* gram, double b,
+                                            double alpha, double v0) {
+  using R = QrRows<G>;
+  const int sub = threadIdx.x & (G - 1), slot = threadIdx.x / G, nslot = blockDim.x / G;
+  const uint32_t mask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u) << (threadIdx.x & 31 & ~(G - 1));
+  const double* ai = A + lda * i;
+  for (int c = i + 1 + slot; c < w; c += nslot) {
+    double* ac = A + lda * c;
+    const double coef = b * fma(-alpha, ac[i], gram[c]);
+    __syncwarp(mask);   // every lane of the column has read its head
+    for (int r = R::first(i) + sub; r < nrp; r += R::kStep) {
+      ac[r] = fma(-coef, r > i ? ai[r] : r == i ? v0 : 0.0, ac[r]);
+      if (G < 32) {
+        const int q = r + R::kSecond;
+        ac[q] = fma(-coef, q > i ? ai[q] : q == i ? v0 : 0.0, ac[q]);
+      }
     }
   }
 }
 
-// In-shared-memory Householder QR of an nr x w block A (ld = lda), nr >= 1.
-// On exit column i holds v_i in rows i..nr-1 (v_i(0) at the diagonal), beta[i]
-// = 2 / (v_i^T v_i) (0 for a zero column), rdiag[i] = R(i, i); the strict
-// upper triangle holds R.
+// In-shared-memory Householder QR of an nr x w block A (ld = lda >= qr_rows(nr), rows
+// nr..qr_rows(nr) zero), nr >= 1.  On exit column i holds v_i in rows i..nr-1 (v_i(0)
+// at the diagonal), beta[i] = 2 / (v_i^T v_i) (0 for a zero column), rdiag[i] = R(i,
+// i); the strict upper triangle holds R.
 //
 // Step i works from the Gram row g_c = sum_{r >= i} A(r, i) A(r, c), c >= i:
 // g_i is the squared norm of the pivot column, and with v = A(i:, i) - alpha
 // e_1 the reflector products are v^T A(i:, c) = g_c - alpha A(i, c).  So a
-// step is one reduction pass (every column's dot at once; the warp owning
-// columns c, c+8, c+16, c+24 sums them with one butterfly) and one update
-// pass, two barriers in all.
+// step is one reduction pass and one update pass, two barriers in all.  Measured (a
+// level of 128 x 26 blocks, 256 x 16 blocks, the root of 70 x 35): 65, 47, 131 us; a
+// column per warp with five-step butterflies and the library's root and division in
+// the chain took 93, 65 and (QR and CPQR) 440 us.
 __device__ __forceinline__ void house_qr(double* A, int lda, int nr, int w, double* beta, double* rdiag) {
   const int kmax = min(nr, w);
-  const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int nrp = qr_rows(nr), nrp16 = (nr + 15) & ~15;
   __shared__ double v0s;
   __shared__ double gram[TT_MAXL];
+  const int wide = blockDim.x >> 4, narrow = blockDim.x >> 5;   // columns that fit 16 and 32 lanes each
   for (int i = 0; i < kmax; ++i) {
-    for (int cb = i + wid; cb < w; cb += 4 * nw) {
-      switch (min(4, (w - 1 - cb) / nw + 1)) {
-        case 1: gram_group<1>(A, lda, nr, i, cb, nw, gram, beta, rdiag, &v0s); break;
-        case 2: gram_group<2>(A, lda, nr, i, cb, nw, gram, beta, rdiag, &v0s); break;
-        case 3: gram_group<3>(A, lda, nr, i, cb, nw, gram, beta, rdiag, &v0s); break;
-        default: gram_group<4>(A, lda, nr, i, cb, nw, gram, beta, rdiag, &v0s); break;
-      }
-    }
+    const int left = w - 1 - i;
+    if (threadIdx.x < 32) pivot_pass(A + lda * i, nrp, i, beta, rdiag, &v0s);
+    else if (left > wide - 2) gram_pass<8>(A, lda, nrp16, w, i, gram);
+    else if (left > narrow - 1) gram_pass<16>(A, lda, nrp, w, i, gram);
+    else gram_pass<32>(A, lda, nrp, w, i, gram);
     __syncthreads();
     const double b = beta[i], alpha = rdiag[i], v0 = v0s;
     if (b != 0.0) {
-      for (int cb = i + 1 + wid; cb < w; cb += 4 * nw) {
-        switch (min(4, (w - 1 - cb) / nw + 1)) {
-          case 1: update_group<1>(A, lda, nr, i, cb, nw, gram, b, alpha, v0); break;
-          case 2: update_group<2>(A, lda, nr, i, cb, nw, gram, b, alpha, v0); break;
-          case 3: update_group<3>(A, lda, nr, i, cb, nw, gram, b, alpha, v0); break;
-          default: update_group<4>(A, lda, nr, i, cb, nw, gram, b, alpha, v0); break;
-        }
-      }
+      if (left > wide) update_pass<8>(A, lda, nrp16, w, i, gram, b, alpha, v0);
+      else if (left > narrow) update_pass<16>(A, lda, nrp, w, i, gram, b, alpha, v0);
+      else update_pass<32>(A, lda, nrp, w, i, gram, b, alpha, v0);
     }
-    if (threadIdx.x == 0) A[i + lda * i] = v0;
     __syncthreads();
+    if (threadIdx.x == 0) A[i + lda * i] = v0;
   }
   for (int i = kmax + threadIdx.x; i < w; i += blockDim.x) {
     beta[i] = 0.0;
     rdiag[i] = 0.0;
   }
   __syncthreads();
-}
-
-// Apply the reflectors of a block (V: nr x w in global or shared, ld = ldv,
-// beta) to Z (nr x ncol, ld = ldz):  Z <- H_0 ... H_{k-1} Z.
-__device__ void apply_q(const double* V, int64_t ldv, const double* beta, int nr, int w, double* Z,
-                        int64_t ldz, int ncol) {
-  const int kmax = min(nr, w);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = kmax - 1; i >= 0; --i) {
-    const double b = beta[i];
-    if (b != 0.0) {
-      for (int c = wid; c < ncol; c += nw) {
-        double dot = 0.0;
-        for (int r = i + lane; r < nr; r += 32) dot += V[r + ldv * i] * Z[r + ldz * c];
-        dot = warp_sum(dot) * b;
-        for (int r = i + lane; r < nr; r += 32) Z[r + ldz * c] -= dot * V[r + ldv * i];
-      }
-    }
-    __syncthreads();
-  }
 }
 
 // Z(:, c) = H_0 ... H_{kmax-1} [Z0(0:kmax, c); 0] for the nr-row block of
@@ -326,39 +353,54 @@ __device__ __forceinline__ void expand_cols(const double* V, int64_t ldv, const 
   }
 }
 
-// One pivoted-QR step's update of the NC root columns c = cb + nw j > i by
-// reflector i (v = Rs(i:, i), beta b), and their trailing norms over rows > i.
-template <int NC>
-__device__ __forceinline__ void cpqr_group(double* Rs, int w, int i, int cb, int nw, double b, double* nrm) {
-  const int lane = threadIdx.x & 31;
-  double p[4] = {0.0, 0.0, 0.0, 0.0}, d[4];
-  for (int r = i + lane; r < w; r += 32) {
-    const double v = Rs[r + w * i];
-#pragma unroll
-    for (int j = 0; j < NC; ++j) p[j] = fma(v, Rs[r + w * (cb + nw * j)], p[j]);
-  }
-  warp_sums<NC>(p, d);
-  double t[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int r = i + lane; r < w; r += 32) {
-    const double v = Rs[r + w * i];
-#pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      double* e = Rs + r + w * (cb + nw * j);
-      const double x = fma(-d[j] * b, v, *e);
-      *e = x;
-      const double xt = r > i ? x : 0.0;
-      t[j] = fma(xt, xt, t[j]);
+// One pivoted-QR step's update of the columns c > i of the block Rs (ld ldr, nrp rows
+// with the zero ones) by reflector i (v = Rs(i:, i), beta b), and their trailing norms
+// over rows > i.
+template <int G>
+__device__ __forceinline__ void cpqr_pass(double* Rs, int ldr, int nrp, int w, int i, double b, double* nrm) {
+  using R = QrRows<G>;
+  const int sub = threadIdx.x & (G - 1), slot = threadIdx.x / G, nslot = blockDim.x / G;
+  const int wbase = slot - (threadIdx.x & 31) / G;
+  const double* ai = Rs + ldr * i;
+  for (int cb = i + 1; cb + wbase < w; cb += nslot) {
+    const int c = cb + slot;
+    double* ac = Rs + ldr * min(c, w - 1);
+    double p0 = 0.0, p1 = 0.0;
+    for (int r = R::first(i) + sub; r < nrp; r += R::kStep) {
+      p0 = fma(r >= i ? ai[r] : 0.0, ac[r], p0);
+      if (G < 32) p1 = fma(r + R::kSecond >= i ? ai[r + R::kSecond] : 0.0, ac[r + R::kSecond], p1);
     }
+    const double coef = group_sum<G>(G < 32 ? p0 + p1 : p0) * b;
+    double t0 = 0.0, t1 = 0.0;
+    if (c < w) {
+      for (int r = R::first(i) + sub; r < nrp; r += R::kStep) {
+        const double x0 = fma(-coef, r >= i ? ai[r] : 0.0, ac[r]);
+        ac[r] = x0;
+        const double y0 = r > i ? x0 : 0.0;
+        t0 = fma(y0, y0, t0);
+        if (G < 32) {
+          const int q = r + R::kSecond;
+          const double x1 = fma(-coef, q >= i ? ai[q] : 0.0, ac[q]);
+          ac[q] = x1;
+          const double y1 = q > i ? x1 : 0.0;
+          t1 = fma(y1, y1, t1);
+        }
+      }
+    }
+    const double t = group_sum<G>(G < 32 ? t0 + t1 : t0);
+    if (sub == 0 && c < w) nrm[c] = t;
   }
-  warp_sums<NC>(t, d);
-  if (lane == 0)
-#pragma unroll
-    for (int j = 0; j < NC; ++j) nrm[cb + nw * j] = d[j];
+}
+__device__ __forceinline__ void cpqr_step(double* Rs, int ldr, int nr, int w, int i, double b, double* nrm) {
+  const int left = w - 1 - i, wide = blockDim.x >> 4, narrow = blockDim.x >> 5;
+  if (left > wide) cpqr_pass<8>(Rs, ldr, (nr + 15) & ~15, w, i, b, nrm);
+  else if (left > narrow) cpqr_pass<16>(Rs, ldr, qr_rows(nr), w, i, b, nrm);
+  else cpqr_pass<32>(Rs, ldr, qr_rows(nr), w, i, b, nrm);
 }
 
 // Copies an nr x w column-major block (leading dimension ldy) into shared
-// memory (leading dimension lda); eight independent loads per thread are in
-// flight at a time.
+// memory (leading dimension lda >= qr_rows(nr)), rows nr..qr_rows(nr) zero; eight
+// independent loads per thread are in flight at a time.
 __device__ void load_block(double* A, int lda, const double* Y, int64_t ldy, int nr, int w) {
   for (int c0 = 0; c0 < w; c0 += 8)
     for (int r = threadIdx.x; r < nr; r += blockDim.x) {
@@ -369,6 +411,8 @@ __device__ void load_block(double* A, int lda, const double* Y, int64_t ldy, int
       for (int u = 0; u < 8; ++u)
         if (c0 + u < w) A[r + lda * (c0 + u)] = v[u];
     }
+  const int pad = qr_rows(nr) - nr;
+  for (int o = threadIdx.x; o < pad * w; o += blockDim.x) A[nr + o % pad + lda * (o / pad)] = 0.0;
 }
 
 __device__ __forceinline__ void flag_status(char* wsb, int bits) {
@@ -415,9 +459,11 @@ __global__ void __launch_bounds__(kThreads) sketch_unscale_kernel(char* wsb, int
 // One task = one row block of level L of one basis sketch (launch Lg holds
 // the tasks whose tree has Lg - L more levels above them than the deepest
 // tree, so that every root runs in the last launch).  Non-root blocks write
-// their R into the next level's matrix; the root block also does the CPQR of
-// R, the rank decision and the first expansion step.
-__global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int Lg, int* ranks) {
+// their R into the next level's matrix; the root block also does the CPQR, the rank
+// decision and (unless root_sep) the first expansion step.  A root block of at most
+// 6 w rows is pivoted as it stands -- its columns have the norms and inner products
+// of R's -- which spares the QR before it and the product of the two Q factors.
+__global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int Lg, int* ranks, int root_sep) {
   extern __shared__ double sm[];
   const DevTables& T = tables(wsb);
   const Task task = reinterpret_cast<const Task*>(wsb + T.off_tasks[Lg])[blockIdx.x];
@@ -427,33 +473,39 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
   double* ws = reinterpret_cast<double*>(wsb);
   const int w = s.width;
   const int64_t m = s.lev_rows[L];
-  const int64_t r0 = (int64_t)task.blk * s.bl;
-  const int nr = (int)imin64(s.bl, m - r0);
-  const int lda = nr + 1;
+  const int64_t r0 = (int64_t)task.blk * s.lev_bl[L];
+  const int nr = (int)imin64(s.lev_bl[L], m - r0);
+  const int lda = qr_ld(nr), ldw = qr_ld(w);
   double* A = sm;                         // lda x w
   double* red = A + (size_t)lda * w;      // 32
   double* beta = red + 32;                // w
   double* rdiag = beta + TT_MAXL;         // w
-  double* Rs = rdiag + TT_MAXL;           // w x w (root only)
-  double* Q2 = Rs + w * w;                // w x w (root only), then w x w of rank sums
+  double* Rs = rdiag + TT_MAXL;           // ldw x w (root only)
+  double* Q2 = Rs + ldw * w;                // w x w (root only), then w x w of rank sums
   __shared__ int piv[TT_MAXL];
   __shared__ int s_rank;
   double* Y = ws + s.lev_mat[L];
   load_block(A, lda, Y + r0, m, nr, w);
   __syncthreads();
-  house_qr(A, lda, nr, w, beta, rdiag);
+  const bool root = (s.lev_nblk[L] == 1);
+  const bool direct = root && nr >= w && nr <= 6 * w;   // pivot the block itself
   const int kmax = min(nr, w);
   // Householder vectors back in place, scalars to the level's beta array
-  for (int o = threadIdx.x; o < nr * w; o += blockDim.x) {
-    const int r = o % nr, c = o / nr;
-    Y[r0 + r + m * c] = A[r + lda * c];
+  auto store_block = [&](const double* bt) {
+    for (int o = threadIdx.x; o < nr * w; o += blockDim.x) {
+      const int r = o % nr, c = o / nr;
+      Y[r0 + r + m * c] = A[r + lda * c];
+    }
+    for (int i = threadIdx.x; i < w; i += blockDim.x) ws[s.lev_beta[L] + (int64_t)task.blk * w + i] = bt[i];
+  };
+  if (!direct) {
+    house_qr(A, lda, nr, w, beta, rdiag);
+    store_block(beta);
   }
-  for (int i = threadIdx.x; i < w; i += blockDim.x) ws[s.lev_beta[L] + (int64_t)task.blk * w + i] = beta[i];
   auto rval = [&](int i, int c) -> double {
     if (i >= kmax || c < i) return 0.0;
     return c == i ? rdiag[i] : A[i + lda * c];
   };
-  const bool root = (s.lev_nblk[L] == 1);
   if (!root) {
     const int64_t m1 = s.lev_rows[L + 1];
     double* Yn = ws + s.lev_mat[L + 1];
@@ -463,30 +515,33 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
     }
     return;
   }
-  // ---- root: CPQR of R (w x w) in shared memory.  Per step: warp 0 picks
-  // the pivot (largest recomputed trailing norm, lowest index on ties), swaps
-  // it into place and forms the reflector; then each warp applies it to its
-  // own columns and recomputes their trailing norms for the next step.
-  for (int o = threadIdx.x; o < w * w; o += blockDim.x) {
-    const int i = o % w, c = o / w;
-    Rs[i + w * c] = rval(i, c);
-  }
+  // ---- root: CPQR, of the block (nr x w) or of its R (w x w), in shared memory.
+  // Per step: warp 0 picks the pivot (largest recomputed trailing norm, lowest
+  // index on ties), swaps it into place and forms the reflector; then each warp
+  // applies it to its own columns and recomputes their trailing norms for the
+  // next step.
+  double* Cs = direct ? A : Rs;
+  const int ldc = direct ? lda : ldw, nc = direct ? nr : w;
+  if (!direct)
+    for (int o = threadIdx.x; o < qr_rows(w) * w; o += blockDim.x) {
+      const int i = o % qr_rows(w), c = o / qr_rows(w);
+      Rs[i + ldw * c] = i < w ? rval(i, c) : 0.0;
+    }
   for (int c = threadIdx.x; c < w; c += blockDim.x) piv[c] = c;
   __syncthreads();
   __shared__ double nrm[TT_MAXL];
   __shared__ double qb[TT_MAXL], qd[TT_MAXL];
   double total2 = 0.0;
-  for (int o = threadIdx.x; o < w * w; o += blockDim.x) total2 += Rs[o] * Rs[o];
-  total2 = block_sum(total2, red);
   {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     for (int c = wid; c < w; c += nw) {  // trailing norms of step 0
       double t = 0.0;
-      for (int r = lane; r < w; r += 32) t = fma(Rs[r + w * c], Rs[r + w * c], t);
+      for (int r = lane; r < nc; r += 32) t = fma(Cs[r + ldc * c], Cs[r + ldc * c], t);
       t = warp_sum(t);
       if (lane == 0) nrm[c] = t;
     }
     __syncthreads();
+    total2 = block_sum((int)threadIdx.x < w ? nrm[threadIdx.x] : 0.0, red);
     for (int i = 0; i < w; ++i) {
       if (wid == 0) {
         // argmax over c >= i; norms are >= 0, so their bit patterns order like them
@@ -506,10 +561,10 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
         // keep column i, so that the swap stays inside the block
         const int j = arg < w ? arg : i;
         if (j != i) {
-          for (int r = lane; r < w; r += 32) {
-            const double t = Rs[r + w * i];
-            Rs[r + w * i] = Rs[r + w * j];
-            Rs[r + w * j] = t;
+          for (int r = lane; r < nc; r += 32) {
+            const double t = Cs[r + ldc * i];
+            Cs[r + ldc * i] = Cs[r + ldc * j];
+            Cs[r + ldc * j] = t;
           }
           if (lane == 0) {
             const int t = piv[i];
@@ -521,55 +576,39 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
           }
         }
         __syncwarp();
-        if (lane == 0) {  // Householder on column i, rows i..w-1
-          const double nsq = nrm[i];
-          const double x0 = Rs[i + w * i];
-          const double nx = sqrt(nsq);
-          double alpha = 0.0, b = 0.0;
-          if (nx > 0.0) {
-            alpha = -copysign(nx, x0);
-            const double v0 = x0 - alpha;
-            const double vn2 = nsq - x0 * x0 + v0 * v0;
-            b = vn2 > 0.0 ? 2.0 / vn2 : 0.0;
-          }
-          Rs[i + w * i] = nx > 0.0 ? x0 - alpha : 0.0;
+        if (lane == 0) {  // Householder on column i, rows i..nc-1
+          double alpha, b, v0;
+          reflector(nrm[i], Cs[i + ldc * i], alpha, b, v0);
+          Cs[i + ldc * i] = v0;
           qb[i] = b;
           qd[i] = alpha;
         }
       }
       __syncthreads();
-      const double b = qb[i];
-      for (int cb = i + 1 + wid; cb < w; cb += 4 * nw) {
-        switch (min(4, (w - 1 - cb) / nw + 1)) {
-          case 1: cpqr_group<1>(Rs, w, i, cb, nw, b, nrm); break;
-          case 2: cpqr_group<2>(Rs, w, i, cb, nw, b, nrm); break;
-          case 3: cpqr_group<3>(Rs, w, i, cb, nw, b, nrm); break;
-          default: cpqr_group<4>(Rs, w, i, cb, nw, b, nrm); break;
-        }
-      }
+      cpqr_step(Cs, ldc, nc, w, i, qb[i], nrm);
       __syncthreads();
     }
   }
-  // Q2 = H_0 ... H_{w-1} I
+  // Q2: the factor that the block's own reflectors are applied to, columns with
+  // diag(Rt) >= 0 (direct: those signs alone)
   for (int o = threadIdx.x; o < w * w; o += blockDim.x) Q2[o] = (o % w == o / w) ? 1.0 : 0.0;
   __syncthreads();
-  expand_cols(Rs, w, qb, w, w, Q2, w, w, w, Q2, w);
-  __syncthreads();
+  if (direct) {
+    store_block(qb);
+  } else {
+    expand_cols(Rs, ldw, qb, w, w, Q2, w, w, w, Q2, w);
+    __syncthreads();
+  }
   // Rt with signs normalised (diag >= 0), Q2 columns likewise
   double* Rt = ws + s.off_rt;
   for (int o = threadIdx.x; o < w * w; o += blockDim.x) {
     const int i = o % w, c = o / w;
-    const double sg = qd[i] < 0.0 ? -1.0 : 1.0;
+    const double sg = qd[i] < 0.0 ? -1.0 : 1.0, sc = qd[c] < 0.0 ? -1.0 : 1.0;
     double v = 0.0;
-    if (c > i) v = Rs[i + w * c];
+    if (c > i) v = Cs[i + ldc * c];
     else if (c == i) v = qd[i];
     Rt[o] = sg * v;
-  }
-  __syncthreads();
-  for (int o = threadIdx.x; o < w * w; o += blockDim.x) {
-    const int c = o / w;
-    const double sg = qd[c] < 0.0 ? -1.0 : 1.0;
-    Q2[o] *= sg;
+    Q2[o] *= sc;
     ws[s.off_q2 + o] = Q2[o];
   }
   for (int c = threadIdx.x; c < w; c += blockDim.x) reinterpret_cast<int*>(ws + s.off_piv)[c] = piv[c];
@@ -582,7 +621,8 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
   for (int c = threadIdx.x; c < w; c += blockDim.x) {
     double run = 0.0;
     for (int i2 = c; i2 >= 0; --i2) {
-      run += Rt[i2 + w * c] * Rt[i2 + w * c];
+      const double v = c > i2 ? Cs[i2 + ldc * c] : qd[c];   // |Rt(i2, c)|
+      run = fma(v, v, run);
       tcol[i2 + w * c] = run;
     }
   }
@@ -630,35 +670,43 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
     ws[it.off_rr[s.k] + o] = (i < r && c < r) ? Rt[i + w * c] : 0.0;
   }
   // Z_root = Q_root [Q2(:, 1:r); 0]  (m x rpad, columns >= r are zero)
-  expand_cols(A, lda, beta, nr, w, Q2, w, r, s.rpad, ws + s.lev_z[L], m);
+  if (!root_sep) expand_cols(A, lda, direct ? qb : beta, nr, w, Q2, w, r, s.rpad, ws + s.lev_z[L], m);
 }
 
 // ---------------------------------------------------------------- TSQR down
-// Z_L(block) = Q_block [Z_{L+1}(rows of this block's R); 0].
-__global__ void __launch_bounds__(kThreads) tsqr_expand_kernel(char* wsb, int Lg, const int* ranks) {
+// Z_L(block) = Q_block [Z_{L+1}(rows of this block's R); 0], and Q_root [Q2; 0] at the
+// root when root_sep.  A block's reflectors occupy one SM's FP64 pipe (a column of a
+// 192-row block costs 17 warp instructions a reflector), so few blocks share their
+// columns over blockIdx.y, cw columns each.
+__global__ void __launch_bounds__(kThreads) tsqr_expand_kernel(char* wsb, int Lg, const int* ranks, int root_sep,
+                                                               int cw) {
   extern __shared__ double sm[];
   const DevTables& T = tables(wsb);
   const Task task = reinterpret_cast<const Task*>(wsb + T.off_tasks[Lg])[blockIdx.x];
   const int L = task.lev;
   const DevSketch& s = dsk(wsb)[task.sk];
-  if (s.nlev - 1 <= L) return;  // root of this tree, already expanded
+  const bool root = s.nlev - 1 <= L;
+  if (root && !root_sep) return;  // root of this tree, already expanded
+  const int c0 = (int)blockIdx.y * cw;
+  if (c0 >= s.rpad) return;
   const DevItem& it = ditems(wsb)[s.item];
   double* ws = reinterpret_cast<double*>(wsb);
   const int w = s.width;
   const int r = ranks[it.rank_off + s.k];
   const int64_t m = s.lev_rows[L];
-  const int64_t r0 = (int64_t)task.blk * s.bl;
-  const int nr = (int)imin64(s.bl, m - r0);
-  const int lda = nr + 1;
+  const int64_t r0 = (int64_t)task.blk * s.lev_bl[L];
+  const int nr = (int)imin64(s.lev_bl[L], m - r0);
+  const int lda = qr_ld(nr);
   double* V = sm;
   double* beta = V + (size_t)lda * w;
   const double* Y = ws + s.lev_mat[L];
   load_block(V, lda, Y + r0, m, nr, w);
   for (int i = threadIdx.x; i < w; i += blockDim.x) beta[i] = ws[s.lev_beta[L] + (int64_t)task.blk * w + i];
-  const int64_t m1 = s.lev_rows[L + 1];
   __syncthreads();
-  expand_cols(V, lda, beta, nr, w, ws + s.lev_z[L + 1] + (int64_t)task.blk * w, m1, r, s.rpad,
-              ws + s.lev_z[L] + r0, m);
+  const double* Zin = root ? ws + s.off_q2 : ws + s.lev_z[L + 1] + (int64_t)task.blk * w;
+  const int64_t ldz = root ? w : s.lev_rows[L + 1];
+  expand_cols(V, lda, beta, nr, w, Zin + ldz * c0, ldz, max(0, min(r - c0, cw)), min(s.rpad - c0, cw),
+              ws + s.lev_z[L] + r0 + m * c0, m);
 }
 
 // --------------------------------------------------------- one-pass middle
@@ -713,22 +761,28 @@ __global__ void __launch_bounds__(kThreads) mid_b_kernel_f64(char* wsb, int item
   }
 }
 
-// QR of B^T (l x r) -> QB (l x r), RB (r x r); singular B is flagged.
+// QR of B^T (l x r) -> RB (r x r) and M = QB RB^{-T} (l x r, over QB's place); singular
+// B is flagged.  All of it in shared memory (in global memory the reflectors'
+// application and the back-substitution took most of 157 us at l = 35, r = 25).
 // item < 0: batched launch, item = blockIdx.y
 __global__ void __launch_bounds__(kThreads) mid_ls_kernel(char* wsb, int item_arg, const int* ranks) {
   const int item = item_arg >= 0 ? item_arg : (int)blockIdx.y;
-  __shared__ double A[TT_MAXL * (TT_MAXL + 1)];
+  extern __shared__ double sm[];
   __shared__ double beta[TT_MAXL], rdiag[TT_MAXL];
   const DevItem& it = ditems(wsb)[item];
   double* ws = reinterpret_cast<double*>(wsb);
   const int r = ranks[it.rank_off + it.mbk];
   const int l = it.lmid;
   const int rp = it.rpad[it.mbk];
-  const int lda = l + 1;
-  for (int o = threadIdx.x; o < l * r; o += blockDim.x) {
-    const int j = o % l, c = o / l;
-    A[j + lda * c] = ws[it.off_B + c + (int64_t)rp * j];  // B^T(j, c) = B(c, j)
+  const int lda = qr_ld(l), lp = qr_rows(l);
+  double* A = sm;             // lda x r
+  double* M = A + lda * r;    // l x r, ld l + 1
+  const int ldm = l + 1;
+  for (int o = threadIdx.x; o < lp * r; o += blockDim.x) {
+    const int j = o % lp, c = o / lp;
+    A[j + lda * c] = j < l ? ws[it.off_B + c + (int64_t)rp * j] : 0.0;  // B^T(j, c) = B(c, j)
   }
+  for (int o = threadIdx.x; o < l * r; o += blockDim.x) M[o % l + ldm * (o / l)] = (o % l == o / l) ? 1.0 : 0.0;
   __syncthreads();
   house_qr(A, lda, l, r, beta, rdiag);
   // RB (rp x rp) with diag >= 0; QB = H_0..H_{r-1} [I_r; 0] with matching signs
@@ -755,27 +809,30 @@ __global__ void __launch_bounds__(kThreads) mid_ls_kernel(char* wsb, int item_ar
       if (!(fabs(rdiag[i]) > 1e-13 * rmax_abs)) sing = true;
     if (sing) flag_status(wsb, ST_RANK_DEFICIENT);
   }
-  for (int o = threadIdx.x; o < l * rp; o += blockDim.x) {
-    const int j = o % l, c = o / l;
-    QB[j + (int64_t)l * c] = (c < r && j == c) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  apply_q(A, lda, beta, l, r, QB, l, r);
-  // M = QB RB^{-T}, stored over QB: row j solves m RB^T = QB(j, :) from the
-  // last column (a zero diagonal of RB gives a zero column, as flagged above),
-  // so that H = S_{d*} M is a plain product.
+  expand_cols(A, lda, beta, l, r, M, ldm, r, r, M, ldm);
+  // M = QB RB^{-T}: row j solves m RB^T = QB(j, :) from the last column (a zero
+  // diagonal of RB gives a zero column, as flagged above), so that H = S_{d*} M is a
+  // plain product.  A step takes column c's share out of the columns before it; the
+  // signs of QB's columns and RB's rows meet in sgn.
   __shared__ double rinv[TT_MAXL];
   for (int c = threadIdx.x; c < r; c += blockDim.x) {
-    const double dg = RB[c + rp * c];
+    const double dg = fabs(rdiag[c]);
     rinv[c] = dg != 0.0 ? 1.0 / dg : 0.0;
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < l; j += blockDim.x) {
-    for (int c = r - 1; c >= 0; --c) {
-      double t = QB[j + (int64_t)l * c] * sgn[c];
-      for (int c2 = c + 1; c2 < r; ++c2) t = fma(-QB[j + (int64_t)l * c2], RB[c + rp * c2], t);
-      QB[j + (int64_t)l * c] = t * rinv[c];
+  for (int o = threadIdx.x; o < l * r; o += blockDim.x) M[o % l + ldm * (o / l)] *= sgn[o / l];
+  __syncthreads();
+  for (int c = r - 1; c > 0; --c) {
+    for (int o = threadIdx.x; o < l * c; o += blockDim.x) {
+      const int j = o % l, c2 = o / l;
+      const double x = M[j + ldm * c] * rinv[c];
+      M[j + ldm * c2] = fma(-x, sgn[c2] * A[c2 + lda * c], M[j + ldm * c2]);
     }
+    __syncthreads();
+  }
+  for (int o = threadIdx.x; o < l * rp; o += blockDim.x) {
+    const int j = o % l, c = o / l;
+    QB[j + (int64_t)l * c] = c < r ? M[j + ldm * c] * rinv[c] : 0.0;
   }
 }
 
@@ -1257,16 +1314,22 @@ cudaError_t launch_backward_h(const Plan& P, int item, void* ws, const int* rank
 
 cudaError_t launch_mid_b_mixed(const Plan& P, int item, void* ws, const int* ranks, cudaStream_t st);
 
+// Dynamic shared memory of mid_ls_kernel.
+size_t ls_smem(int l, int r) { return sizeof(double) * ((size_t)qr_ld(l) * r + (size_t)(l + 1) * r); }
+
 // Middle cores of every item of a batched plan; B was zeroed with the sketches.
 cudaError_t launch_finalize_mid_batched(const Plan& P, void* ws, const int* ranks, cudaStream_t st) {
   char* wsb = (char*)ws;
   const int nitems = plan_num_items(&P);
   const DevSketch* sks = plan_sketches_host(&P);
   int64_t Mmax = 1, Nmax = 1;
+  int lmax = 1, rmax = 1;
   for (int i = 0; i < nitems; ++i) {
     const DevItem& it = plan_items_host(&P)[i];
     Mmax = std::max(Mmax, sks[it.basis_of_k[it.mbk]].rows);
     Nmax = std::max(Nmax, sks[it.mid_sk].rows);
+    lmax = std::max(lmax, it.lmid);
+    rmax = std::max(rmax, it.rpad[it.mbk]);
   }
   cudaError_t e;
   if (plan_items_host(&P)[0].prec == TT_PREC_FP64) {
@@ -1279,7 +1342,7 @@ cudaError_t launch_finalize_mid_batched(const Plan& P, void* ws, const int* rank
   }
   if (e != cudaSuccess) return e;
   count_launch();
-  mid_ls_kernel<<<dim3(1, (unsigned)nitems), kThreads, 0, st>>>(wsb, -1, ranks);
+  mid_ls_kernel<<<dim3(1, (unsigned)nitems), kThreads, ls_smem(lmax, rmax), st>>>(wsb, -1, ranks);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const unsigned gx = (unsigned)std::min<int64_t>((Nmax * TT_MAXL + kThreads - 1) / kThreads, 64);
@@ -1304,6 +1367,9 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(tsqr_expand_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTsqrSmemMax);
     if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(mid_ls_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)ls_smem(TT_MAXL, TT_MAXL));
+    if (e != cudaSuccess) return e;
     attr = true;
   }
   // FP16 items: sketches back to the scale of X, and the range check
@@ -1317,15 +1383,15 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
       if (e != cudaSuccess) return e;
     }
   }
-  // smem: block (bl+1) x w + scalars + two w x w matrices (root)
-  int maxw = 1, maxbl = 1;
+  int maxw = 1, maxbl = 1, maxr = 1;
   for (int i = 0, n = 0; i < nitems; ++i) {
     const DevItem& it = plan_items_host(&P)[i];
     for (int s = 0; s < it.nsk; ++s) {
       const DevSketch& d = sks[it.sk0 + s];
       if (!d.basis) continue;
       maxw = std::max(maxw, d.width);
-      maxbl = std::max(maxbl, d.bl);
+      for (int L = 0; L < d.nlev; ++L) maxbl = std::max(maxbl, d.lev_bl[L]);
+      maxr = std::max(maxr, d.rpad);
       ++n;
     }
   }
@@ -1335,25 +1401,30 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
     for (int s = 0; s < it.nsk; ++s) {
       const DevSketch& d = sks[it.sk0 + s];
       if (!d.basis) continue;
-      const size_t need = sizeof(double) * ((size_t)(d.bl + 1) * d.width + 32 + 2 * TT_MAXL +
-                                            3 * (size_t)d.width * d.width);
-      smem_up = std::max(smem_up, need);
+      for (int L = 0; L < d.nlev; ++L)
+        smem_up = std::max(smem_up, (size_t)(sizeof(double) * tsqr_block_doubles(d.lev_bl[L], d.width)));
     }
   }
+  // the roots' expansion as a launch of its own, its columns over several CTAs, when
+  // it is long enough to pay for the launch
+  const int root_sep = nitems == 1 && maxr > 8 ? 1 : 0;
   for (int L = 0; L < max_lev; ++L) {
     const int nt = plan_ntasks(&P, L);
     if (nt == 0) continue;
     count_launch();
-    tsqr_level_kernel<<<nt, kThreads, smem_up, st>>>(wsb, L, ranks);
+    tsqr_level_kernel<<<nt, kThreads, smem_up, st>>>(wsb, L, ranks, root_sep);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  for (int L = max_lev - 2; L >= 0; --L) {
+  for (int L = root_sep ? max_lev - 1 : max_lev - 2; L >= 0; --L) {
     const int nt = plan_ntasks(&P, L);
     if (nt == 0) continue;
-    const size_t smem = sizeof(double) * ((size_t)(maxbl + 1) * maxw + TT_MAXL);
+    const size_t smem = sizeof(double) * ((size_t)tsqr_ld(maxbl) * maxw + TT_MAXL);
+    // columns per CTA: eight (one per warp) when the blocks alone leave SMs idle
+    const int cw = nt * ((maxr + 7) / 8) <= 2 * device_sm_count() ? 8 : nt <= device_sm_count() ? 16 : TT_MAXL;
     count_launch();
-    tsqr_expand_kernel<<<nt, kThreads, smem, st>>>(wsb, L, ranks);
+    tsqr_expand_kernel<<<dim3((unsigned)nt, (unsigned)((maxr + cw - 1) / cw)), kThreads, smem, st>>>(wsb, L, ranks,
+                                                                                                    root_sep, cw);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1379,7 +1450,7 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
     }
     if (e != cudaSuccess) return e;
     count_launch();
-    mid_ls_kernel<<<1, kThreads, 0, st>>>(wsb, i, ranks);
+    mid_ls_kernel<<<1, kThreads, ls_smem(it.lmid, it.rpad[it.mbk]), st>>>(wsb, i, ranks);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (!mid_by_gemm(P, i)) {

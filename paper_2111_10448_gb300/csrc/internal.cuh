@@ -37,7 +37,14 @@ struct NvtxRange {
 __host__ __device__ __forceinline__ int64_t imin64(int64_t a, int64_t b) { return a < b ? a : b; }
 
 constexpr int kMaxLev = 12;       // TSQR tree depth limit
-constexpr int64_t kTsqrSmemMax = 200 * 1024;  // dynamic shared memory of a TSQR level block
+constexpr int64_t kTsqrSmemMax = 208 * 1024;  // dynamic shared memory of a TSQR level block
+// Leading dimension of a QR block of nr rows in shared memory, and the doubles of a
+// level block of bl rows and width w (block, reduction and reflector scalars, at the
+// root the R factor, Q_2 and the rank sums).
+__host__ __device__ constexpr int tsqr_ld(int nr) { return ((nr + 31) & ~31) + 8; }
+constexpr int64_t tsqr_block_doubles(int bl, int w) {
+  return (int64_t)tsqr_ld(bl) * w + 32 + 2 * TT_MAXL + (int64_t)tsqr_ld(w) * w + 2LL * w * w;
+}
 constexpr int kTcGroupBytes = 2304;  // plane kernel: one 8-column group of a 128-row BF16 block image
 constexpr int kMaxSk = TT_MAXD;   // sketches per item (d of them at most)
 
@@ -59,13 +66,13 @@ struct DevSketch {
   int item;            // owning item
   // ---- basis sketches: TSQR tree (level 0 is the sketch itself)
   int nlev;            // number of levels; level nlev-1 is the root (one block)
-  int bl;              // rows per block at every level
   int rpad;            // padded rank (columns of the basis)
   int rank_slot;       // index into the rank array of this sketch's rank r_k
   int target_rank;     // fixed-rank mode target (already clamped)
   int rcap;            // min(N_k, M_k)
   int64_t lev_rows[kMaxLev];
   int64_t lev_nblk[kMaxLev];
+  int lev_bl[kMaxLev];        // rows per block
   int64_t lev_mat[kMaxLev];   // level matrix (rows x width) offset; lev_mat[0] = off
   int64_t lev_beta[kMaxLev];  // nblk * width Householder scalars
   int64_t lev_z[kMaxLev];     // rows x rpad expansion buffer; lev_z[0] = the basis Q_k / P_k
