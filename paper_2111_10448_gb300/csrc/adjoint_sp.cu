@@ -50,7 +50,7 @@ struct AdjSk {
 struct AdjArgs {
   char* wsb;
   float* dX;
-  uint64_t seed;
+  PhiloxKeys keys;
   int64_t n1, nd, W, Nd1, WL;
   int nsk;
   AdjSk sk[kMaxSk];
@@ -114,7 +114,7 @@ __global__ void split_kernel(char* wsb, int item, int lpad) {
 // elements of a row-major rows x lpad source (the split adjoint, a staged
 // table or the warp's generated rows).
 template <int LPAD, bool TF>
-__global__ void __launch_bounds__(kThreads, 2) adjoint_kernel(const AdjArgs ga) {
+__global__ void __launch_bounds__(kThreads, 2) adjoint_kernel(const __grid_constant__ AdjArgs ga) {
   using E = typename std::conditional<TF, float, __nv_bfloat16>::type;
   constexpr int KS = TF ? 8 : 16;  // k per MMA
   __shared__ AdjArgs g;
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kThreads, 2) adjoint_kernel(const AdjArgs ga) 
           const int r = c / nq, q = c - r * nq;
           const uint64_t row = s.col ? (uint64_t)(whi + s.hstride * r) : (uint64_t)(r + g.n1 * wlo);
           float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (4 * q < s.ell) z = normals4_f32(g.seed, (uint32_t)s.sid, row, (uint32_t)q);
+          if (4 * q < s.ell) z = normals4_f32(ga.keys, (uint32_t)s.sid, row, (uint32_t)q);
           const float zz[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
@@ -275,7 +275,7 @@ cudaError_t launch_adjoint_sp(const Plan& P, int item, void* dX, void* ws, cudaS
   memset(&g, 0, sizeof(g));
   g.wsb = (char*)ws;
   g.dX = (float*)dX;
-  g.seed = it.seed;
+  g.keys = philox_keys(it.seed);
   g.n1 = it.n[0];
   g.nd = it.n[it.d - 1];
   g.W = it.W;

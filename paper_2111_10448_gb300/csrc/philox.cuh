@@ -42,6 +42,37 @@ __device__ __forceinline__ void philox4x32_10(uint32_t& c0, uint32_t& c1, uint32
   }
 }
 
+// The ten rounds' keys, made on the host.  A kernel that has them among its launch
+// arguments takes each from the constant bank as an operand of the round's xor; the
+// additions above are 20 instructions a quad that the compiler leaves in the loop
+// (91 against 117 issue slots measured).
+struct PhiloxKeys {
+  uint32_t k[20];
+};
+__host__ __device__ inline PhiloxKeys philox_keys(uint64_t seed) {
+  PhiloxKeys p;
+  uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+  for (int r = 0; r < 10; ++r) {
+    p.k[2 * r] = k0;
+    p.k[2 * r + 1] = k1;
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+  }
+  return p;
+}
+__device__ __forceinline__ void philox4x32_10(uint32_t& c0, uint32_t& c1, uint32_t& c2, uint32_t& c3,
+                                              const PhiloxKeys& p) {
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)c0 * 0xD2511F53u;
+    const uint64_t p1 = (uint64_t)c2 * 0xCD9E8D57u;
+    c0 = (uint32_t)(p1 >> 32) ^ c1 ^ p.k[2 * r];
+    c1 = (uint32_t)p1;
+    c2 = (uint32_t)(p0 >> 32) ^ c3 ^ p.k[2 * r + 1];
+    c3 = (uint32_t)p0;
+  }
+}
+
 // Four consecutive FP64 normals z[4q..4q+3] of row `row` of stream `sid`.
 __device__ __forceinline__ void normals4_f64(uint64_t seed, uint32_t sid, uint64_t row, uint32_t q,
                                              double z[4]) {
@@ -68,17 +99,30 @@ __device__ __forceinline__ void normals4_f64(uint64_t seed, uint32_t sid, uint64
 // in every kernel that regenerates these entries (the sketch, the staged
 // test-matrix tables, the middle-core matrix B, the backward), computes the
 // same bits.
-__device__ __forceinline__ float4 normals4_f32(uint64_t seed, uint32_t sid, uint64_t row, uint32_t q) {
-  uint32_t c0 = (uint32_t)row, c1 = (uint32_t)(row >> 32), c2 = q, c3 = sid;
-  philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
+//
+// What bounds it: issue slots.  A quad took 247 (117 Philox, the rest two logarithms,
+// roots and sine/cosine pairs with their conversions) and takes 225 with the
+// branch-free root below, 189 with the keys from the constant bank as well: 0.52 ->
+// 0.68 quads per cycle and SM.
+
+// sqrt(x) rounded to nearest for x = -2 ln u, u of the 32-bit words: x = 0 or 2^-24 <=
+// x < 46.  Markstein's correction of an approximate reciprocal root (IBM J. Res. Dev.
+// 34, 1990): s = x y, s + (x - s^2) (y / 2).  No branch, so that independent chains
+// interleave; compared with the correctly rounded root over all 2^32 words: equal.
+__device__ __forceinline__ float rho_root(float x) {
+  const float y = rsqrtf(fmaxf(x, 0x1p-60f));
+  const float s = __fmul_rn(x, y);
+  return __fmaf_rn(__fmaf_rn(-s, s, x), __fmul_rn(0.5f, y), s);
+}
+__device__ __forceinline__ float4 box_muller4(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
   // u = (x + 1/2) 2^-32 in FP32: x is rounded to 24 bits (relative error
   // 2^-24 at any magnitude), then scaled exactly and offset by 2^-33.
   const float u0 = __fmaf_rn(__uint2float_rn(c0), 0x1p-32f, 0x1p-33f);
   const float u1 = __fmaf_rn(__uint2float_rn(c1), 0x1p-32f, 0x1p-33f);
   const float u2 = __fmaf_rn(__uint2float_rn(c2), 0x1p-32f, 0x1p-33f);
   const float u3 = __fmaf_rn(__uint2float_rn(c3), 0x1p-32f, 0x1p-33f);
-  const float ra = __fsqrt_rn(__fmul_rn(-2.0f, logf(u0)));
-  const float rb = __fsqrt_rn(__fmul_rn(-2.0f, logf(u2)));
+  const float ra = rho_root(__fmul_rn(-2.0f, logf(u0)));
+  const float rb = rho_root(__fmul_rn(-2.0f, logf(u2)));
   // centred angles 2 pi u - pi in (-pi, pi]: cos(2 pi u) = -cos(.), sin likewise
   const float ta = __fmaf_rn(u1, 6.28318530717958647692f, -3.14159265358979323846f);
   const float tb = __fmaf_rn(u3, 6.28318530717958647692f, -3.14159265358979323846f);
@@ -86,6 +130,16 @@ __device__ __forceinline__ float4 normals4_f32(uint64_t seed, uint32_t sid, uint
   __sincosf(ta, &sa, &ca);
   __sincosf(tb, &sb, &cb);
   return make_float4(-__fmul_rn(ra, ca), -__fmul_rn(ra, sa), -__fmul_rn(rb, cb), -__fmul_rn(rb, sb));
+}
+__device__ __forceinline__ float4 normals4_f32(uint64_t seed, uint32_t sid, uint64_t row, uint32_t q) {
+  uint32_t c0 = (uint32_t)row, c1 = (uint32_t)(row >> 32), c2 = q, c3 = sid;
+  philox4x32_10(c0, c1, c2, c3, (uint32_t)seed, (uint32_t)(seed >> 32));
+  return box_muller4(c0, c1, c2, c3);
+}
+__device__ __forceinline__ float4 normals4_f32(const PhiloxKeys& keys, uint32_t sid, uint64_t row, uint32_t q) {
+  uint32_t c0 = (uint32_t)row, c1 = (uint32_t)(row >> 32), c2 = q, c3 = sid;
+  philox4x32_10(c0, c1, c2, c3, keys);
+  return box_muller4(c0, c1, c2, c3);
 }
 
 // Round an FP32 value to the MMA input type, nearest-even, returned as FP32.

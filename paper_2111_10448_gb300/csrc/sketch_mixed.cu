@@ -516,7 +516,7 @@ struct TcArgs {
   double* ws;
   int* status;
   int64_t n1, first, W, WL, WR, Nd1, tilesL, tilesR;
-  uint64_t seed;
+  PhiloxKeys keys;
   int H1, H4, T2, T3, ell, nL, nR, NL, NR, tmem_cols;
   int64_t runL;  // tiles of one kL block accumulated in the L slots before a flush
   int genL[4], genR[4], ngenL, ngenR;  // sketches whose blocks the RNG warps generate
@@ -583,7 +583,7 @@ __device__ __forceinline__ int64_t row_key(const TcArgs& g, const SkTc& sk, int6
 }
 
 template <int ELL, bool F16>
-__global__ void __launch_bounds__(kThreads, 1) sketch_tc_kernel(const TcArgs g) {
+__global__ void __launch_bounds__(kThreads, 1) sketch_tc_kernel(const __grid_constant__ TcArgs g) {
   extern __shared__ __align__(1024) unsigned char smraw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kOffBar);
@@ -813,8 +813,8 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_tc_kernel(const TcArgs g) 
             for (int u = u_beg; u < u_end; ++u) {
               const int k = 2 * rp;  // row of the block (i_d or i_1 offset)
               const int64_t row = bs.row0 + bs.rstep * k;
-              const float4 ra = tm_quad_f32(g.ws, bs.kr, g.seed, bs.sid, (uint64_t)row, (uint32_t)nq);
-              const float4 rb = tm_quad_f32(g.ws, bs.kr, g.seed, bs.sid, (uint64_t)(row + bs.rstep), (uint32_t)nq);
+              const float4 ra = tm_quad_f32(g.ws, bs.kr, g.keys, bs.sid, (uint64_t)row, (uint32_t)nq);
+              const float4 rb = tm_quad_f32(g.ws, bs.kr, g.keys, bs.sid, (uint64_t)(row + bs.rstep), (uint32_t)nq);
               const int n0 = bs.n0 + 4 * nq;  // a multiple of 4: one core matrix holds n0 .. n0 + 3
               const uint32_t dst = bs.dst0 + (k >> 3) * kS1 + (n0 >> 3) * kS4 + (n0 & 7) * 16 + (k & 7) * 2;
               st_shared_b32(dst, op16x2_bits<F16>(ra.x, rb.x));
@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(kThreads, 1) sketch_tc_kernel(const TcArgs g) 
 // 128 rows v + hstride (first + 128 h + k) (column side) or 128 h + k + n1 v
 // (row side), k = 0..127, as the K-major core-matrix image the MMA reads (BF16
 // or FP16: the same layout and rounding the RNG warps produce).
-__global__ void tc_table_kernel(const TcArgs g, int colside, int s, int64_t nv, int H) {
+__global__ void tc_table_kernel(const __grid_constant__ TcArgs g, int colside, int s, int64_t nv, int H) {
   const SkTc sk = colside ? g.col[s] : g.row[s];
   const int qps = g.ell / 4;
   const int64_t blkB = (int64_t)(g.ell / 8) * kS4;
@@ -1070,7 +1070,7 @@ __global__ void tc_table_kernel(const TcArgs g, int colside, int s, int64_t nv, 
     const int64_t v = rest / H;
     const int64_t k = 128 * h + 8 * kg + r8;
     const uint64_t row = colside ? (uint64_t)(v + sk.hstride * (g.first + k)) : (uint64_t)(k + g.n1 * v);
-    const float4 z = tm_quad_f32(g.ws, kr_of(g.ws, sk.kr), g.seed, (uint32_t)sk.sid, row, (uint32_t)q);
+    const float4 z = tm_quad_f32(g.ws, kr_of(g.ws, sk.kr), g.keys, (uint32_t)sk.sid, row, (uint32_t)q);
     const float zz[4] = {z.x, z.y, z.z, z.w};
     char* blk = tab + (v * H + h) * blkB;
 #pragma unroll
@@ -1175,7 +1175,7 @@ bool plan_tc(const Plan& P, int item, int64_t count, TcArgs* out) {
   }
   g.NL = NL;
   g.NR = NR;
-  g.seed = it.seed;
+  g.keys = philox_keys(it.seed);
   g.f16 = it.prec == TT_PREC_FP16 ? 1 : 0;
   g.xscale = g.f16 ? it.xscale : 1.0f;
   *out = g;

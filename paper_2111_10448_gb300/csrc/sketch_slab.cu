@@ -106,7 +106,7 @@ struct SlabArgs {
   int64_t n1, first, W, WL, WR, Nd1;
   int64_t WRg;             // kR groups: WR / G
   int64_t tilesL, tilesR;  // tiles of T2 kL values x T3 kR groups
-  uint64_t seed;
+  PhiloxKeys keys;
   int H1, T2, T3, ell, c, lc, G;
   int colL, colR;          // tensor-memory columns of the L slots and of the R_2 buffers
   int kry;                 // Khatri-Rao test matrices: R_3 mode by mode (fixed mode-1 block)
@@ -167,7 +167,7 @@ __device__ __forceinline__ bool next_super_plane(const SlabArgs& g, int64_t ntil
 }
 
 template <int ELL, int C, bool KRY, bool F16>
-__global__ void __launch_bounds__(Roles<KRY>::threads, 1) sketch_slab_kernel(const SlabArgs g) {
+__global__ void __launch_bounds__(Roles<KRY>::threads, 1) sketch_slab_kernel(const __grid_constant__ SlabArgs g) {
   constexpr int kRngWarps = Roles<KRY>::rng;
   constexpr int kThreads = Roles<KRY>::threads;
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -490,8 +490,8 @@ __global__ void __launch_bounds__(Roles<KRY>::threads, 1) sketch_slab_kernel(con
             } else {
               const int64_t key = bi == 0 ? w0 + g.WL * gg : kR0 + gg;  // w / wdiv for wdiv = 1, n2
               const int64_t row = key + sk.hstride * (g.first + kk);
-              ra = normals4_f32(g.seed, (uint32_t)sk.sid, (uint64_t)row, (uint32_t)nq);
-              rb = normals4_f32(g.seed, (uint32_t)sk.sid, (uint64_t)(row + sk.hstride), (uint32_t)nq);
+              ra = normals4_f32(g.keys, (uint32_t)sk.sid, (uint64_t)row, (uint32_t)nq);
+              rb = normals4_f32(g.keys, (uint32_t)sk.sid, (uint64_t)(row + sk.hstride), (uint32_t)nq);
             }
             const int n0 = bi * ell + 4 * nq;
             const uint32_t dst = sL + buf * kLBlkB + (k >> 3) * kS1 + (n0 >> 3) * kS4 + (n0 & 7) * 16 + (k & 7) * 2;
@@ -547,8 +547,8 @@ __global__ void __launch_bounds__(Roles<KRY>::threads, 1) sketch_slab_kernel(con
                 kk2[h] = 2 * rp;
                 nn2[h] = gp * ell + 4 * nq;
                 const int64_t row = h1 * 128 + kk2[h] + g.n1 * (w0 + g.WL * gp);
-                z[h][0] = normals4_f32(g.seed, (uint32_t)sk.sid, (uint64_t)row, (uint32_t)nq);
-                z[h][1] = normals4_f32(g.seed, (uint32_t)sk.sid, (uint64_t)(row + 1), (uint32_t)nq);
+                z[h][0] = normals4_f32(g.keys, (uint32_t)sk.sid, (uint64_t)row, (uint32_t)nq);
+                z[h][1] = normals4_f32(g.keys, (uint32_t)sk.sid, (uint64_t)(row + 1), (uint32_t)nq);
               }
 #pragma unroll
               for (int h = 0; h < 2; ++h) {
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(Roles<KRY>::threads, 1) sketch_slab_kernel(con
 // Staged R_3 blocks (dense test matrices): block (h, kL, kR) holds the 128
 // rows 128 h + k + n_1 (kL + WL kR) of Psi_3 as the K-major core-matrix
 // image the MMA reads (BF16 or FP16), kR fastest.
-__global__ void slab_ytab_kernel(const SlabArgs g) {
+__global__ void slab_ytab_kernel(const __grid_constant__ SlabArgs g) {
   const SkTc sk = g.row[1];
   const int qps = g.ell / 4;
   const int64_t blkB = (int64_t)(g.ell / 8) * kS4;
@@ -988,7 +988,7 @@ __global__ void slab_ytab_kernel(const SlabArgs g) {
     const int64_t kR = blk % g.WR, hl = blk / g.WR;
     const int64_t kL = hl % g.WL, h = hl / g.WL;
     const int64_t k = 128 * h + 8 * kg + r8;
-    const float4 z = normals4_f32(g.seed, (uint32_t)sk.sid, (uint64_t)(k + g.n1 * (kL + g.WL * kR)), (uint32_t)q);
+    const float4 z = normals4_f32(g.keys, (uint32_t)sk.sid, (uint64_t)(k + g.n1 * (kL + g.WL * kR)), (uint32_t)q);
     const float zz[4] = {z.x, z.y, z.z, z.w};
     char* bp = tab + blk * blkB;
 #pragma unroll
@@ -1024,7 +1024,7 @@ __global__ void s2_fold_kernel(double* __restrict__ s2, float* __restrict__ stag
 // Staged R_2 blocks: block (v, h) holds the 128 rows 128 h + k + n_1 v of the
 // test matrix (v = kL) as the K-major core-matrix image the MMA reads (BF16
 // or FP16).
-__global__ void slab_table_kernel(const SlabArgs g, int64_t nv) {
+__global__ void slab_table_kernel(const __grid_constant__ SlabArgs g, int64_t nv) {
   const SkTc sk = g.row[0];
   const int qps = g.ell / 4;
   const int64_t blkB = (int64_t)(g.ell / 8) * kS4;
@@ -1041,7 +1041,7 @@ __global__ void slab_table_kernel(const SlabArgs g, int64_t nv) {
     const int h = (int)(rest % g.H1);
     const int64_t v = rest / g.H1;
     const int64_t k = 128 * h + 8 * kg + r8;
-    const float4 z = tm_quad_f32(g.ws, kr, g.seed, (uint32_t)sk.sid, (uint64_t)(k + g.n1 * v), (uint32_t)q);
+    const float4 z = tm_quad_f32(g.ws, kr, g.keys, (uint32_t)sk.sid, (uint64_t)(k + g.n1 * v), (uint32_t)q);
     const float zz[4] = {z.x, z.y, z.z, z.w};
     char* blk = tab + (v * g.H1 + h) * blkB;
 #pragma unroll
@@ -1143,7 +1143,7 @@ bool plan_slab(const Plan& P, int item, int64_t count, slab::SlabArgs* out) {
   if (it.tctab_doubles * 8 < g.WL * g.H1 * blk) return false;
   g.row[0].tab = it.off_tctab * 8;
   g.tab_tx = (uint32_t)(g.H1 * blk);
-  g.seed = it.seed;
+  g.keys = philox_keys(it.seed);
   g.f16 = it.prec == TT_PREC_FP16 ? 1 : 0;
   g.xscale = g.f16 ? it.xscale : 1.0f;
   *out = g;

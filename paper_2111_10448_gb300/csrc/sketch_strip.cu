@@ -82,6 +82,7 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
     k.width = d.width;
     k.nq = (d.width + 3) / 4;
     k.inv_nq = 1.0f / (float)k.nq;
+    k.rpi = kThreads / k.nq;
     k.sid = d.stream_id;
     k.kr = d.kr_nm ? it.sk0 + s : -1;
     k.mbm = d.kr_nm && d.kr_mbm ? 1 : 0;
@@ -119,6 +120,7 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
   g.cnt = count;
   g.Nd1 = it.N[it.d - 1];
   g.seed = it.seed;
+  g.keys = philox_keys(it.seed);
   g.xscale = fmt == kFmtFP16 ? it.xscale : 1.0f;
   g.WL = (uint32_t)WL;
   g.WR = (uint32_t)WR;

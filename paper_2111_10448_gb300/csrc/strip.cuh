@@ -41,6 +41,7 @@ struct StSk {
   int kind;
   int64_t mulr;         // column sketch: WL / wdiv
   float inv_nq;         // 1 / nq
+  int rpi;              // rows a pass of the block generates: kThreads / nq
 };
 
 struct StripArgs {
@@ -49,6 +50,7 @@ struct StripArgs {
   int item;                   // index in its plan (batched launches)
   int64_t n1, cnt, first, Nd1;
   uint64_t seed;
+  PhiloxKeys keys;            // of the seed
   uint32_t WL, WR, q2, q3;    // kL = i_2 + q2 i_3 (q2 q3 = WL)
   int ncol, nrow, vec;
   uint32_t tabs;              // bit s (columns), kMaxCol + r (rows): the sketch has a table
@@ -267,8 +269,12 @@ __device__ __forceinline__ void convert_x(const StripArgs& a, const TileDesc& d,
 // staged block.
 template <int FMT>
 __device__ __forceinline__ void put_quad(char* gs, int ldg, int r, int q, float4 z, int width) {
-  const float z0 = 4 * q < width ? z.x : 0.f, z1 = 4 * q + 1 < width ? z.y : 0.f;
-  const float z2 = 4 * q + 2 < width ? z.z : 0.f, z3 = 4 * q + 3 < width ? z.w : 0.f;
+  float z0 = z.x, z1 = z.y, z2 = z.z, z3 = z.w;
+  if (width & 3) {   // uniform: a last quad that is not full
+    z1 = 4 * q + 1 < width ? z1 : 0.f;
+    z2 = 4 * q + 2 < width ? z2 : 0.f;
+    z3 = 4 * q + 3 < width ? z3 : 0.f;
+  }
   if constexpr (FMT == kFmtTF32)
     *reinterpret_cast<float4*>(gs + r * ldg + 16 * q) = make_float4(round_tf32(z0), round_tf32(z1), round_tf32(z2), round_tf32(z3));
   else
@@ -301,8 +307,10 @@ __device__ __noinline__ void stage_g_kr(const char* wsb, const DevSketch* krs, i
   }
 }
 
-// Generated test-matrix rows.
-template <int FMT, int NT>
+// Generated test-matrix rows.  A thread keeps its quad q and goes through the rows in
+// steps of kThreads / nq: no division a quad (KEYS: the Philox keys are launch arguments
+// in the constant bank; a batched launch's lie in shared memory and are not used).
+template <int FMT, int NT, bool KEYS>
 __device__ __forceinline__ void make_g(const StripArgs& a, const StSk& s, char* gs, const Rows& w, int64_t grow,
                                        int64_t f0) {
   constexpr int LDG = ldg_bytes(FMT, NT);
@@ -310,15 +318,18 @@ __device__ __forceinline__ void make_g(const StripArgs& a, const StSk& s, char* 
     stage_g_kr<FMT, NT>(a.wsb, ws_sketches(a.wsb) + s.kr, s.mbm, gs, w, grow, f0, s.width);
     return;
   }
-  const int rows = w.no * w.ni, jobs = w.nblk * rows * s.nq;
+  const int rows = w.no * w.ni;
   const float inv_rows = __frcp_rn((float)rows);
-  for (int o = threadIdx.x; o < jobs; o += kThreads) {
-    int e = fdiv(o, s.inv_nq);
-    const int q = o - e * s.nq;
-    int p = 0, oo = 0;
+  const int r0 = fdiv((int)threadIdx.x, s.inv_nq), q = (int)threadIdx.x - r0 * s.nq;
+  if (r0 >= s.rpi) return;
+  for (int r = r0; r < w.nblk * rows; r += s.rpi) {
+    int e = r, p = 0, oo = 0;
     if (w.nblk > 1) p = fdiv(e, inv_rows), e -= p * rows;
     if (w.no > 1) oo = fdiv(e, w.inv_ni), e -= oo * w.ni;
-    const float4 z = normals4_f32(a.seed, (uint32_t)s.sid, (uint64_t)(grow + w.gp * p + w.go * oo + w.gi * e), (uint32_t)q);
+    const uint64_t row = (uint64_t)(grow + w.gp * p + w.go * oo + w.gi * e);
+    float4 z;
+    if constexpr (KEYS) z = normals4_f32(a.keys, (uint32_t)s.sid, row, (uint32_t)q);
+    else z = normals4_f32(a.seed, (uint32_t)s.sid, row, (uint32_t)q);
     put_quad<FMT>(gs, LDG, p * w.bstep + oo * w.pad + e, q, z, s.width);
   }
 }
@@ -381,7 +392,7 @@ __device__ __forceinline__ void step(float (*t)[4], const uint32_t* xh, const ui
 }
 
 // One unit of work: strip ab of i_1, a set of column tiles, a range of positions.
-template <int FMT, int NT, int NCOL>
+template <int FMT, int NT, int NCOL, bool KEYS>
 __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, char* sm, TileDesc* td, UnitState& us, uint64_t* bar,
                                            volatile int* abort_flag) {
   constexpr int E = esz(FMT), KSTEP = FMT == kFmtTF32 ? 8 : 16, KS = 32 / KSTEP, LDG = ldg_bytes(FMT, NT);
@@ -627,15 +638,15 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
       if (fresh & ~a.tabs & (1u << s)) {
         const StSk& sk = a.col[s];
         const int64_t dq = sk.mulr * a.sR;
-        make_g<FMT, NT>(a, sk, sm + sk.soff, Rows{sk.per ? d.nl : 1, a.TB, d.nr, d.tb, a.ndp, 1, dq, sk.hstride,
-                                                          d.inv_tb},
+        make_g<FMT, NT, KEYS>(a, sk, sm + sk.soff,
+                              Rows{sk.per ? d.nl : 1, a.TB, d.nr, d.tb, a.ndp, 1, dq, sk.hstride, d.inv_tb},
                         d.grow[s], 0);
       }
 #pragma unroll
     for (int r = 0; r < kMaxRow; ++r)
       if (fresh & ~a.tabs & (1u << (kMaxCol + r))) {
         const StSk& sk = a.row[r];
-        make_g<FMT, NT>(a, sk, sm + sk.soff,
+        make_g<FMT, NT, KEYS>(a, sk, sm + sk.soff,
                         Rows{sk.per ? d.nr : 1, a.TA, d.nl, d.ta, a.n1p, (int64_t)a.WL * a.sR * a.n1, a.n1, 1,
                              d.inv_ta},
                         d.grow[kMaxCol + r], a0);
@@ -758,7 +769,7 @@ __global__ void __launch_bounds__(kThreads, NCOL * NT <= 12 ? 2 : 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  strip_unit<FMT, NT, NCOL>(a, blockIdx.x, sm, td, us, &bar, &abort_flag);
+  strip_unit<FMT, NT, NCOL, true>(a, blockIdx.x, sm, td, us, &bar, &abort_flag);
 }
 
 // Batched form: one launch over the units of every tensor of a plan, largest
@@ -800,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, 2) sketch_strip_batched_kernel(const
     a.vec = a.vec && ((uintptr_t)a.X & 15) == 0;
   }
   __syncthreads();
-  strip_unit<FMT, NT, kMaxCol>(a, blockIdx.x - prefix[lo], sm, td, us, &bar, &abort_flag);
+  strip_unit<FMT, NT, kMaxCol, false>(a, blockIdx.x - prefix[lo], sm, td, us, &bar, &abort_flag);
 }
 
 using KernelFn = void (*)(const StripArgs);

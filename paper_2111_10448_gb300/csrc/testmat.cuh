@@ -121,7 +121,9 @@ __device__ __forceinline__ float4 kr_scale_quad(const void* wsb, const DevSketch
 
 // The quad a kernel uses: kr = the sketch's device record when its test
 // matrix is Khatri-Rao, nullptr for the dense stream.
-__device__ __forceinline__ float4 tm_quad_f32(const void* wsb, const DevSketch* kr, uint64_t seed, uint32_t sid,
+// seed: the seed or its Philox keys.
+template <typename Seed>
+__device__ __forceinline__ float4 tm_quad_f32(const void* wsb, const DevSketch* kr, const Seed& seed, uint32_t sid,
                                               uint64_t row, uint32_t q) {
   if (kr) return kr_quad_f32(wsb, *kr, row, q);
   return normals4_f32(seed, sid, row, q);
