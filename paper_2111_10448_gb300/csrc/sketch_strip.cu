@@ -213,7 +213,7 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
   // m-tile of the strip starts with its column products
   int load[kWarps], cnt[kWarps];
   for (int w = 0; w < kWarps; ++w) {
-    load[w] = w < mtA ? g.ncol * g.TB : 0;
+    load[w] = (w < mtA ? g.ncol * g.TB : 0) + (w == kDescWarp ? kDescLoad : 0);
     cnt[w] = 0;
     memset(g.task[w], 255, kWarpTasks);
   }

@@ -18,6 +18,8 @@ namespace strip {
 constexpr int kThreads = 256, kWarps = 8;
 constexpr int kMaxCol = 3, kMaxRow = 3;   // sketches a side
 constexpr int kMaxTA = 128;               // rows of i_1 per strip: one 16-row m-tile per warp
+constexpr int kDescWarp = kWarps - 1;     // describes the tiles, two ahead: the warp with the fewest column rows
+constexpr int kDescLoad = 96;             // what that costs, in row-product columns (planning)
 constexpr int kWarpTasks = 4;             // row products (m-tile, sketch) of one warp and tile, at most
 constexpr int kAddsMax = 32;              // FP32 additions into one accumulator between FP64 flushes
 constexpr int kRowAddsMax = 16;           // the same for the row sketches' shared sums (4 chunks each)
@@ -149,7 +151,7 @@ struct TileDesc {
 // the 16-byte boundary below, so entry i of a row lies at word (start word mod 4) +
 // i; no copy leaves the slab.  (One bulk copy per row, 256 to 512 bytes each, was
 // slower: 960^3 5.2 ms against 3.4.)
-// Per CTA and unit: the cursor over the tiles (warp 0's) and every warp's row products.
+// Per CTA and unit: the cursor over the tiles (kDescWarp's) and every warp's row products.
 struct UnitState {
   uint32_t i2, i3, rg, rlo;
   int bb, gi, adds[kMaxCol];
@@ -574,7 +576,7 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
     const uint32_t on = __ballot_sync((1u << kWarpTasks) - 1u, tk != 255);
     if (lane == 0) us.ntask[warp] = __popc(on);
   }
-  if (warp == 0) {
+  if (warp == kDescWarp) {
     if (lane == 0) {
       us.i2 = u0 / a.q3;
       us.i3 = u0 - us.i2 * a.q3;
@@ -583,6 +585,11 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
     }
     __syncwarp();
     describe(td[0], nullptr);
+    if (ntile > 1) {
+      if (lane == 0) advance();
+      __syncwarp();
+      describe(td[1], &td[0]);
+    }
   }
   __syncthreads();
   issue_x(a, td[0], raw, mi);
@@ -590,8 +597,10 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
   int row_adds = 0;
   uint32_t gphase = 0;
   const uint32_t xhs = s_u32(xh), xls = s_u32(xl);
+  int cur = 0;
   for (uint32_t t = 0; t < ntile; ++t) {
-    const TileDesc& d = td[t & 1];
+    const TileDesc& d = td[cur];
+    const int nxt = cur == 2 ? 0 : cur + 1;
     const int tbk = a.PR > 1 ? a.TB : (d.tb + 15) & ~15;
     cp_wait<0>();
     __syncthreads();          // the raw tile is there; products of the tile before are done
@@ -658,19 +667,20 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
           reinterpret_cast<float4*>(scale)[tid] = c;
         }
       }
-    if (warp == 0 && t + 1 < ntile) {
-      if (lane == 0) advance();
-      __syncwarp();
-      describe(td[(t + 1) & 1], &d);
-    }
     if (copies) {
       if (!*abort_flag) tc::mbar_wait(bar_g, gphase, abort_flag, status);   // bounded
       gphase ^= 1;
     }
     __syncthreads();
     if (t + 1 < ntile) {      // the next tile travels while this one is multiplied
-      issue_x(a, td[(t + 1) & 1], raw, mi);
+      issue_x(a, td[nxt], raw, mi);
       cp_commit();
+    }
+    // the tile after that, in the slot of the one before this
+    if (warp == kDescWarp && t + 2 < ntile) {
+      if (lane == 0) advance();
+      __syncwarp();
+      describe(td[nxt == 2 ? 0 : nxt + 1], &td[nxt]);
     }
     // ---- column products of this warp's m-tile
     if (16 * warp < tak) {
@@ -747,10 +757,11 @@ __device__ __forceinline__ void strip_unit(const StripArgs& a, uint32_t unit, ch
       __syncthreads();
       flush_rows();
     }
+    if (t + 1 < ntile) cur = nxt;
   }
 #pragma unroll
   for (int s = 0; s < NCOL; ++s)
-    if (s < a.ncol) flush_col(s, td[(ntile - 1) & 1].wlo[s]);
+    if (s < a.ncol) flush_col(s, td[cur].wlo[s]);
   __syncthreads();
   if (row_adds) flush_rows();
 }
@@ -759,7 +770,7 @@ template <int FMT, int NT, int NCOL>
 __global__ void __launch_bounds__(kThreads, NCOL * NT <= 12 ? 2 : 1)
     sketch_strip_kernel(const __grid_constant__ StripArgs a) {
   extern __shared__ __align__(16) char sm[];
-  __shared__ TileDesc td[2];
+  __shared__ TileDesc td[3];
   __shared__ UnitState us;
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
@@ -785,7 +796,7 @@ struct StripBatch {
 template <int FMT, int NT>
 __global__ void __launch_bounds__(kThreads, 2) sketch_strip_batched_kernel(const __grid_constant__ StripBatch b) {
   extern __shared__ __align__(16) char sm[];
-  __shared__ TileDesc td[2];
+  __shared__ TileDesc td[3];
   __shared__ UnitState us;
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
