@@ -464,10 +464,14 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   // find no room are drawn per tile.  Reading a staged row costs less than drawing it
   // even when it comes from HBM (a 64-byte row 3 cycles of an SM's share of the
   // bandwidth, its seven column quads 13 cycles at 0.52 quads a cycle).
+  // The FP64 kernel's rows (width doubles each; a quad of its normals costs some 90 FMAs
+  // of the units that bound it) take the same room; its launch says which it fills.
   {
-    const bool ok = (op16 || q.prec == TT_PREC_TF32) && q.x_dtype == TT_F32 && it.tctab_doubles == 0 &&
-                    (single || it.sptab_doubles > 0);
-    const int64_t tilesA = (q.n[0] + 127) / 128, tilesB = (q.n[d - 1] + 63) / 64;
+    const bool f64 = q.prec == TT_PREC_FP64 && single;
+    const bool ok = f64 || ((op16 || q.prec == TT_PREC_TF32) && q.x_dtype == TT_F32 && it.tctab_doubles == 0 &&
+                            (single || it.sptab_doubles > 0));
+    const int64_t tilesA = (q.n[0] + (f64 ? 63 : 127)) / (f64 ? 64 : 128);
+    const int64_t tilesB = (q.n[d - 1] + (f64 ? 31 : 63)) / (f64 ? 32 : 64);
     int lmax = 1;
     for (int si = it.sk0; si < it.sk0 + it.nsk; ++si) lmax = std::max(lmax, P.sketches[si].width);
     // (a batched launch uses the row format of its widest tensor, at most 32 columns)
@@ -478,8 +482,9 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
       s.st_tab = -1;
       // a mode-by-mode Khatri-Rao sketch reads one factor row per tile row: nothing to stage
       if (!ok || s.kr_mbm) continue;
-      if (s.type == SK_COL && s.wdiv * tilesA >= 2) want.emplace_back((it.W / s.wdiv) * q.n[d - 1] * row, si);
-      if (s.type == SK_ROW && (it.W / s.wdiv) * tilesB >= 2) want.emplace_back(s.wdiv * q.n[0] * row, si);
+      const int64_t rb = f64 ? 8LL * s.width : row;
+      if (s.type == SK_COL && s.wdiv * tilesA >= 2) want.emplace_back((it.W / s.wdiv) * q.n[d - 1] * rb, si);
+      if (s.type == SK_ROW && (it.W / s.wdiv) * tilesB >= 2) want.emplace_back(s.wdiv * q.n[0] * rb, si);
     }
     std::sort(want.begin(), want.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
     // (start, end) of the free regions, bytes

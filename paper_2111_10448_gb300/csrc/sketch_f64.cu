@@ -7,8 +7,14 @@
 //   column sketch: S_k[a + n_1 wlo, j] += sum_b X(a, w, b) Omega_k[whi + hs b, j]
 //   row sketch:    R_k[whi + hs b, j]  += sum_a X(a, w, b) Psi_k[a + n_1 wlo, j]
 // with the test-matrix tile regenerated from Philox into shared memory.  The
-// per-tile partial sums are added to the FP64 sketches with atomics.  On
-// GB300 FP64 arithmetic is the bound of this kernel (not HBM).
+// per-tile partial sums are added to the FP64 sketches with atomics.
+//
+// What bounds it: the FP64 units (1.7 FMAs per cycle and SM measured), by the products
+// and as much again by drawing the test-matrix rows, whose logarithms, roots and sines
+// are FP64 too: a quad of normals costs as much as some 90 FMAs.  So rows that
+// many tiles share are drawn once per accumulate into the backward's scratch (st_tab)
+// and read from there, and planes wide enough take 64 x 64 tiles, which halves what is
+// left on the row side.  @MEASURED@
 #include <algorithm>
 
 #include "internal.cuh"
@@ -23,11 +29,13 @@ constexpr int64_t kTableOffB = 256;
 constexpr int kTA = 64;   // rows (i_1) per tile of the single-tensor launch
 constexpr int kTB = 32;   // columns (i_d) per tile
 constexpr int kThreads = 256;
+constexpr int64_t kTableQuads = 1 << 17;   // quads of normals that pay for staging them (some 4 us of a launch)
 
 struct SkArg {
   int64_t rows, off, wdiv, hstride;
   int type, width, sid;
   int kr;  // global sketch index when the test matrix is Khatri-Rao, -1: dense
+  const double* tab;  // its staged rows (width doubles each), nullptr: drawn per tile
 };
 
 struct F64Args {
@@ -78,7 +86,15 @@ __device__ void f64_tile(const F64Args& a, int64_t item, double* smem) {
     const int nr = sk.type == SK_COL ? tb : ta;
     const int nq = (l + 3) / 4;
     __syncthreads();
-    for (int o = tid; o < nr * nq; o += kThreads) {
+    if (sk.tab) {
+      // rows (whi, b0 ...) of a column sketch, (wlo, a0 ...) of a row sketch: consecutive
+      const double* src = sk.tab + (sk.type == SK_COL ? whi * a.cnt + b0 : wlo * a.n1 + a0) * l;
+      for (int o = tid; o < nr * l; o += kThreads) {
+        const int r = o / l;
+        Gs[r * LDG + (o - r * l)] = src[o];
+      }
+    }
+    for (int o = tid; o < (sk.tab ? 0 : nr * nq); o += kThreads) {
       const int r = o % nr, q = o / nr;
       const uint64_t grow = sk.type == SK_COL
                                 ? (uint64_t)(whi + sk.hstride * (a.first + b0 + r))
@@ -116,10 +132,29 @@ __host__ __device__ constexpr size_t f64_smem(int lmax) {
   return sizeof(double) * ((size_t)(TA + 1) * TB + (size_t)(TA > TB ? TA : TB) * (lmax + 1));
 }
 
+template <int TB>
 __global__ void __launch_bounds__(kThreads) sketch_f64_kernel(const F64Args a) {
   extern __shared__ double smem[];
-  const int64_t total = f64_tiles<kTA, kTB>(a.W, a.n1, a.cnt);
-  for (int64_t item = blockIdx.x; item < total; item += gridDim.x) f64_tile<kTA, kTB>(a, item, smem);
+  const int64_t total = f64_tiles<kTA, TB>(a.W, a.n1, a.cnt);
+  for (int64_t item = blockIdx.x; item < total; item += gridDim.x) f64_tile<kTA, TB>(a, item, smem);
+}
+
+// Rows (key, r), r < nr, of sketch s into its table: the test-matrix row key + hstride
+// (first + r) of a column sketch, r + n_1 key of a row sketch.
+__global__ void __launch_bounds__(256) f64_table_kernel(const F64Args a, int s, int64_t nkeys, int nr, double* tab) {
+  const SkArg sk = a.sk[s];
+  const int nq = (sk.width + 3) / 4;
+  const int64_t total = nkeys * nr * nq;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t row = e / nq, key = row / nr;
+    const int q = (int)(e - row * nq), r = (int)(row - key * nr);
+    const uint64_t grow = sk.type == SK_COL ? (uint64_t)(key + sk.hstride * (a.first + r)) : (uint64_t)(r + a.n1 * key);
+    double z[4];
+    tm_quad_f64(a.ws, kr_of(a.ws, sk.kr), a.seed, (uint32_t)sk.sid, grow, (uint32_t)q, z);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (4 * q + t < sk.width) tab[row * sk.width + 4 * q + t] = z[t];
+  }
 }
 
 // Batched form: one persistent launch over the tiles of every tensor of the
@@ -178,7 +213,7 @@ __global__ void __launch_bounds__(kThreads) sketch_f64_batched_kernel(const Batc
           sa.nsk = it.nsk;
           for (int s = 0; s < it.nsk; ++s) {
             const DevSketch& d = sks[it.sk0 + s];
-            sa.sk[s] = SkArg{d.rows, d.off, d.wdiv, d.hstride, d.type, d.width, d.stream_id, -1};
+            sa.sk[s] = SkArg{d.rows, d.off, d.wdiv, d.hstride, d.type, d.width, d.stream_id, -1, nullptr};
           }
         }
         __syncthreads();
@@ -210,21 +245,40 @@ cudaError_t launch_sketch_f64(const Plan& P, int item, const void* X, int64_t fi
   int lmax = 1;
   for (int s = 0; s < it.nsk; ++s) {
     const DevSketch& d = sks[it.sk0 + s];
-    a.sk[s] = SkArg{d.rows, d.off, d.wdiv, d.hstride, d.type, d.width, d.stream_id, d.kr_nm ? it.sk0 + s : -1};
+    a.sk[s] = SkArg{d.rows, d.off, d.wdiv, d.hstride, d.type, d.width, d.stream_id, d.kr_nm ? it.sk0 + s : -1, nullptr};
     lmax = d.width > lmax ? d.width : lmax;
   }
-  const size_t smem = f64_smem<kTA, kTB>(lmax);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(sketch_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         96 * 1024);
+  // 64 columns a tile where the planes have them and the tiles still fill the SMs
+  const bool wide = count > kTB && f64_tiles<kTA, 64>(a.W, a.n1, count) >= 4LL * device_sm_count();
+  const int64_t nA = (a.n1 + kTA - 1) / kTA, nB = wide ? (count + 63) / 64 : (count + kTB - 1) / kTB;
+  for (int s = 0; s < it.nsk; ++s) {
+    const DevSketch& d = sks[it.sk0 + s];
+    if (d.st_tab < 0) continue;
+    // rows staged once and the rows drawn by the tiles otherwise; a launch costs as much
+    // as kTableQuads drawn quads
+    const bool col = d.type == SK_COL;
+    const int64_t nkeys = col ? it.W / d.wdiv : d.wdiv, nr = col ? count : a.n1;
+    const int64_t uses = col ? d.wdiv * nA : (it.W / d.wdiv) * nB, nq = (d.width + 3) / 4;
+    if (nr >= (1LL << 31) || (uses - 1) * nkeys * nr * nq < kTableQuads) continue;
+    double* tab = (double*)((char*)ws + d.st_tab);
+    const int64_t blocks = std::min<int64_t>((nkeys * nr * nq + 255) / 256, 8LL * device_sm_count());
+    count_launch();
+    f64_table_kernel<<<(unsigned)blocks, 256, 0, st>>>(a, s, nkeys, (int)nr, tab);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    attr_set = true;
+    a.sk[s].tab = tab;
   }
-  const int64_t total = f64_tiles<kTA, kTB>(a.W, a.n1, count);
-  const int64_t grid = std::min<int64_t>(total, (int64_t)device_sm_count() * 8);
+  const size_t smem = wide ? f64_smem<kTA, 64>(lmax) : f64_smem<kTA, kTB>(lmax);
+  const auto kern = wide ? sketch_f64_kernel<64> : sketch_f64_kernel<kTB>;
+  static bool attr_set[2] = {false, false};
+  if (!attr_set[wide]) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+    if (e != cudaSuccess) return e;
+    attr_set[wide] = true;
+  }
+  const int64_t grid = std::min<int64_t>(a.W * nA * nB, (1LL << 31) - 1);   // a CTA per tile: no uneven last share
   count_launch();
-  sketch_f64_kernel<<<(unsigned)grid, kThreads, smem, st>>>(a);
+  kern<<<(unsigned)grid, kThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
