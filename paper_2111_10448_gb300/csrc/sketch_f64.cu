@@ -14,7 +14,9 @@
 // are FP64 too: a quad of normals costs as much as some 90 FMAs.  So rows that
 // many tiles share are drawn once per accumulate into the backward's scratch (st_tab)
 // and read from there, and planes wide enough take 64 x 64 tiles, which halves what is
-// left on the row side.  @MEASURED@
+// left on the row side.  Accumulate at 64^4, l = 50: 11.1 ms
+// with every row drawn by every 64 x 32 tile, now 7.4, of which the products' FMAs are 6.7;
+// 40^4, l = 16: 1.00 -> 0.49 ms; 300 x 200 x 100, l = 30: 2.18 -> 1.24.
 #include <algorithm>
 
 #include "internal.cuh"
@@ -29,6 +31,7 @@ constexpr int64_t kTableOffB = 256;
 constexpr int kTA = 64;   // rows (i_1) per tile of the single-tensor launch
 constexpr int kTB = 32;   // columns (i_d) per tile
 constexpr int kThreads = 256;
+constexpr int64_t kGroupDoubles = 4096;    // rows of a group of sketches: 32 KB beside a tile of at most 33
 constexpr int64_t kTableQuads = 1 << 17;   // quads of normals that pay for staging them (some 4 us of a launch)
 
 struct SkArg {
@@ -56,12 +59,16 @@ __host__ __device__ constexpr int64_t f64_tiles(int64_t W, int64_t n1, int64_t c
   return W * ((n1 + TA - 1) / TA) * ((cnt + TB - 1) / TB);
 }
 
-// One tile (TA rows of i_1 x TB columns of i_d of plane w) into every sketch.
+// One tile (TA rows of i_1 x TB columns of i_d of plane w) into every sketch.  The
+// sketches go in groups whose rows fit gcap doubles together: a small tile has work
+// for a few warps in each sketch only, and each is a chain of FP64 latencies, so
+// the threads take the quads, then the products, of a whole group at once (40^4, l = 16:
+// 0.72 -> 0.49 ms; 7 x 9 x 8 x 5 x 6, l = 8: 88 -> 54 us).
 template <int TA, int TB>
-__device__ void f64_tile(const F64Args& a, int64_t item, double* smem) {
+__device__ void f64_tile(const F64Args& a, int64_t item, double* smem, int gcap) {
   constexpr int LDX = TA + 1;
   double* Xs = smem;                         // LDX x TB
-  double* Gs = smem + LDX * TB;              // max(TA, TB) rows x LDG
+  double* Gs = smem + LDX * TB;              // gcap: per sketch of a group, nr rows x (width + 1)
   const int tid = threadIdx.x;
   const int64_t nA = (a.n1 + TA - 1) / TA;
   const int64_t nB = (a.cnt + TB - 1) / TB;
@@ -72,71 +79,96 @@ __device__ void f64_tile(const F64Args& a, int64_t item, double* smem) {
   const int ta = (int)imin64(TA, a.n1 - a0);
   const int tb = (int)imin64(TB, a.cnt - b0);
   __syncthreads();
-  for (int o = tid; o < TA * TB; o += kThreads) {
-    const int ia = o % TA, ib = o / TA;
-    double v = 0.0;
-    if (ia < ta && ib < tb) v = load_x(a.X, a.x_f64, (a0 + ia) + a.n1 * w + a.Nd1 * (b0 + ib));
-    Xs[ia + LDX * ib] = v;
+  for (int o = tid; o < ta * tb; o += kThreads) {
+    const int ib = o / ta, ia = o - ib * ta;
+    Xs[ia + LDX * ib] = load_x(a.X, a.x_f64, (a0 + ia) + a.n1 * w + a.Nd1 * (b0 + ib));
   }
-  for (int s = 0; s < a.nsk; ++s) {
-    const SkArg sk = a.sk[s];
-    const int l = sk.width;
-    const int LDG = l + 1;
-    const int64_t wlo = w % sk.wdiv, whi = w / sk.wdiv;
-    const int nr = sk.type == SK_COL ? tb : ta;
-    const int nq = (l + 3) / 4;
-    __syncthreads();
-    if (sk.tab) {
-      // rows (whi, b0 ...) of a column sketch, (wlo, a0 ...) of a row sketch: consecutive
-      const double* src = sk.tab + (sk.type == SK_COL ? whi * a.cnt + b0 : wlo * a.n1 + a0) * l;
-      for (int o = tid; o < nr * l; o += kThreads) {
-        const int r = o / l;
-        Gs[r * LDG + (o - r * l)] = src[o];
-      }
-    }
-    for (int o = tid; o < (sk.tab ? 0 : nr * nq); o += kThreads) {
-      const int r = o % nr, q = o / nr;
-      const uint64_t grow = sk.type == SK_COL
-                                ? (uint64_t)(whi + sk.hstride * (a.first + b0 + r))
-                                : (uint64_t)((a0 + r) + a.n1 * wlo);
-      double z[4];
-      tm_quad_f64(a.ws, kr_of(a.ws, sk.kr), a.seed, (uint32_t)sk.sid, grow, (uint32_t)q, z);
+  for (int s0 = 0; s0 < a.nsk;) {
+    int s1 = s0, used = 0;
+    do {
+      used += (a.sk[s1].type == SK_COL ? tb : ta) * (a.sk[s1].width + 1);
+      ++s1;
+    } while (s1 < a.nsk && used + (a.sk[s1].type == SK_COL ? tb : ta) * (a.sk[s1].width + 1) <= gcap);
+    if (s0) __syncthreads();   // the products of the group before
+    // test-matrix rows: sketch s's jobs follow those of s - 1 over the threads
+    int base = 0;
+    double* G = Gs;
+    for (int s = s0; s < s1; ++s) {
+      const SkArg& sk = a.sk[s];
+      const int l = sk.width, LDG = l + 1, nr = sk.type == SK_COL ? tb : ta, nq = (l + 3) / 4;
+      const int64_t wlo = w % sk.wdiv, whi = w / sk.wdiv;
+      const int first = (tid - base) & (kThreads - 1);
+      if (sk.tab) {
+        // rows (whi, b0 ...) of a column sketch, (wlo, a0 ...) of a row sketch: consecutive
+        const double* src = sk.tab + (sk.type == SK_COL ? whi * a.cnt + b0 : wlo * a.n1 + a0) * l;
+        for (int o = first; o < nr * l; o += kThreads) {
+          const int r = o / l;
+          G[r * LDG + (o - r * l)] = src[o];
+        }
+        base += nr * l;
+      } else {
+        for (int o = first; o < nr * nq; o += kThreads) {
+          const int q = o / nr, r = o - q * nr;
+          const uint64_t grow = sk.type == SK_COL ? (uint64_t)(whi + sk.hstride * (a.first + b0 + r))
+                                                  : (uint64_t)((a0 + r) + a.n1 * wlo);
+          double z[4];
+          tm_quad_f64(a.ws, kr_of(a.ws, sk.kr), a.seed, (uint32_t)sk.sid, grow, (uint32_t)q, z);
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
-        if (4 * q + t < l) Gs[r * LDG + 4 * q + t] = z[t];
+          for (int t = 0; t < 4; ++t)
+            if (4 * q + t < l) G[r * LDG + 4 * q + t] = z[t];
+        }
+        base += nr * nq;
+      }
+      G += nr * LDG;
     }
     __syncthreads();
-    double* out = a.ws + sk.off;
-    if (sk.type == SK_COL) {
-      for (int o = tid; o < TA * l; o += kThreads) {
-        const int ia = o % TA, j = o / TA;
-        if (ia >= ta) continue;
-        double acc = 0.0;
-        for (int ib = 0; ib < tb; ++ib) acc = fma(Xs[ia + LDX * ib], Gs[ib * LDG + j], acc);
-        atomicAdd(out + (a0 + ia + a.n1 * wlo) + sk.rows * j, acc);
-      }
-    } else {
-      for (int o = tid; o < TB * l; o += kThreads) {
-        const int ib = o % TB, j = o / TB;
-        if (ib >= tb) continue;
-        double acc = 0.0;
-        for (int ia = 0; ia < ta; ++ia) acc = fma(Xs[ia + LDX * ib], Gs[ia * LDG + j], acc);
-        atomicAdd(out + (whi + sk.hstride * (a.first + b0 + ib)) + sk.rows * j, acc);
+    base = 0;
+    G = Gs;
+    for (int s = s0; s < s1; ++s) {
+      const SkArg& sk = a.sk[s];
+      const int l = sk.width, LDG = l + 1;
+      const int64_t wlo = w % sk.wdiv, whi = w / sk.wdiv;
+      const int first = (tid - base) & (kThreads - 1);
+      double* out = a.ws + sk.off;
+      if (sk.type == SK_COL) {
+        for (int o = first; o < ta * l; o += kThreads) {
+          const int j = o / ta, ia = o - j * ta;
+          double acc = 0.0;
+          for (int ib = 0; ib < tb; ++ib) acc = fma(Xs[ia + LDX * ib], G[ib * LDG + j], acc);
+          atomicAdd(out + (a0 + ia + a.n1 * wlo) + sk.rows * j, acc);
+        }
+        base += ta * l;
+        G += tb * LDG;
+      } else {
+        for (int o = first; o < tb * l; o += kThreads) {
+          const int j = o / tb, ib = o - j * tb;
+          double acc = 0.0;
+          for (int ia = 0; ia < ta; ++ia) acc = fma(Xs[ia + LDX * ib], G[ia * LDG + j], acc);
+          atomicAdd(out + (whi + sk.hstride * (a.first + b0 + ib)) + sk.rows * j, acc);
+        }
+        base += tb * l;
+        G += ta * LDG;
       }
     }
+    s0 = s1;
   }
 }
 
+// gcap: doubles for the rows of one group of sketches, at least one sketch's.
 template <int TA, int TB>
-__host__ __device__ constexpr size_t f64_smem(int lmax) {
-  return sizeof(double) * ((size_t)(TA + 1) * TB + (size_t)(TA > TB ? TA : TB) * (lmax + 1));
+__host__ __device__ constexpr int f64_gcap(int lmax) {
+  return (TA > TB ? TA : TB) * (lmax + 1);
+}
+template <int TA, int TB>
+__host__ __device__ constexpr size_t f64_smem(int gcap) {
+  return sizeof(double) * ((size_t)(TA + 1) * TB + (size_t)gcap);
 }
 
 template <int TB>
-__global__ void __launch_bounds__(kThreads) sketch_f64_kernel(const F64Args a) {
+__global__ void __launch_bounds__(kThreads) sketch_f64_kernel(const __grid_constant__ F64Args a, int gcap) {
   extern __shared__ double smem[];
   const int64_t total = f64_tiles<kTA, TB>(a.W, a.n1, a.cnt);
-  for (int64_t item = blockIdx.x; item < total; item += gridDim.x) f64_tile<kTA, TB>(a, item, smem);
+  for (int64_t item = blockIdx.x; item < total; item += gridDim.x) f64_tile<kTA, TB>(a, item, smem, gcap);
 }
 
 // Rows (key, r), r < nr, of sketch s into its table: the test-matrix row key + hstride
@@ -162,7 +194,7 @@ __global__ void __launch_bounds__(256) f64_table_kernel(const F64Args a, int s, 
 // their tiles numbered consecutively (prefix[] = first tile of each); a CTA
 // takes `chunk` consecutive tiles at a time from a global counter.
 template <int TA, int TB>
-__global__ void __launch_bounds__(kThreads) sketch_f64_batched_kernel(const BatchLaunch b) {
+__global__ void __launch_bounds__(kThreads) sketch_f64_batched_kernel(const BatchLaunch b, int gcap) {
   extern __shared__ double smem[];
   __shared__ F64Args sa;
   __shared__ int64_t s_base;
@@ -219,7 +251,7 @@ __global__ void __launch_bounds__(kThreads) sketch_f64_batched_kernel(const Batc
         __syncthreads();
         cur = it_idx;
       }
-      f64_tile<TA, TB>(sa, t - prefix[pos], smem);
+      f64_tile<TA, TB>(sa, t - prefix[pos], smem, gcap);
     }
     __syncthreads();
   }
@@ -268,7 +300,14 @@ cudaError_t launch_sketch_f64(const Plan& P, int item, const void* X, int64_t fi
     if (e != cudaSuccess) return e;
     a.sk[s].tab = tab;
   }
-  const size_t smem = wide ? f64_smem<kTA, 64>(lmax) : f64_smem<kTA, kTB>(lmax);
+  // the rows of all sketches in one group where they are few
+  int64_t all = 0;
+  for (int s = 0; s < it.nsk; ++s)
+    all += std::min<int64_t>(a.sk[s].type == SK_COL ? count : a.n1, a.sk[s].type == SK_COL && !wide ? kTB : 64) *
+           (a.sk[s].width + 1);
+  const int gcap = (int)std::max<int64_t>(wide ? f64_gcap<kTA, 64>(lmax) : f64_gcap<kTA, kTB>(lmax),
+                                          std::min<int64_t>(all, kGroupDoubles));
+  const size_t smem = wide ? f64_smem<kTA, 64>(gcap) : f64_smem<kTA, kTB>(gcap);
   const auto kern = wide ? sketch_f64_kernel<64> : sketch_f64_kernel<kTB>;
   static bool attr_set[2] = {false, false};
   if (!attr_set[wide]) {
@@ -278,7 +317,7 @@ cudaError_t launch_sketch_f64(const Plan& P, int item, const void* X, int64_t fi
   }
   const int64_t grid = std::min<int64_t>(a.W * nA * nB, (1LL << 31) - 1);   // a CTA per tile: no uneven last share
   count_launch();
-  kern<<<(unsigned)grid, kThreads, smem, st>>>(a);
+  kern<<<(unsigned)grid, kThreads, smem, st>>>(a, gcap);
   return cudaGetLastError();
 }
 
@@ -287,7 +326,8 @@ int64_t batched_tiles_f64(int64_t W, int64_t n1, int64_t cnt, int ta) {
 }
 
 cudaError_t launch_sketch_f64_batched(const BatchLaunch& b, const BatchCfg& cfg, int lmax, cudaStream_t st) {
-  const size_t smem = cfg.ta == 32 ? f64_smem<32, kTB>(lmax) : f64_smem<64, kTB>(lmax);
+  const int gcap = cfg.ta == 32 ? f64_gcap<32, kTB>(lmax) : f64_gcap<64, kTB>(lmax);
+  const size_t smem = cfg.ta == 32 ? f64_smem<32, kTB>(gcap) : f64_smem<64, kTB>(gcap);
   auto kern = cfg.ta == 32 ? sketch_f64_batched_kernel<32, kTB> : sketch_f64_batched_kernel<64, kTB>;
   static bool attr_set[2] = {false, false};
   if (!attr_set[cfg.ta == 32]) {
@@ -296,7 +336,7 @@ cudaError_t launch_sketch_f64_batched(const BatchLaunch& b, const BatchCfg& cfg,
     attr_set[cfg.ta == 32] = true;
   }
   count_launch();
-  kern<<<cfg.ctas_per_sm * device_sm_count(), kThreads, smem, st>>>(b);
+  kern<<<cfg.ctas_per_sm * device_sm_count(), kThreads, smem, st>>>(b, gcap);
   return cudaGetLastError();
 }
 
