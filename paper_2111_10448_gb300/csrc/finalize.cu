@@ -262,7 +262,7 @@ __device__ __forceinline__ void house_qr(double* A, int lda, int nr, int w, doub
 // barrier between reflectors; one butterfly per reflector for the NC dots;
 // NC > 1 only for blocks of at most 64 rows); NT = ceil(nr / 32) rows per
 // lane, nr <= 256.
-constexpr int kRowsPerLane = 8;
+constexpr int kRowsPerLane = kTsqrMaxRows / 32;
 template <int NC>
 __device__ __forceinline__ void warp_sums(const double (&p)[4], double (&d)[4]) {
   if (NC == 1) {
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kThreads) sketch_unscale_kernel(char* wsb, int
 // tree, so that every root runs in the last launch).  Non-root blocks write
 // their R into the next level's matrix; the root block also does the CPQR, the rank
 // decision and (unless root_sep) the first expansion step.  A root block of at most
-// 6 w rows is pivoted as it stands -- its columns have the norms and inner products
+// 6 w rows or kTsqrOneBlock entries is pivoted as it stands -- its columns have the norms and inner products
 // of R's -- which spares the QR before it and the product of the two Q factors.
 __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int Lg, int* ranks, int root_sep) {
   extern __shared__ double sm[];
@@ -488,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 4) tsqr_level_kernel(char* wsb, int 
   load_block(A, lda, Y + r0, m, nr, w);
   __syncthreads();
   const bool root = (s.lev_nblk[L] == 1);
-  const bool direct = root && nr >= w && nr <= 6 * w;   // pivot the block itself
+  const bool direct = root && nr >= w && (nr <= 6 * w || nr * w <= kTsqrOneBlock);   // pivot the block itself
   const int kmax = min(nr, w);
   // Householder vectors back in place, scalars to the level's beta array
   auto store_block = [&](const double* bt) {
@@ -1383,26 +1383,29 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
       if (e != cudaSuccess) return e;
     }
   }
-  int maxw = 1, maxbl = 1, maxr = 1;
+  int maxw = 1, maxr = 1;
   for (int i = 0, n = 0; i < nitems; ++i) {
     const DevItem& it = plan_items_host(&P)[i];
     for (int s = 0; s < it.nsk; ++s) {
       const DevSketch& d = sks[it.sk0 + s];
       if (!d.basis) continue;
       maxw = std::max(maxw, d.width);
-      for (int L = 0; L < d.nlev; ++L) maxbl = std::max(maxbl, d.lev_bl[L]);
       maxr = std::max(maxr, d.rpad);
       ++n;
     }
   }
-  size_t smem_up = 0;
+  // shared memory of each level's launch (the trees are aligned at their roots)
+  size_t smem_up[kMaxLev] = {}, smem_down[kMaxLev] = {};
   for (int i = 0; i < nitems; ++i) {
     const DevItem& it = plan_items_host(&P)[i];
     for (int s = 0; s < it.nsk; ++s) {
       const DevSketch& d = sks[it.sk0 + s];
       if (!d.basis) continue;
-      for (int L = 0; L < d.nlev; ++L)
-        smem_up = std::max(smem_up, (size_t)(sizeof(double) * tsqr_block_doubles(d.lev_bl[L], d.width)));
+      for (int L = 0; L < d.nlev; ++L) {
+        const int g = L + max_lev - d.nlev;
+        smem_up[g] = std::max(smem_up[g], (size_t)(sizeof(double) * tsqr_block_doubles(d.lev_bl[L], d.width)));
+        smem_down[g] = std::max(smem_down[g], sizeof(double) * ((size_t)tsqr_ld(d.lev_bl[L]) * d.width + TT_MAXL));
+      }
     }
   }
   // the roots' expansion as a launch of its own, its columns over several CTAs, when
@@ -1412,18 +1415,17 @@ cudaError_t launch_finalize(const Plan& P, void* ws, double* cores, int* ranks, 
     const int nt = plan_ntasks(&P, L);
     if (nt == 0) continue;
     count_launch();
-    tsqr_level_kernel<<<nt, kThreads, smem_up, st>>>(wsb, L, ranks, root_sep);
+    tsqr_level_kernel<<<nt, kThreads, smem_up[L], st>>>(wsb, L, ranks, root_sep);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   for (int L = root_sep ? max_lev - 1 : max_lev - 2; L >= 0; --L) {
     const int nt = plan_ntasks(&P, L);
     if (nt == 0) continue;
-    const size_t smem = sizeof(double) * ((size_t)tsqr_ld(maxbl) * maxw + TT_MAXL);
     // columns per CTA: eight (one per warp) when the blocks alone leave SMs idle
     const int cw = nt * ((maxr + 7) / 8) <= 2 * device_sm_count() ? 8 : nt <= device_sm_count() ? 16 : TT_MAXL;
     count_launch();
-    tsqr_expand_kernel<<<dim3((unsigned)nt, (unsigned)((maxr + cw - 1) / cw)), kThreads, smem, st>>>(wsb, L, ranks,
+    tsqr_expand_kernel<<<dim3((unsigned)nt, (unsigned)((maxr + cw - 1) / cw)), kThreads, smem_down[L], st>>>(wsb, L, ranks,
                                                                                                     root_sep, cw);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

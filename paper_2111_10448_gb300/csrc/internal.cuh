@@ -38,6 +38,13 @@ __host__ __device__ __forceinline__ int64_t imin64(int64_t a, int64_t b) { retur
 
 constexpr int kMaxLev = 12;       // TSQR tree depth limit
 constexpr int64_t kTsqrSmemMax = 208 * 1024;  // dynamic shared memory of a TSQR level block
+// Entries up to which a single problem's sketch (or a level's stack of R factors) is one
+// block (of at most kTsqrMaxRows), pivoted as it stands, instead of a QR of blocks and a
+// pivoted QR of their R's: one launch and chain for two or three.  Finalize, split and
+// whole: 256 rows x 9 105 -> 89 us (16^4), 128 x 32 310 -> 273 (128^4), 200 x 20 211 -> 181, 256
+// x 32 404 -> 392.
+constexpr int kTsqrOneBlock = 8192;
+constexpr int kTsqrMaxRows = 256;   // rows of a block: eight a lane in the expansion's registers
 // Leading dimension of a QR block of nr rows in shared memory, and the doubles of a
 // level block of bl rows and width w (block, reduction and reflector scalars, at the
 // root the R factor, Q_2 and the rank sums).

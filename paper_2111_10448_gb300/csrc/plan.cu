@@ -264,16 +264,17 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
     // four).  A level's rows are split evenly, into blocks up to a fifth larger where
     // that spares a block: 572 rows of width 26 make four blocks and a 104-row root
     // instead of five, two of 130 rows and a root (100 us less at d = 6, n = 24).
+    // Up to kTsqrOneBlock entries and kTsqrMaxRows a single problem's rows stay whole.
     const int bl = w <= 16 ? 256 : std::min(192, std::max(128, (4 * w + 31) / 32 * 32));
     if (8 * tsqr_block_doubles(bl, w) > kTsqrSmemMax) return TT_ERR_UNSUPPORTED;
-    int cap = std::min(256, bl + bl / 5);
+    int cap = std::min(kTsqrMaxRows, bl + bl / 5);
     if (8 * tsqr_block_doubles(cap, w) > kTsqrSmemMax) cap = bl;
     int64_t m = s.rows;
     int L = 0;
     while (true) {
       if (L >= kMaxLev) return TT_ERR_UNSUPPORTED;
       s.lev_rows[L] = m;
-      s.lev_nblk[L] = (m + cap - 1) / cap;
+      s.lev_nblk[L] = single && m <= kTsqrMaxRows && m * w <= kTsqrOneBlock ? 1 : (m + cap - 1) / cap;
       s.lev_bl[L] = (int)((m + s.lev_nblk[L] - 1) / s.lev_nblk[L]);
       s.lev_nblk[L] = (m + s.lev_bl[L] - 1) / s.lev_bl[L];
       s.lev_mat[L] = (L == 0) ? s.off : ws.take(m * w);

@@ -1,6 +1,6 @@
 """Basis QRs at the edges of their splits: fewer rows than columns, one block, roots small
-enough to be pivoted as they stand (up to six times the width) and larger ones, several
-levels, widths from one to eight octets of columns.  A tensor of exact rank is recovered
+enough to be pivoted as they stand (up to six times the width, or 8192 entries in up to 256
+rows: width 32 at its 8 l rows) and larger ones, several levels, widths from one to eight octets of columns.  A tensor of exact rank is recovered
 to rounding (a Gaussian sketch of width rank + 6 or more is conditioned below 1e3:
 1e-11), and the right core's rows are orthonormal to 1e-12."""
 import numpy as np
@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("r,p", [(1, 6), (5, 6), (10, 7), (20, 12), (26, 9), (50, 14)])
-@pytest.mark.parametrize("blocks,extra", [(1, -1), (1, 0), (1, 1), (6, 0), (6, 1), (0, 900), (0, 20011)])
+@pytest.mark.parametrize("blocks,extra", [(1, -1), (1, 0), (1, 1), (6, 0), (6, 1), (8, 0), (8, 1), (0, 256), (0, 257), (0, 900), (0, 20011)])
 def test_exact_rank_is_recovered(blocks, extra, r, p):
     n2 = blocks * (r + p) + extra
     g = torch.Generator(device="cuda")
