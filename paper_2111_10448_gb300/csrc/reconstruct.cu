@@ -199,6 +199,186 @@ __global__ void __launch_bounds__(128) wgram_kernel(const void* dX, int dx_f64, 
   }
 }
 
+// The two products with dX in FP32, in digit arithmetic (digits.cuh): C(o, j) += sum_k
+// x(o, k) F(k, j), o the rows u and k the columns v of dX (ROWS, F = Rt^T: Z), or the
+// reverse (F = L: W).  The FP64 pipe bounds the kernels above (1.7 FMAs per cycle and
+// SM); here a block takes 64 outputs and a range of the contraction, 64 at a time:
+// the 64 x 64 tile of dX goes through shared memory (loaded along u either way, the
+// next one in flight meanwhile), a warp scales one output's 64 values by their largest
+// exponent and writes their seven digits, likewise the columns of F, and each 16 x 8
+// tile of sums takes the digit products of weight up to seven of half the 64 (32 x 7
+// x 2^14 < 2^24: exact in FP32), then adds them to its FP64 sums.  What is dropped is
+// below 2^-57 of the largest product of the chunk.  NB column octets.
+// Measured (the whole adjoint, FP64 products and these): 32^5 of rank 8 1.22 -> 0.63 ms,
+// 64^4 of rank 16 1.15 -> 0.48, 48^4 of rank 40 1.30 -> 0.52, 32^4 of rank 8 120 -> 96 us.
+// Entries from which they serve (FP32 dX, both sides at least one tile wide): 512 x 512 of
+// rank 8 72 -> 60 us, 256 x 256 74 -> 57, of rank 32 109 -> 71.
+constexpr int64_t kDxMin = 1 << 16;
+constexpr int kDxP = 7, kDxK = 64, kDxLD = kDxK + 8, kDxRaw = kDxK + 1;
+__host__ __device__ constexpr int dx_smem(int nb) {
+  return 2 * kDxP * (64 + 8 * nb) * kDxLD + 4 * 64 * kDxRaw + 4 * (64 + 8 * nb);
+}
+// An FP32 value as FP64 without the conversion instruction (FP64-pipe rate).
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 255u;
+  if (e - 1u >= 254u) return (double)x;   // zero, subnormal, infinite, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+template <int NB, bool ROWS>
+__global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
+    dx_gemm_kernel(const float* X, int64_t Nk, int64_t Mk, const double* F, int64_t fk, int64_t fj, int rp, double* C,
+                   int64_t co, int64_t cj, int64_t chunks) {
+  using namespace digit;
+  constexpr int P = kDxP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P + 1, ROWS_D = 64 + 8 * NB;
+  extern __shared__ __align__(16) char dsm[];
+  uint16_t* Dg = reinterpret_cast<uint16_t*>(dsm);                         // [P][ROWS_D][kDxLD]
+  float* raw = reinterpret_cast<float*>(dsm + 2 * P * ROWS_D * kDxLD);     // [v][u], ld kDxRaw
+  int* er = reinterpret_cast<int*>(raw + 64 * kDxRaw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
+  const int64_t O = ROWS ? Nk : Mk, K = ROWS ? Mk : Nk, o0 = 64 * (int64_t)blockIdx.x;
+  const int64_t nch = (K + 63) / 64, c0 = (int64_t)blockIdx.y * chunks, c1 = imin64(nch, c0 + chunks);
+  float nx[16];
+  auto fetch = [&](int64_t ch) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int e = tid + 256 * q;
+      const int64_t u = (ROWS ? o0 : 64 * ch) + (e & 63), v = (ROWS ? 64 * ch : o0) + (e >> 6);
+      nx[q] = u < Nk && v < Mk ? __ldg(X + u + Nk * v) : 0.0f;
+    }
+  };
+  double c[NB][4];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) c[q][0] = c[q][1] = c[q][2] = c[q][3] = 0.0;
+  int bad = 0;
+  auto put = [&](int r, double x0, double x1) {   // one digit column, two values a lane
+    bad |= (nonfinite(x0) || nonfinite(x1)) ? 1 : 0;
+    const int m = __reduce_max_sync(0xffffffffu, max(exp_of(x0), exp_of(x1)));
+    if (lane == 0) er[r] = m;
+    uint32_t d0[P], d1[P];
+    digits<P>(fixed<B>(x0, m), d0);
+    digits<P>(fixed<B>(x1, m), d1);
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+      *reinterpret_cast<uint32_t*>(Dg + (p * ROWS_D + r) * kDxLD + 2 * lane) = d0[p] | (d1[p] << 16);
+  };
+  if (c0 < c1) fetch(c0);
+  for (int64_t ch = c0; ch < c1; ++ch) {
+    __syncthreads();   // the products of the chunk before
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int e = tid + 256 * q;
+      raw[(e >> 6) * kDxRaw + (e & 63)] = nx[q];
+    }
+    double fx[NB][2];
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int64_t k = 64 * ch + 2 * lane + e;
+        const int j = warp + 8 * q;
+        fx[q][e] = j < rp && k < K ? __ldg(F + k * fk + j * fj) : 0.0;
+      }
+    __syncthreads();
+    if (ch + 1 < c1) fetch(ch + 1);
+#pragma unroll 2
+    for (int r = warp; r < 64; r += 8) {
+      const float* p = ROWS ? raw + 2 * lane * kDxRaw + r : raw + r * kDxRaw + 2 * lane;
+      put(r, widen(p[0]), widen(p[ROWS ? kDxRaw : 1]));
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) put(64 + warp + 8 * q, fx[q][0], fx[q][1]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+      const int t = warp + 8 * q, kk = 32 * (t & 1), mt = (t >> 1) & 3, nt = t >> 3;
+      float acc[NW][4];
+#pragma unroll
+      for (int w = 0; w < NW; ++w) acc[w][0] = acc[w][1] = acc[w][2] = acc[w][3] = 0.0f;
+      const uint32_t pa = s_u32(Dg + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kDxLD + kk + 8 * (lane >> 4));
+      const uint32_t pb = s_u32(Dg + (64 + 8 * nt + (lane & 7)) * kDxLD + kk + 8 * (lane >> 3));
+      constexpr int stride = 2 * ROWS_D * kDxLD;
+      uint32_t fb[P][4];   // both k-steps of each digit of F
+#pragma unroll
+      for (int p = 0; p < P; ++p) ldsm4(pb + p * stride, fb[p]);
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          uint32_t fa[4];
+          ldsm4(pa + p * stride + 32 * ks, fa);
+#pragma unroll
+          for (int p2 = 0; p2 < P; ++p2)
+            if (p + p2 < NW) mma(acc[(p + p2) % NW], fa, fb[p2] + 2 * ks);
+        }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int x = er[16 * mt + gq + 8 * (e >> 1)] + er[64 + 8 * nt + 2 * tq + (e & 1)] - 2 * LEAD - 56;
+        long long hi = 0, lo = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          hi = hi * 256 + __float2int_rn(acc[w][e]);
+          lo = lo * 256 + __float2int_rn(acc[w + 4][e]);
+        }
+        if (hi | lo) {   // (hi 2^32 + lo) 2^x; a column of zeros has no exponent
+          const double v = fma((double)hi, 4294967296.0, (double)lo);
+          if (x > -900 && x < 900) c[q][e] = fma(v, __hiloint2double((x + 1023) << 20, 0), c[q][e]);
+          else c[q][e] += ldexp(v, x);
+        }
+      }
+    }
+  }
+  // a non-finite value in this block's range: its products as FP64 FMAs
+  if (__syncthreads_or(bad)) {
+    for (int i = tid; i < 64 * rp; i += 256) {
+      const int64_t o = o0 + (i & 63);
+      const int j = i >> 6;
+      if (o >= O) continue;
+      double t = 0.0;
+      for (int64_t k = 64 * c0; k < imin64(K, 64 * c1); ++k)
+        t = fma((double)__ldg(X + (ROWS ? o + Nk * k : k + Nk * o)), __ldg(F + k * fk + j * fj), t);
+      atomicAdd(C + o * co + j * cj, t);
+    }
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < NB; ++q) {
+    const int t = warp + 8 * q, mt = (t >> 1) & 3, nt = t >> 3;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int64_t o = o0 + 16 * mt + gq + 8 * (e >> 1);
+      const int j = 8 * nt + 2 * tq + (e & 1);
+      if (o < O && j < rp) atomicAdd(C + o * co + j * cj, c[q][e]);
+    }
+  }
+}
+template <int NB, bool ROWS>
+cudaError_t launch_dx_gemm_nb(const float* X, int64_t Nk, int64_t Mk, const double* F, int64_t fk, int64_t fj, int rp,
+                              double* C, int64_t co, int64_t cj, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(dx_gemm_kernel<NB, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, dx_smem(NB));
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const int64_t ob = ((ROWS ? Nk : Mk) + 63) / 64, nch = ((ROWS ? Mk : Nk) + 63) / 64;
+  // about four blocks an SM: an output's sums are added once a block
+  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(nch, 4LL * device_sm_count() / ob));
+  const int64_t chunks = (nch + want - 1) / want;
+  count_launch();
+  dx_gemm_kernel<NB, ROWS><<<dim3((unsigned)ob, (unsigned)((nch + chunks - 1) / chunks)), 256, dx_smem(NB), st>>>(
+      X, Nk, Mk, F, fk, fj, rp, C, co, cj, chunks);
+  return cudaGetLastError();
+}
+template <bool ROWS>
+cudaError_t launch_dx_gemm(const float* X, int64_t Nk, int64_t Mk, const double* F, int64_t fk, int64_t fj, int rp,
+                           double* C, int64_t co, int64_t cj, cudaStream_t st) {
+  if (rp <= 8) return launch_dx_gemm_nb<1, ROWS>(X, Nk, Mk, F, fk, fj, rp, C, co, cj, st);
+  if (rp <= 16) return launch_dx_gemm_nb<2, ROWS>(X, Nk, Mk, F, fk, fj, rp, C, co, cj, st);
+  if (rp <= 32) return launch_dx_gemm_nb<4, ROWS>(X, Nk, Mk, F, fk, fj, rp, C, co, cj, st);
+  return launch_dx_gemm_nb<8, ROWS>(X, Nk, Mk, F, fk, fj, rp, C, co, cj, st);
+}
+
 // Z_{k-1}(u, a) = sum_{i, c} Z_k(u + N_{k-1} i, c) G_k(a, i, c): one warp per entry,
 // the lanes over (i, c).
 __global__ void zdown_kernel(const double* Z, int64_t Np, int64_t nk, int rpc, const double* G, int rpa, double* Zo) {
@@ -395,8 +575,8 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
 // others; from there the cores absorb one mode at a time (Z_{k-1} from Z_k and G_k,
 // W_k from W_{k-1} and G_k), so only these two products see every entry (2 N r
 // FMAs).  One contraction per core (d N r FMAs, and the interfaces of length
-// N_{d-1}) took 4.5 ms for 32^5 of rank 8; this takes 1.2 ms, 1.1 of them FP64-pipe
-// time of the two products.
+// N_{d-1}) took 4.5 ms for 32^5 of rank 8; this takes 1.2 ms with the two products on the
+// FP64 pipe and 0.63 with them in digit arithmetic.
 cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* cores, const void* dXt,
                                         int dx_f64, double* dcores, void* ws, cudaStream_t st) {
   const DevItem& it = plan_items_host(&P)[item];
@@ -414,6 +594,8 @@ cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* c
   const int64_t Nm = it.N[ds], Mm = it.N[d] / Nm;
   const int rp = it.rpad[ds];
   const int64_t sms = device_sm_count();
+  const bool dig = !dx_f64 && Nm >= 64 && Mm >= 64 && Nm * Mm >= kDxMin && (Nm + 63) / 64 < (1LL << 31) &&
+                     (Mm + 63) / 64 < (1LL << 31);
   {  // Z_ds = dX Rt_{ds+1}^T; v chunks sized so that about 32k warp jobs cover the entries
     double* Z = W + it.off_Z[ds];
     e = cudaMemsetAsync(Z, 0, sizeof(double) * Nm * rp, st);
@@ -422,15 +604,20 @@ cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* c
     const int64_t nrb = (Nm + 31) / 32, nvg = ((Mm + vc - 1) / vc + 3) / 4;
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>(nrb * nvg, 16 * sms));
     const double* Rt = W + it.off_Rt[ds + 1];
-    count_launch();
-    if (rp <= 8)
-      ygram_kernel<8><<<g, 128, 4 * 8 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
-    else if (rp <= 16)
-      ygram_kernel<16><<<g, 128, 4 * 16 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
-    else if (rp <= 32)
-      ygram_kernel<32><<<g, 128, 4 * 32 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
-    else
-      ygram_kernel<64><<<g, 128, 4 * 64 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+    if (dig) {
+      e = launch_dx_gemm<true>((const float*)dXt, Nm, Mm, Rt, rp, 1, rp, Z, 1, Nm, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      count_launch();
+      if (rp <= 8)
+        ygram_kernel<8><<<g, 128, 4 * 8 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+      else if (rp <= 16)
+        ygram_kernel<16><<<g, 128, 4 * 16 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+      else if (rp <= 32)
+        ygram_kernel<32><<<g, 128, 4 * 32 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+      else
+        ygram_kernel<64><<<g, 128, 4 * 64 * 32 * sizeof(double), st>>>(dXt, dx_f64, Nm, Mm, Rt, rp, Z, vc);
+    }
   }
   {  // W_ds = L_ds^T dX; row chunks likewise
     double* Wd = W + it.off_Wd[ds];
@@ -443,11 +630,16 @@ cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* c
     const int64_t jobs = nvg * ((Nm + uc - 1) / uc);
     const int g = (int)std::max<int64_t>(1, std::min<int64_t>((jobs + 3) / 4, 16 * sms));
     const double* L = W + it.off_L[ds];
-    count_launch();
-    if (rp <= 8) wgram_kernel<8, 4><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
-    else if (rp <= 16) wgram_kernel<16, 2><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
-    else if (rp <= 32) wgram_kernel<32, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
-    else wgram_kernel<64, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+    if (dig) {
+      e = launch_dx_gemm<false>((const float*)dXt, Nm, Mm, L, 1, Nm, rp, Wd, rp, 1, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      count_launch();
+      if (rp <= 8) wgram_kernel<8, 4><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+      else if (rp <= 16) wgram_kernel<16, 2><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+      else if (rp <= 32) wgram_kernel<32, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+      else wgram_kernel<64, 1><<<g, 128, 0, st>>>(dXt, dx_f64, Nm, Mm, L, rp, Wd, uc);
+    }
   }
   for (int k = ds; k >= 1; --k) {
     const int64_t Np = it.N[k - 1], nk = it.n[k - 1];
