@@ -211,8 +211,9 @@ tt_status tt_plan_sketch_info(tt_plan_t plan, int item, int index, int* type, in
 
 /* Which sketch kernel an accumulate of `count_last` last-mode slices runs for
  * item 0: 0 = FP64 SIMT kernel, 1 = generic tensor-core kernel (mma.sync,
- * any shape; in single-problem plans the test-matrix rows that several
- * tiles read are staged once per call, up to 256 MB a sketch), 2 = a tcgen05
+ * any shape: the strip kernel where there are at most three sketches a side,
+ * else 64 x 32 tiles; test-matrix rows that several tiles read are staged once
+ * per call where they find room in scratch), 2 = a tcgen05
  * kernel: the plane kernel (n_1 and count_last in {128, 256}, d in {3, 4},
  * dense Gaussian test matrices, equal widths with 16 <= l * #sketches per
  * side <= 32) or the slab kernel (d = 4, n_1 in {128, 256}, l in {8, 16},
@@ -221,8 +222,9 @@ tt_status tt_plan_sketch_info(tt_plan_t plan, int item, int index, int* type, in
  * launch), both BF16 or FP16 and two-sided; 3 = small-plane kernel (BF16,
  * FP16 or TF32,
  * n_1 and count_last <= 32, widths l_k <= 32, padded to the widest; mma.sync
- * with test-matrix rows shared by many planes staged once per call).  Host
- * only. */
+ * with test-matrix rows shared by many planes staged once per call; with dense
+ * Gaussian test matrices and at most three sketches a side the strip kernel
+ * takes these shapes, several planes a tile).  Host only. */
 int tt_sketch_kernel_kind(tt_plan_t plan, int64_t count_last);
 
 /* Problem of item `item` as stored by the plan (ranks clamped). */
@@ -319,7 +321,9 @@ tt_status tt_pstt2_batched(tt_plan_t plan, const void* const* X_ptrs, void* ws, 
  * the largest number of kR values in a 16-plane block (1, 2, 4 or 8; other
  * values mean 4); chunk = tiles (blocks) a CTA takes from the work counter at
  * a time (>= 1), ctas_per_sm = persistent CTAs per SM (1..32; the small-plane
- * kernel always runs one).  Host only. */
+ * kernel always runs one).  A batch of such items with at most three
+ * sketches a side is one launch of the strip kernel, whose split follows from
+ * the shapes: the values are kept and have no effect there.  Host only. */
 tt_status tt_plan_batch_config(tt_plan_t plan, int ta, int chunk, int ctas_per_sm);
 
 /* Autotuner of the batched sketch (not in the paper): runs the batched

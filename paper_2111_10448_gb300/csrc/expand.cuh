@@ -38,13 +38,18 @@ struct ExpandArgs {
   int64_t nub, vlen;   // blocks of u, columns v per CTA
   float* out;          // FP32 output
   const float* X;      // or the tensor to compare with
-  double* out2;
+  double* out2;        // [2], added to with atomics, or kErrSlots pairs of it (slots)
+  int slots;
   int vec;             // float4 accesses are aligned
 };
 
 __device__ __forceinline__ float pow2f(int e) {  // 2^e, zero below the normal range, e <= 127
   return e < -126 ? 0.0f : __int_as_float((min(e, 127) + 127) << 23);
 }
+
+// A thousand CTAs' error sums added into one FP64 word one after another drift (the
+// addends are alike: 1.4e-15 of the sum); they go to this many pairs first.
+constexpr int kErrSlots = 64;
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -137,14 +142,17 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
   // rows within 2^60 of one another: products with fu are exact
   const bool narrow = eU - eLow <= 60;
 
-  float s_e = 0.f, s_el = 0.f, s_x = 0.f, s_xl = 0.f;   // error sums, scaled by 2^(-2 kb)
+  // Error sums, scaled by 2^(-2 kb): the sum, the rounding errors of its additions and
+  // those of the squares.  (Both kinds in one word lose 5e-15 of the sum, always
+  // downwards; apart 5e-16.)
+  float s_e = 0.f, s_el = 0.f, s_er = 0.f, s_x = 0.f, s_xl = 0.f, s_xr = 0.f;
   int kb = -100;
   // into the FP64 sums (a sum that is not finite keeps its leading part only)
   auto fold = [&]() {
     const double sc = __hiloint2double((2 * kb + 1023) << 20, 0);
-    e2 += (fabsf(s_e) <= 3.0e38f ? (double)s_e + (double)s_el : (double)s_e) * sc;
-    x2 += (fabsf(s_x) <= 3.0e38f ? (double)s_x + (double)s_xl : (double)s_x) * sc;
-    s_e = s_el = s_x = s_xl = 0.f;
+    e2 += (fabsf(s_e) <= 3.0e38f ? (double)s_e + ((double)s_el + (double)s_er) : (double)s_e) * sc;
+    x2 += (fabsf(s_x) <= 3.0e38f ? (double)s_x + ((double)s_xl + (double)s_xr) : (double)s_x) * sc;
+    s_e = s_el = s_er = s_x = s_xl = s_xr = 0.f;
   };
   for (int64_t vc = v0; vc < v1; vc += kVT) {
     const int nv = (int)imin64(kVT, v1 - vc);
@@ -325,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
           k2 = min(k2, 126);
           if (k2 != kb) {
             const float f = pow2f(max(2 * (kb - k2), -126));
-            s_e *= f, s_el *= f, s_x *= f, s_xl *= f;
+            s_e *= f, s_el *= f, s_er *= f, s_x *= f, s_xl *= f, s_xr *= f;
             kb = k2;
           }
           const float fx = pow2f(-kb), ft = pow2f(min(eb - kb, 127));
@@ -346,11 +354,13 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
             float s, c;
             two_sum(s_e, p, s, c);
             s_e = s;
-            s_el += c + pe;
+            s_el += c;
+            s_er += pe;
             const float px = __fmul_rn(xs, xs);
             two_sum(s_x, px, s, c);
             s_x = s;
-            s_xl += c + __fmaf_rn(xs, xs, -px);
+            s_xl += c;
+            s_xr += __fmaf_rn(xs, xs, -px);
           }
         }
       }
@@ -369,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
     if (tid < 2) {
       double s = 0.0;
       for (int w = 0; w < kWarps; ++w) s += red[tid][w];
-      atomicAdd(a.out2 + tid, s);
+      atomicAdd(a.out2 + (a.slots ? 2 * (blockIdx.x % kErrSlots) : 0u) + tid, s);
     }
   }
 }

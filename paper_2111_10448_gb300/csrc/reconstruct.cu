@@ -527,6 +527,16 @@ cudaError_t run_expand_ks(const expand::ExpandArgs& a, cudaStream_t st) {
   }
 }
 
+// out2 = the sums of the kErrSlots pairs of slots.
+__global__ void err_slots_kernel(const double* slots, double* out2) {
+  static_assert(expand::kErrSlots == 64, "two pairs a lane");
+  double a = slots[2 * threadIdx.x] + slots[2 * threadIdx.x + 64];   // pairs lane, lane + 32
+  double b = slots[2 * threadIdx.x + 1] + slots[2 * threadIdx.x + 65];
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (threadIdx.x == 0) out2[0] = a, out2[1] = b;
+}
+
 }  // namespace
 
 cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, void* Xt, int x_f64,
@@ -546,9 +556,10 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
   // interfaces at least as long as a staging step.  Measured (whole call, us, FP64
   // kernel -> digit kernel): below the line 64^3 rank 2: 8 -> 11, 9^6 rank 8: 23 ->
   // 26; above it 1000 x 1000 rank 3: 12.8 -> 12.2, 100^3 rank 10: 28 -> 17, 128^3
-  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 4750 (3.6 TB/s
+  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 4770 (3.6 TB/s
   // of the output; the epilogue and the digit products share the issue slots);
-  // error sums 24^6 rank 10: 4590 -> 859.
+  // error sums 24^6 rank 10: 4590 -> 923 (859 before the rounding errors of sums and
+  // squares were kept apart).
   if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && Nm * Mm >= (3 << 18)) {
     expand::ExpandArgs a;
     a.L = W + it.off_L[ds];
@@ -560,7 +571,17 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
     a.X = (const float*)Xcmp;
     a.out2 = out2;
     a.vec = Nm % 4 == 0 && ((uintptr_t)(Xt ? Xt : Xcmp) & 15) == 0 ? 1 : 0;
-    return Xt ? run_expand_ks<5, 4, 0>(a, st) : run_expand_ks<7, 2, 1>(a, st);
+    a.slots = 0;
+    if (Xt) return run_expand_ks<5, 4, 0>(a, st);
+    if (it.off_small == 0) return run_expand_ks<7, 2, 1>(a, st);   // (a batched plan of one has no such scratch)
+    a.out2 = W + it.off_small;
+    a.slots = 1;
+    e = cudaMemsetAsync(a.out2, 0, 2 * expand::kErrSlots * sizeof(double), st);
+    if (e == cudaSuccess) e = run_expand_ks<7, 2, 1>(a, st);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    err_slots_kernel<<<1, 32, 0, st>>>(a.out2, out2);
+    return cudaGetLastError();
   }
   count_launch();
   dense_kernel<<<grid_for(Nm * Mm), kThreads, 0, st>>>(W + it.off_L[ds], W + it.off_Rt[ds + 1], Nm, Mm,
