@@ -464,7 +464,7 @@ static tt_status build_item(Plan& P, const tt_problem& q0, WsAlloc& ws, int64_t&
   // scratch and the other tile kernels' staging areas, largest table first; rows that
   // find no room are drawn per tile.  Reading a staged row costs less than drawing it
   // even when it comes from HBM (a 64-byte row 3 cycles of an SM's share of the
-  // bandwidth, its seven column quads 13 cycles at 0.52 quads a cycle).
+  // bandwidth, its seven column quads 10 cycles at 0.68 quads a cycle).
   // The FP64 kernel's rows (width doubles each; a quad of its normals costs some 90 FMAs
   // of the units that bound it) take the same room; its launch says which it fills.
   {

@@ -1,7 +1,9 @@
 // Small-plane fused multi-sketch (BF16, FP16 or TF32 tensor cores, X split
 // into hi + lo; the description below uses BF16)
-// for tensors whose first and last modes are small (n_1, n_d <= 32), e.g. the
-// d = 6, n = 24 random-TT workload and the many small tensors of a batch.
+// for tensors whose first and last modes are small (n_1, n_d <= 32) that the strip
+// kernel (strip.cuh) does not take: Khatri-Rao test matrices, and d >= 7 (more than three
+// sketches a side), e.g. d = 9, n = 12.  Dense ones up to d = 6 are its own now (d = 6, n =
+// 24: 5.9 ms here, 2.7 there).
 //
 // Every plane X(:, w, :) (n_1 x n_d, w = kL + WL kR with WL = N_{d*}/n_1)
 // contributes a plain product to every sketch of the one-pass sketch

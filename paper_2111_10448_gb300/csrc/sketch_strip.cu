@@ -19,13 +19,18 @@
 // (cp.async) while this one is multiplied; two CTAs per SM overlap one's staging
 // with the other's products.
 //
-// What bounds it: mma.sync (1015 FMA per cycle and SM measured in 16 bits):
-// 2 d round8(l) FMAs an entry.
+// What bounds it: issue slots, of which 53-60 % are used (16 warps an SM leave
+// barriers and dependent chains uncovered).  At 96^4 x 48, l = 28, leaving one part out
+// saved: the normals 7.6 of 32.7 ms (5.3 since they take fewer slots), the rest of the
+// staging 5, conversion 4, copies of X 2, column products 2.2, row products 3.7.
+// mma.sync itself (1015 FMA per cycle and SM measured in 16 bits, 2 d round8(l) FMAs an
+// entry) is busy 15 %.
 //
 // Measured (one accumulate, BF16 unless named; the 64 x 32 tile kernel that served
-// these shapes before in brackets): 960^3, l = 35: 3.45 ms (13.0); 64^5, l = 28:
-// 9.3 ms (26); 300^3, l = 60: 0.36 ms (0.79), TF32 0.55 (0.87); 200 x 128 x 100 x
-// 80, l = 16, FP16 Khatri-Rao: 1.08 ms (4.33); 16 x 300 x 300: 0.071 ms (0.150).
+// these shapes before in brackets): 960^3, l = 35: 3.28 ms (13.0); 64^5, l = 28:
+// 7.4 ms (26); 300^3, l = 60: 0.375 ms (0.79), TF32 0.53 (0.87); 200 x 128 x 100 x
+// 80, l = 16, FP16 Khatri-Rao: 1.03 ms (4.33); 16 x 300 x 300: 0.072 ms (0.150).
+// 24^6, l = 26: 2.68 ms (small-plane kernel: 10.7).
 // No shape tried was slower, down to 9 x 9 x 1000 and 2 x 1000 x 1000, so every
 // call with at most three sketches a side takes it (d <= 6 two-sided, d <= 4
 // one-sided; more accumulators than that do not fit the registers and the
