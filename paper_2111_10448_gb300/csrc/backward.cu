@@ -44,8 +44,12 @@ __device__ __forceinline__ const DevSketch* sketches_of(const char* wsb) {
   return reinterpret_cast<const DevSketch*>(wsb + T.off_sketches);
 }
 
-// 1. Qbar_k / Pbar_k from the core adjoints (gather form: one thread per entry).
-__global__ void qbar_kernel(char* wsb, int item, int k, const double* dG, const int* ranks) {
+// 1. Qbar_k / Pbar_k from the core adjoints (gather form).  A block takes 32 entries, one a
+// lane, and its warps share each entry's sums (up to n_k r_k terms; the outermost
+// k has n_1 r entries only, which one thread each held to a single SM).  Measured
+// (backward of 32^5, rank 8, k = 1..4): 225 us with a thread per entry, now 46.
+constexpr int kQbarParts = kThreads / 32;
+__global__ void __launch_bounds__(kThreads) qbar_kernel(char* wsb, int item, int k, const double* dG, const int* ranks) {
   const DevItem& it = item_of(wsb, item);
   const DevSketch* S = sketches_of(wsb);
   const DevSketch& sb = S[it.basis_of_k[k]];
@@ -58,21 +62,22 @@ __global__ void qbar_kernel(char* wsb, int item, int k, const double* dG, const 
   auto G = [&](int kk, int a, int64_t i, int c) -> double {
     return dG[it.core_off[kk] + a + (int64_t)it.rpad[kk - 1] * (i + it.n[kk - 1] * c)];
   };
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * rp;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t row = e % rows;
+  __shared__ double sums[kQbarParts][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  for (int64_t e0 = 32 * (int64_t)blockIdx.x; e0 < rows * rp; e0 += 32 * (int64_t)gridDim.x) {
+    const int64_t e = e0 + lane, row = e % rows;
     const int c = (int)(e / rows);
     double val = 0.0;
-    if (c < rk[k]) {
+    if (e < rows * rp && c < rk[k]) {
       if (k < ds) {
         // B side of core k
         if (k == 1) {
-          val += G(1, 0, row, c);
+          if (part == 0) val += G(1, 0, row, c);
         } else {
           const DevSketch& sa = S[it.basis_of_k[k - 1]];
           const int64_t Np = it.N[k - 1];
           const int64_t u = row % Np, i = row / Np;
-          for (int a = 0; a < rk[k - 1]; ++a) val += ws[sa.lev_z[0] + u + sa.rows * a] * G(k, a, i, c);
+          for (int a = part; a < rk[k - 1]; a += kQbarParts) val += ws[sa.lev_z[0] + u + sa.rows * a] * G(k, a, i, c);
         }
         // A side of core k+1
         const int64_t nk1 = it.n[k], Nk = it.N[k];
@@ -86,28 +91,37 @@ __global__ void qbar_kernel(char* wsb, int item, int k, const double* dG, const 
           Bm = ws + s2.lev_z[0];
           ldb = s2.rows;
         }
-        for (int64_t i2 = 0; i2 < nk1; ++i2)
+        for (int64_t i2 = part; i2 < nk1; i2 += kQbarParts)
           for (int c2 = 0; c2 < rk[k + 1]; ++c2) val += G(k + 1, c, i2, c2) * Bm[row + Nk * i2 + ldb * c2];
       } else {
         // A side of core k+1: P_k(i + n_{k+1} v, a)
         const int64_t nk1 = it.n[k];
         const int64_t i = row % nk1, v = row / nk1;
         if (k + 1 == d) {
-          val += G(d, c, i, 0);
+          if (part == 0) val += G(d, c, i, 0);
         } else {
           const DevSketch& s2 = S[it.basis_of_k[k + 1]];
-          for (int c2 = 0; c2 < rk[k + 1]; ++c2) val += G(k + 1, c, i, c2) * ws[s2.lev_z[0] + v + s2.rows * c2];
+          for (int c2 = part; c2 < rk[k + 1]; c2 += kQbarParts)
+            val += G(k + 1, c, i, c2) * ws[s2.lev_z[0] + v + s2.rows * c2];
         }
         // B side of core k (k > d*): P_k(v, c)
         if (k > ds) {
           const DevSketch& sa = S[it.basis_of_k[k - 1]];
           const int64_t nk = it.n[k - 1];
           for (int a = 0; a < rk[k - 1]; ++a)
-            for (int64_t i2 = 0; i2 < nk; ++i2) val += ws[sa.lev_z[0] + i2 + nk * row + sa.rows * a] * G(k, a, i2, c);
+            for (int64_t i2 = part; i2 < nk; i2 += kQbarParts) val += ws[sa.lev_z[0] + i2 + nk * row + sa.rows * a] * G(k, a, i2, c);
         }
       }
     }
-    out[row + rows * c] = val;
+    sums[part][lane] = val;
+    __syncthreads();
+    if (part == 0 && e < rows * rp) {
+      double t = 0.0;
+#pragma unroll
+      for (int p = 0; p < kQbarParts; ++p) t += sums[p][lane];
+      out[row + rows * c] = t;
+    }
+    __syncthreads();
   }
 }
 
@@ -317,7 +331,7 @@ cudaError_t launch_backward(const Plan& P, int item, const double* dcores, void*
   for (int k = 1; k < d; ++k) {
     const int64_t n = sks[it.basis_of_k[k]].rows * sks[it.basis_of_k[k]].rpad;
     count_launch();
-    qbar_kernel<<<grid_for(n), kThreads, 0, st>>>(wsb, item, k, dcores, ranks_dev);
+    qbar_kernel<<<grid_for(n * kQbarParts), kThreads, 0, st>>>(wsb, item, k, dcores, ranks_dev);
   }
   count_launch();
   hbar_kernel<<<grid_for(it.N[ds] * it.rpad[ds]), kThreads, 0, st>>>(wsb, item, dcores, ranks_dev);
