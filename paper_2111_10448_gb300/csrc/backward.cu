@@ -366,7 +366,9 @@ cudaError_t launch_backward(const Plan& P, int item, const double* dcores, void*
     gram_kernel<<<g2, kThreads, 0, st>>>(W + sb.lev_z[0], sb.rows, W + it.off_qbar[k], sb.rows, sb.rows, sb.rpad,
                                           sb.rpad, Wk, sb.rpad);
     count_launch();
-    qr_abar_kernel<<<grid_for(sb.rows, 8), 128, 0, st>>>(wsb, item, k, ranks_dev, Wk);
+    // one warp a block: a row is a chain of r^2 FP64 steps, so few rows go over many SMs
+    qr_abar_kernel<<<(unsigned)std::min<int64_t>((sb.rows + 31) / 32, 32LL * device_sm_count()), 32, 0, st>>>(
+        wsb, item, k, ranks_dev, Wk);
   }
   // 4. dX
   return launch_sketch_adjoint(P, item, dX, ws, st);
