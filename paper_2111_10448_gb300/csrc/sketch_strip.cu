@@ -31,7 +31,7 @@
 // 7.4 ms (26); 300^3, l = 60: 0.375 ms (0.79), TF32 0.53 (0.87); 200 x 128 x 100 x
 // 80, l = 16, FP16 Khatri-Rao: 1.03 ms (4.33); 16 x 300 x 300: 0.072 ms (0.150).
 // 24^6, l = 26: 2.68 ms (small-plane kernel: 10.7).
-// No shape tried was slower, down to 9 x 9 x 1000 and 2 x 1000 x 1000, so every
+// No shape tried was slower, down to 8^3, 9 x 9 x 1000 and 2 x 1000 x 1000, so every
 // call with at most three sketches a side takes it (d <= 6 two-sided, d <= 4
 // one-sided; more accumulators than that do not fit the registers and the
 // 64 x 32 kernel stays).
@@ -52,6 +52,10 @@ namespace {
 
 constexpr int kSmemTwo = 111 * 1024;   // dynamic shared memory of a CTA, two per SM
 constexpr int kSmemOne = 224 * 1024;   // one per SM
+// Quads of normals that pay for staging them: 2.6 us at 2.0e11 a second, a launch.  Sketch
+// with every shared row staged -> with this: 16^4 47 -> 40 us, 9^6 TF32 172 -> 161, 4 x 30 x 30 x
+// 30 x 5 106 -> 92, 512 x 512 45 -> 39; 24^6 and 960^3 stage as before.
+constexpr int64_t kTableQuads = 1 << 19;
 constexpr int64_t kBatchUnit = 1 << 17;  // entries of a batched unit, about
 
 int strip_octets(const Plan& P, int item) {
@@ -83,6 +87,13 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
     k.hstride = d.hstride;
     k.tab = d.st_tab;
     if (d.wdiv >= (1LL << 31)) return false;
+    if (!nt_batch && k.tab >= 0) {
+      // quads drawn without the table (a row per tile row that reads it) less those it holds
+      const bool col = d.type == SK_COL;
+      const int64_t rows = col ? it.W / d.wdiv * count : d.wdiv * it.n[0];
+      const int64_t uses = col ? d.wdiv * ((it.n[0] + kMaxTA - 1) / kMaxTA) : it.W / d.wdiv * ((count + 63) / 64);
+      if ((uses - 1) * rows * ((d.width + 3) / 4) < kTableQuads) k.tab = -1;
+    }
     k.wdiv = (uint32_t)d.wdiv;
     k.width = d.width;
     k.nq = (d.width + 3) / 4;
@@ -264,9 +275,10 @@ cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t 
   g.vec = it.n[0] % 4 == 0 && ((uintptr_t)X & 15) == 0 ? 1 : 0;
   g.cpr = g.rawld / 4;
   g.total = g.Nd1 * count;
+  int ic = 0, ir = 0;
   for (int s = 0; s < it.nsk; ++s) {
     const DevSketch& d = sks[it.sk0 + s];
-    if (d.st_tab < 0) continue;
+    if ((d.type == SK_COL ? g.col[ic++] : g.row[ir++]).tab < 0) continue;
     // stage the sketch's rows for this call, in the kernel's own row format: the
     // slab's i_d (column side) or i_1 (row side)
     const bool col = d.type == SK_COL;

@@ -41,6 +41,8 @@ CASES = [
     ([64, 4, 64], 30, 34, [64]),                  # 8 octets
     ([144, 3, 2, 200], 5, 6, [100, 100]),         # several column tiles a unit
     ([1, 50, 70], 2, 5, [70]),                    # a single row of i_1
+    ([129, 40, 40, 65], 6, 5, [65]),              # staged test-matrix rows on both sides
+    ([129, 40, 40, 65], 6, 5, [33, 32]),          # on the row side alone
 ]
 
 
@@ -107,6 +109,7 @@ GROUPED = [
     ([1, 6, 5, 3], 2, 2, [3]),
     ([20, 18], 6, 6, [18]),
     ([10, 40, 12, 8], 5, 6, [1, 7]),
+    ([24, 24, 24, 24, 24], 10, 10, [24]),         # with staged test-matrix rows
     ([40, 5, 6, 7, 20], 9, 6, [20]),              # grouped along i_{d-1} and i_2, past the small-plane limit
 ]
 
