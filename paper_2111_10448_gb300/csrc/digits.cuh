@@ -19,6 +19,12 @@ __device__ __forceinline__ void mma(float* c, const uint32_t* a, const uint32_t*
                "{%0,%1,%2,%3};" : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+// The same with c = 0 on entry (no registers cleared first).
+__device__ __forceinline__ void mma0(float* c, const uint32_t* a, const uint32_t* b) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+               "{%10,%10,%10,%10};" : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.0f));
+}
 
 // Exponent e with |x| < 2^e (kExpZero for zero and subnormal numbers, which count as zero).
 __device__ __forceinline__ int exp_of(double x) {
@@ -26,6 +32,11 @@ __device__ __forceinline__ int exp_of(double x) {
   return e == 0 ? kExpZero : e - 1022;
 }
 __device__ __forceinline__ bool nonfinite(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) == 0x7ff; }
+// Infinite, NaN or subnormal: not what the digits hold.
+__device__ __forceinline__ bool undigital(double x) {
+  const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  return e - 1u >= 0x7feu && x != 0.0;
+}
 
 // round(x 2^(B - E)), |x| < 2^E, in integer arithmetic.
 template <int B>

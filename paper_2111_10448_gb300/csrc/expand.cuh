@@ -5,18 +5,27 @@
 // What bounded the FP64 form: a warp's FP64 FMA holds its sub-partition for 64
 // cycles on this GPU (1.72 FMA per cycle and SM measured), so rank 6 cost 51 ms
 // for 256^4 entries where writing them takes 2.5 ms.  Here every FP64 value is
-// written in P balanced base-256 digits (8 P - 3 or 4 bits below the scale of its row
-// or column); the digits are exact BF16 values, a product of two digits summed
-// over a contraction of up to 64 and over the pairs of equal weight stays below
-// 2^23, so the FP32 accumulation of mma.sync is exact.  Pairs (i, j) with i + j <
-// P are kept (P (P + 1) / 2 MMAs per k-step), one accumulator per weight, and the
-// result is put together by Horner's rule.
+// written in P = 7 balanced base-256 digits, 53 bits (52 at ranks above 48) below the
+// scale of its row or column; the digits are exact BF16 values, a product of two
+// digits summed over a contraction of up to 64 and over the pairs of equal weight stays
+// below 2^23, so the FP32 accumulation of mma.sync is exact.  (Splitting operands so
+// that low-precision products sum without error: Ozaki, Ogita, Oishi, Rump, Numer.
+// Algorithms 59, 2012.)  Pairs (i, j) with i + j < P are kept (P (P + 1) / 2 MMAs per
+// k-step), one accumulator per weight, and the result is put together by Horner's rule.
 //
 // Scales (powers of two): per column c of the CTA's rows of L (moved over to the
 // rows of Rt, so that no gauge between the two costs digits), then per row u of L
-// and per column v of Rt.  The dropped part is below P 2^(7 - 8 P) times the rank
-// times the largest term any entry of that row and column could have: below
-// 2^-35 of that term for P = 5 (FP32 output), 2^-50 for P = 7 (error sums), times the rank.
+// and per column v of Rt.  In units of the largest term that any entry of the row and
+// the column could have, a term is off by at most 2^-53 (two roundings of 2^-54) plus
+// the pairs left out, 6 2^14 2^-56 2^-10 and smaller ones: 2^-49.2 in all (2^-47.2 at
+// ranks above 48; in the accumulators' units 2^-31.2 either way).
+//
+// FP32 output: an entry below 2^27 times that bound, or below sixteen times what the last
+// addition rounds off, is summed again in FP64 (dot64).  So every entry is within 1/4 of a
+// half-ulp of the FP64 sum rounded once, however far it lies below its row's and column's
+// scale -- localised components that are large in different places, cancellation.
+// For random factors one entry in 10^4 is summed again; where all are (components that
+// nowhere meet) the call costs what the FP64 form did and the digits besides.
 #pragma once
 #include <cstdint>
 
@@ -55,6 +64,13 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
   const float bb = __fsub_rn(s, a);
   e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// An entry in FP64.
+__device__ __noinline__ double dot64(const double* L, int64_t ldl, const double* R, int rp) {
+  double s = 0.0;
+  for (int c = 0; c < rp; ++c) s = fma(__ldg(L + ldl * c), __ldg(R + c), s);
+  return s;
 }
 
 // KS k-steps of 16 (rp <= 16 KS; KS = 0: rp <= 8, one k-step holds two digits),
@@ -104,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
     int m = kExpZero;
     for (int i = lane; i < nu; i += 32) {
       const double x = a.L[u0 + i + a.Nm * c];
-      bad |= nonfinite(x) ? 1 : 0;
+      bad |= undigital(x) ? 1 : 0;
       m = max(m, exp_of(x));
     }
     m = __reduce_max_sync(0xffffffffu, m);
@@ -167,7 +183,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
       if (v < nv)
         for (int c = q; c < a.rp; c += 4) {
           const double x = r[c];
-          bad |= nonfinite(x) ? 1 : 0;
+          bad |= undigital(x) ? 1 : 0;
           const int e = exp_of(x);
           if (e != kExpZero && ec[c] != kExpZero) m = max(m, e + ec[c]);
         }
@@ -188,11 +204,10 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
       }
     }
     const bool slow = __syncthreads_or(bad) || bad_l;
-    if (slow) {  // a non-finite entry: FP64 arithmetic as it stands
+    if (slow) {  // a non-finite or subnormal factor: FP64 arithmetic as it stands
       for (int o = tid; o < nu * nv; o += kThreads) {
         const int64_t u = u0 + o % nu, v = vc + o / nu;
-        double s = 0.0;
-        for (int c = 0; c < a.rp; ++c) s += a.L[u + a.Nm * c] * a.Rt[c + (int64_t)a.rp * v];
+        const double s = dot64(a.L + u, a.Nm, a.Rt + v * a.rp, a.rp);
         if constexpr (MODE == 0) {
           a.out[u + a.Nm * v] = (float)s;
         } else {
@@ -227,10 +242,6 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
         }
       }
       float acc[NTL][P][4];
-#pragma unroll
-      for (int n = 0; n < NTL; ++n)
-#pragma unroll
-        for (int w = 0; w < P; ++w) acc[n][w][0] = acc[n][w][1] = acc[n][w][2] = acc[n][w][3] = 0.0f;
       const uint32_t ra = s_u32(Rd + (vs + (lane & 7) + 8 * ((lane >> 3) & 1)) * LD + 8 * (lane >> 4));
       const uint32_t la = s_u32(Ld + (gu * UW + 8 * (lane >> 4) + (lane & 7)) * LD + 8 * ((lane >> 3) & 1));
 #pragma unroll
@@ -251,10 +262,15 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
           for (int i = 0; i < PA; ++i)
             if ((HALF ? 2 * i : i) + j < P)
 #pragma unroll
-              for (int n = 0; n < NTL; ++n) mma(acc[n][((HALF ? 2 * i : i) + j) % P], fa[i], fb[n]);
+              for (int n = 0; n < NTL; ++n) {
+                float* c = acc[n][((HALF ? 2 * i : i) + j) % P];
+                if (ks == 0 && j <= (HALF ? 1 : 0)) mma0(c, fa[i], fb[n]);   // the first pair of its weight
+                else mma(c, fa[i], fb[n]);
+              }
         }
       }
       constexpr float kD = 0x1p-8f;
+      const float least = 0.0625f * (float)a.rp;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int v = vs + g + 8 * h;
@@ -264,17 +280,24 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
         const int e_v = ev[v];
         if constexpr (MODE == 0) {
           float r[2 * NTL];
+          uint32_t redo = 0;   // entries too small for their digits
 #pragma unroll
           for (int n = 0; n < NTL; ++n)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-              // Horner's rule; A0 256 + A1 is exact, so an entry far below its
-              // terms is still rounded only once
+              // (A0 256 + A1) + 2^-8 A2 = x + xe without error (the first sum is an exact
+              // integer and the second a multiple of 2^-8 below 2^16 wherever it is the larger),
+              // then the rest y in one rounding each
               const int q = 2 * h + e;
               float s = acc[n][P - 1][q];
 #pragma unroll
-              for (int w = P - 2; w >= 2; --w) s = fmaf(s, kD, acc[n][w][q]);
-              r[2 * n + e] = fmaf(s, kD, fmaf(acc[n][0][q], 256.0f, acc[n][1][q]));
+              for (int w = P - 2; w >= 3; --w) s = fmaf(s, kD, acc[n][w][q]);
+              const float a01 = fmaf(acc[n][0][q], 256.0f, acc[n][1][q]);
+              const float x = fmaf(acc[n][2][q], kD, a01);
+              const float xe = fmaf(acc[n][2][q], kD, a01 - x);
+              const float y = fmaf(s, 0x1p-16f, xe);
+              r[2 * n + e] = x + y;
+              if (fabsf(r[2 * n + e]) < fmaf(fabsf(y), 16.0f, least)) redo |= 1u << (2 * n + e);
             }
           // times 2^(eu + ev) over full scale
           const int eb = eU + e_v - 2 * LEAD - 8;
@@ -290,6 +313,16 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
               r[n] = r[n] * pow2f(x1) * pow2f(x2);
             }
           }
+          // (a zero row or column has no terms)
+          if (redo && e_v != kExpZero)
+#pragma unroll 1
+            for (; redo; redo &= redo - 1) {
+              const int k = __ffs(redo) - 1;
+              if (ur + k >= nu || eu[ur + k] == kExpZero) continue;
+              const float s = (float)dot64(a.L + u0 + ur + k, a.Nm, a.Rt + (vc + v) * a.rp, a.rp);
+#pragma unroll
+              for (int n = 0; n < 2 * NTL; ++n) r[n] = n == k ? s : r[n];
+            }
           if (a.vec && ur + 2 * NTL <= nu) {
 #pragma unroll
             for (int n = 0; n < NTL; n += 2)

@@ -556,8 +556,9 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
   // interfaces at least as long as a staging step.  Measured (whole call, us, FP64
   // kernel -> digit kernel): below the line 64^3 rank 2: 8 -> 11, 9^6 rank 8: 23 ->
   // 26; above it 1000 x 1000 rank 3: 12.8 -> 12.2, 100^3 rank 10: 28 -> 17, 128^3
-  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 4770 (3.6 TB/s
-  // of the output; the epilogue and the digit products share the issue slots);
+  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 8880 (4770
+  // with five digits, which left entries far below their row's and column's scale without
+  // correct bits; 16 warps an SM wait on their own chains, half of the issue slots used);
   // error sums 24^6 rank 10: 4590 -> 923 (859 before the rounding errors of sums and
   // squares were kept apart).
   if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && Nm * Mm >= (3 << 18)) {
@@ -572,7 +573,7 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
     a.out2 = out2;
     a.vec = Nm % 4 == 0 && ((uintptr_t)(Xt ? Xt : Xcmp) & 15) == 0 ? 1 : 0;
     a.slots = 0;
-    if (Xt) return run_expand_ks<5, 4, 0>(a, st);
+    if (Xt) return run_expand_ks<7, 2, 0>(a, st);
     if (it.off_small == 0) return run_expand_ks<7, 2, 1>(a, st);   // (a batched plan of one has no such scratch)
     a.out2 = W + it.off_small;
     a.slots = 1;
