@@ -45,10 +45,10 @@ __device__ __forceinline__ long long fixed(double x, int E) {
   const int e = (int)((bits >> 52) & 0x7ff);
   if (e == 0) return 0;
   const unsigned long long m = ((unsigned long long)bits & 0xfffffffffffffull) | (1ull << 52);
-  static_assert(B <= 53, "the shift below is not negative");
+  static_assert(B <= 61, "q and its balanced digits fit 64 bits");
   const int s = 1075 + E - B - e;   // >= 53 - B
   if (s > 54) return 0;
-  const long long q = (long long)(s > 0 ? (m + (1ull << (s - 1))) >> s : m);
+  const long long q = (long long)(s > 0 ? (m + (1ull << (s - 1))) >> s : B > 53 ? m << -s : m);
   return bits < 0 ? -q : q;
 }
 

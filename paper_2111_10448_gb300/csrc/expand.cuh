@@ -5,8 +5,8 @@
 // What bounded the FP64 form: a warp's FP64 FMA holds its sub-partition for 64
 // cycles on this GPU (1.72 FMA per cycle and SM measured), so rank 6 cost 51 ms
 // for 256^4 entries where writing them takes 2.5 ms.  Here every FP64 value is
-// written in P = 7 balanced base-256 digits, 53 bits (52 at ranks above 48) below the
-// scale of its row or column; the digits are exact BF16 values, a product of two
+// written in P balanced base-256 digits, P = 7 for the output and 8 for the error sums: 8 P -
+// 3 bits (one less at ranks above 48) below the scale of its row or column; the digits are exact BF16 values, a product of two
 // digits summed over a contraction of up to 64 and over the pairs of equal weight stays
 // below 2^23, so the FP32 accumulation of mma.sync is exact.  (Splitting operands so
 // that low-precision products sum without error: Ozaki, Ogita, Oishi, Rump, Numer.
@@ -16,9 +16,10 @@
 // Scales (powers of two): per column c of the CTA's rows of L (moved over to the
 // rows of Rt, so that no gauge between the two costs digits), then per row u of L
 // and per column v of Rt.  In units of the largest term that any entry of the row and
-// the column could have, a term is off by at most 2^-53 (two roundings of 2^-54) plus
-// the pairs left out, 6 2^14 2^-56 2^-10 and smaller ones: 2^-49.2 in all (2^-47.2 at
-// ranks above 48; in the accumulators' units 2^-31.2 either way).
+// the column could have, a term is off at P = 7 by at most 2^-53 (two roundings of 2^-54)
+// plus the pairs left out, 6 2^14 2^-56 2^-10 and smaller ones: 2^-49.2 in all (2^-47.2 at
+// ranks above 48; in the accumulators' units 2^-31.2 either way); at P = 8 by 2^-57.1
+// (2^-55.1).
 //
 // FP32 output: an entry below 2^27 times that bound, or below sixteen times what the last
 // addition rounds off, is summed again in FP64 (dot64).  So every entry is within 1/4 of a
@@ -26,6 +27,11 @@
 // scale -- localised components that are large in different places, cancellation.
 // For random factors one entry in 10^4 is summed again; where all are (components that
 // nowhere meet) the call costs what the FP64 form did and the digits besides.
+//
+// Error sums: a residual is x minus the three-word sum of the weights, squares and sums are
+// held in words of their own (below), so that neither the residuals nor the sums are further
+// off than in FP64: 1009 x 803, sum of squares 1e-16 off at most (FP64 2e-15), a tensor met
+// to rounding 1e-16 as in FP64.
 #pragma once
 #include <cstdint>
 
@@ -78,8 +84,8 @@ __device__ __noinline__ double dot64(const double* L, int64_t ldl, const double*
 // output; 1: error sums.
 //
 // KS = 0: a k-step of 16 takes two pairs of equal weight at once, [digit 2m, digit
-// 2m + 1] of Rt against [digit j, digit j - 1] of L (weights 2m + j): 9 MMAs instead
-// of 15 (P = 5), 16 instead of 28 (P = 7).
+// 2m + 1] of Rt against [digit j, digit j - 1] of L (weights 2m + j): 16 MMAs instead of
+// 28 (P = 7), 20 instead of 36 (P = 8).
 template <int P, int KS, int UT, int NTL, int MODE>
 __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const ExpandArgs a) {
   constexpr bool HALF = KS == 0;
@@ -158,17 +164,18 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
   // rows within 2^60 of one another: products with fu are exact
   const bool narrow = eU - eLow <= 60;
 
-  // Error sums, scaled by 2^(-2 kb): the sum, the rounding errors of its additions and
-  // those of the squares.  (Both kinds in one word lose 5e-15 of the sum, always
-  // downwards; apart 5e-16.)
-  float s_e = 0.f, s_el = 0.f, s_er = 0.f, s_x = 0.f, s_xl = 0.f, s_xr = 0.f;
+  // Error sums, scaled by 2^(-2 kb): the sum, the rounding errors of its additions, those
+  // of the squares and those of the latter's additions.  (The trailing bits of squares are
+  // not evenly spread, and dl^2 below is always positive: without the last word a sum is
+  // 5e-16 too small.)
+  float s_e = 0.f, s_el = 0.f, s_er = 0.f, s_eq = 0.f, s_x = 0.f, s_xl = 0.f, s_xr = 0.f, s_xq = 0.f;
   int kb = -100;
   // into the FP64 sums (a sum that is not finite keeps its leading part only)
   auto fold = [&]() {
     const double sc = __hiloint2double((2 * kb + 1023) << 20, 0);
-    e2 += (fabsf(s_e) <= 3.0e38f ? (double)s_e + ((double)s_el + (double)s_er) : (double)s_e) * sc;
-    x2 += (fabsf(s_x) <= 3.0e38f ? (double)s_x + ((double)s_xl + (double)s_xr) : (double)s_x) * sc;
-    s_e = s_el = s_er = s_x = s_xl = s_xr = 0.f;
+    e2 += (fabsf(s_e) <= 3.0e38f ? (double)s_e + ((double)s_el + ((double)s_er + (double)s_eq)) : (double)s_e) * sc;
+    x2 += (fabsf(s_x) <= 3.0e38f ? (double)s_x + ((double)s_xl + ((double)s_xr + (double)s_xq)) : (double)s_x) * sc;
+    s_e = s_el = s_er = s_eq = s_x = s_xl = s_xr = s_xq = 0.f;
   };
   for (int64_t vc = v0; vc < v1; vc += kVT) {
     const int nv = (int)imin64(kVT, v1 - vc);
@@ -176,6 +183,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
     __syncthreads();
     // ---- columns vc.. of Rt: four threads a column
     bad = 0;
+    bool low = false, ordinary = false;   // error sums: X~ below 2^-160, or not
     {
       const int v = tid >> 2, q = tid & 3;
       const double* r = a.Rt + (vc + v) * a.rp;
@@ -190,6 +198,11 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
       m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
       m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
       if (q == 0) ev[v] = m;
+      if (MODE == 1 && m != kExpZero && eU != kExpZero) {
+        bad |= m + eU > 110 ? 1 : 0;   // X~ past FP32's range
+        low = m + eU < -160;
+        ordinary = !low;
+      }
       for (int c = 2 * q; c < a.rp; c += 8) {
         uint32_t d0[P], d1[P];
         // a zero column of L has no terms: its entries of Rt count as zero
@@ -203,8 +216,9 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
               d0[p] | (d1[p] << 16);
       }
     }
-    const bool slow = __syncthreads_or(bad) || bad_l;
-    if (slow) {  // a non-finite or subnormal factor: FP64 arithmetic as it stands
+    bool slow = __syncthreads_or(bad) || bad_l;
+    if (MODE == 1 && __syncthreads_or(low)) slow |= !__syncthreads_or(ordinary);
+    if (slow) {  // a non-finite or subnormal factor, X~ out of range: FP64 arithmetic as it stands
       for (int o = tid; o < nu * nv; o += kThreads) {
         const int64_t u = u0 + o % nu, v = vc + o / nu;
         const double s = dot64(a.L + u, a.Nm, a.Rt + v * a.rp, a.rp);
@@ -334,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
               if (ur + n < nu) a.out[at + n] = r[n];
           }
         } else {
-          float hi[2 * NTL], lo[2 * NTL];
+          float hi[2 * NTL], mid[2 * NTL], lo[2 * NTL];
           const float(&x)[2 * NTL] = xv[h];
           float mx = 0.f, mt = 0.f;
 #pragma unroll
@@ -342,22 +356,19 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
               const int k = 2 * n + e, q = 2 * h + e;
+              // (A0 256 + A1) + 2^-8 A2 = hi + r as above and r + 2^-16 A3 = t, a multiple of
+              // 2^-16 below 2^7, exactly; t + 2^-24 A4 = mid + lo, then the rest
+              const float a01 = fmaf(acc[n][0][q], 256.0f, acc[n][1][q]);
+              hi[k] = fmaf(acc[n][2][q], kD, a01);
+              const float t = fmaf(acc[n][3][q], 0x1p-16f, fmaf(acc[n][2][q], kD, a01 - hi[k]));
               float s = acc[n][P - 1][q];
 #pragma unroll
-              for (int w = P - 2; w >= 4; --w) s = fmaf(s, kD, acc[n][w][q]);
-              // A0 256 + A1 (exact) + 2^-8 (A2 + 2^-8 (A3 + 2^-8 s)) as hi + lo
-              float h3, l3, h2, l2, h0, l0;
-              two_sum(acc[n][3][q], s * kD, h3, l3);
-              two_sum(acc[n][2][q], h3 * kD, h2, l2);
-              l2 = fmaf(l3, kD, l2);
-              two_sum(fmaf(acc[n][0][q], 256.0f, acc[n][1][q]), h2 * kD, h0, l0);
-              l0 = fmaf(l2, kD, l0);
-              // (zero for a row past the block, whose x is zero, too)
-              const float f = fu[ur + k];
-              hi[k] = h0 * f;
-              lo[k] = l0 * f;
+              for (int w = P - 2; w >= 5; --w) s = fmaf(s, kD, acc[n][w][q]);
+              mid[k] = fmaf(acc[n][4][q], 0x1p-24f, t);
+              lo[k] = fmaf(s, 0x1p-32f, fmaf(acc[n][4][q], 0x1p-24f, t - mid[k]));
+              // (fu is zero for a row past the block, whose x is zero, too)
               mx = fmaxf(mx, fabsf(x[k]));
-              mt = fmaxf(mt, fabsf(hi[k]));
+              mt = fmaxf(mt, fabsf(hi[k] * fu[ur + k]));
             }
           // running scale 2^kb of the sums: at least this batch's largest value
           const int eb = eU + e_v - 2 * LEAD - 8;
@@ -366,34 +377,41 @@ __global__ void __launch_bounds__(kThreads, KS <= 2 ? 2 : 1) expand_kernel(const
           k2 = min(k2, 126);
           if (k2 != kb) {
             const float f = pow2f(max(2 * (kb - k2), -126));
-            s_e *= f, s_el *= f, s_er *= f, s_x *= f, s_xl *= f, s_xr *= f;
+            s_e *= f, s_el *= f, s_er *= f, s_eq *= f, s_x *= f, s_xl *= f, s_xr *= f, s_xq *= f;
             kb = k2;
           }
           const float fx = pow2f(-kb), ft = pow2f(min(eb - kb, 127));
 #pragma unroll
           for (int k = 0; k < 2 * NTL; ++k) {
-            const float xs = x[k] * fx;
-            float d, dl;
-            two_sum(xs, -(hi[k] * ft), d, dl);
+            // x - hi - mid - lo = d + dl, d the leading 24 bits
+            const float xs = x[k] * fx, f = fu[ur + k] * ft;
+            float d, dl, el;
+            two_sum(xs, -(hi[k] * f), d, dl);
             if (fabsf(d) <= 3.0e38f) {   // an infinite entry stays infinite
-              dl -= lo[k] * ft;
-              const float s = d + dl;
-              dl = dl - (s - d);
+              two_sum(d, -(mid[k] * f), d, el);
+              dl += fmaf(-lo[k], f, el);
+              const float s = __fadd_rn(d, dl);
+              dl = __fsub_rn(dl, __fsub_rn(s, d));
               d = s;
             } else {
               dl = 0.f;
             }
-            const float p = __fmul_rn(d, d), pe = fmaf(2.0f * d, dl, __fmaf_rn(d, d, -p));
+            const float p = __fmul_rn(d, d);
+            const float pe = fmaf(2.0f * d, dl, __fmaf_rn(d, d, -p));   // and dl^2, below its last bit
             float s, c;
             two_sum(s_e, p, s, c);
             s_e = s;
             s_el += c;
-            s_er += pe;
-            const float px = __fmul_rn(xs, xs);
+            s = __fadd_rn(s_er, pe);
+            s_eq = fmaf(dl, dl, __fadd_rn(s_eq, __fsub_rn(pe, __fsub_rn(s, s_er))));
+            s_er = s;
+            const float px = __fmul_rn(xs, xs), pxe = __fmaf_rn(xs, xs, -px);
             two_sum(s_x, px, s, c);
             s_x = s;
             s_xl += c;
-            s_xr += __fmaf_rn(xs, xs, -px);
+            s = __fadd_rn(s_xr, pxe);
+            s_xq += __fsub_rn(pxe, __fsub_rn(s, s_xr));
+            s_xr = s;
           }
         }
       }

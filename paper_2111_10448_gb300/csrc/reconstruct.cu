@@ -519,9 +519,10 @@ cudaError_t run_expand(expand::ExpandArgs a, cudaStream_t st) {
 template <int P, int NTL, int MODE>
 cudaError_t run_expand_ks(const expand::ExpandArgs& a, cudaStream_t st) {
   if (a.rp <= 8) return run_expand<P, 0, 256, NTL, MODE>(a, st);
+  // rows that leave two CTAs an SM in shared memory, as far as 64
   switch ((a.rp + 15) / 16) {
-    case 1: return run_expand<P, 1, 256, NTL, MODE>(a, st);
-    case 2: return run_expand<P, 2, 128, NTL, MODE>(a, st);
+    case 1: return run_expand<P, 1, P == 7 ? 256 : 128, NTL, MODE>(a, st);
+    case 2: return run_expand<P, 2, P == 7 ? 128 : 64, NTL, MODE>(a, st);
     case 3: return run_expand<P, 3, 128, NTL, MODE>(a, st);
     default: return run_expand<P, 4, 128, NTL, MODE>(a, st);
   }
@@ -559,8 +560,8 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
   // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 8880 (4770
   // with five digits, which left entries far below their row's and column's scale without
   // correct bits; 16 warps an SM wait on their own chains, half of the issue slots used);
-  // error sums 24^6 rank 10: 4590 -> 923 (859 before the rounding errors of sums and
-  // squares were kept apart).
+  // error sums 24^6 rank 10: 4590 -> 1117 (923 with seven digits and residuals in FP32
+  // pairs, which were further off than FP64 ones).
   if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && Nm * Mm >= (3 << 18)) {
     expand::ExpandArgs a;
     a.L = W + it.off_L[ds];
@@ -574,11 +575,11 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
     a.vec = Nm % 4 == 0 && ((uintptr_t)(Xt ? Xt : Xcmp) & 15) == 0 ? 1 : 0;
     a.slots = 0;
     if (Xt) return run_expand_ks<7, 2, 0>(a, st);
-    if (it.off_small == 0) return run_expand_ks<7, 2, 1>(a, st);   // (a batched plan of one has no such scratch)
+    if (it.off_small == 0) return run_expand_ks<8, 2, 1>(a, st);   // (a batched plan of one has no such scratch)
     a.out2 = W + it.off_small;
     a.slots = 1;
     e = cudaMemsetAsync(a.out2, 0, 2 * expand::kErrSlots * sizeof(double), st);
-    if (e == cudaSuccess) e = run_expand_ks<7, 2, 1>(a, st);
+    if (e == cudaSuccess) e = run_expand_ks<8, 2, 1>(a, st);
     if (e != cudaSuccess) return e;
     count_launch();
     err_slots_kernel<<<1, 32, 0, st>>>(a.out2, out2);
