@@ -65,5 +65,24 @@ __device__ __forceinline__ void digits(long long q, uint32_t (&d)[P]) {
     d[i] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | byte), 8388736.0f)) >> 16;
   }
 }
+
+// c += |a| |b|: of leading digits, a measure of a product's terms (below).
+__device__ __forceinline__ void mma_abs(float* c, const uint32_t* a, const uint32_t* b) {
+  uint32_t x[4], y[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = a[i] & 0x7fff7fffu;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) y[i] = b[i] & 0x7fff7fffu;
+  mma(c, x, y);
+}
+
+// Whether a sum of digit products has to be formed in FP64 instead.  mag = sum |d0 d0'|
+// of the leading digits, full scale 2^LEAD each; a digit that is not zero is at most twice its
+// value, so the terms' magnitudes add up to at least mag 2^(-2 LEAD) / 4 of the two largest factors'
+// product.  Below `part` of that they may be as small as what the digits drop; then the
+// digits still serve if they are exact below the last bit of the sum so far, |sum| >= 2^e.
+__device__ __forceinline__ bool weak(float mag, float part, int lead, double sum, int e) {
+  return mag < part * (float)(1 << (2 * lead)) && exp_of(sum) <= e;
+}
 }  // namespace digit
 }  // namespace tts

@@ -205,18 +205,24 @@ __global__ void __launch_bounds__(128) wgram_kernel(const void* dX, int dx_f64, 
 // SM); here a block takes 64 outputs and a range of the contraction, 64 at a time:
 // the 64 x 64 tile of dX goes through shared memory (loaded along u either way, the
 // next one in flight meanwhile), a warp scales one output's 64 values by their largest
-// exponent and writes their seven digits, likewise the columns of F, and each 16 x 8
-// tile of sums takes the digit products of weight up to seven of half the 64 (32 x 7
-// x 2^14 < 2^24: exact in FP32), then adds them to its FP64 sums.  What is dropped is
-// below 2^-57 of the largest product of the chunk.  NB column octets.
-// Measured (the whole adjoint, FP64 products and these): 32^5 of rank 8 1.22 -> 0.63 ms,
-// 64^4 of rank 16 1.15 -> 0.48, 48^4 of rank 40 1.30 -> 0.52, 32^4 of rank 8 120 -> 96 us.
+// exponent and writes their eight digits, likewise the columns of F, and each 16 x 8
+// tile of sums takes the digit products of weight up to seven of half the 64 (8 x 32
+// x 2^14 < 2^24: exact in FP32), then adds them to its FP64 sums.  A value keeps 61 bits
+// below the largest of its 64, and a sum of 32 products is off by at most 32 2^-57 of the two
+// largest factors' product (pairs of weight eight and more); where the factors' magnitudes
+// say that this is not small against sum |x F| (digit::weak), the 32 products are FP64
+// FMAs.  So an entry is held to 2^-44 of sum |x F| at worst, and for random factors is
+// closer than FP64 FMAs.  NB column octets.  (The digits' 16-byte chunks are swizzled by their
+// row instead of padded: two CTAs an SM up to NB = 4.)
+// Measured (the whole adjoint, FP64 products and these): 32^5 of rank 8 1.22 -> 0.76 ms,
+// 64^4 of rank 16 1.15 -> 0.57, 48^4 of rank 40 1.30 -> 0.57, 32^4 of rank 8 120 -> 87 us (0.62, 0.47,
+// 0.50 ms and 83 us with seven digits and no test of the terms).
 // Entries from which they serve (FP32 dX, both sides at least one tile wide): 512 x 512 of
-// rank 8 72 -> 60 us, 256 x 256 74 -> 57, of rank 32 109 -> 71.
+// rank 8 72 -> 47 us, 256 x 256 74 -> 47, of rank 32 109 -> 67.
 constexpr int64_t kDxMin = 1 << 16;
-constexpr int kDxP = 7, kDxK = 64, kDxLD = kDxK + 8, kDxRaw = kDxK + 1;
+constexpr int kDxP = 8, kDxK = 64, kDxRaw = kDxK + 1;
 __host__ __device__ constexpr int dx_smem(int nb) {
-  return 2 * kDxP * (64 + 8 * nb) * kDxLD + 4 * 64 * kDxRaw + 4 * (64 + 8 * nb);
+  return 2 * kDxP * (64 + 8 * nb) * kDxK + 4 * 64 * kDxRaw + 4 * (64 + 8 * nb);
 }
 // An FP32 value as FP64 without the conversion instruction (FP64-pipe rate).
 __device__ __forceinline__ double widen(float x) {
@@ -224,15 +230,20 @@ __device__ __forceinline__ double widen(float x) {
   if (e - 1u >= 254u) return (double)x;   // zero, subnormal, infinite, NaN
   return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
 }
+// s + sum_k x(k) F(k) in FP64.
+__device__ __noinline__ double dx_dot(const float* x, int sx, const double* F, int64_t fk, int n, double s) {
+  for (int k = 0; k < n; ++k) s = fma((double)x[k * sx], __ldg(F + k * fk), s);
+  return s;
+}
 template <int NB, bool ROWS>
 __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
     dx_gemm_kernel(const float* X, int64_t Nk, int64_t Mk, const double* F, int64_t fk, int64_t fj, int rp, double* C,
                    int64_t co, int64_t cj, int64_t chunks) {
   using namespace digit;
-  constexpr int P = kDxP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P + 1, ROWS_D = 64 + 8 * NB;
+  constexpr int P = kDxP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P, ROWS_D = 64 + 8 * NB;
   extern __shared__ __align__(16) char dsm[];
-  uint16_t* Dg = reinterpret_cast<uint16_t*>(dsm);                         // [P][ROWS_D][kDxLD]
-  float* raw = reinterpret_cast<float*>(dsm + 2 * P * ROWS_D * kDxLD);     // [v][u], ld kDxRaw
+  uint16_t* Dg = reinterpret_cast<uint16_t*>(dsm);                         // [P][ROWS_D][kDxK]
+  float* raw = reinterpret_cast<float*>(dsm + 2 * P * ROWS_D * kDxK);     // [v][u], ld kDxRaw
   int* er = reinterpret_cast<int*>(raw + 64 * kDxRaw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, tq = lane & 3;
   const int64_t O = ROWS ? Nk : Mk, K = ROWS ? Mk : Nk, o0 = 64 * (int64_t)blockIdx.x;
@@ -251,7 +262,7 @@ __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
   for (int q = 0; q < NB; ++q) c[q][0] = c[q][1] = c[q][2] = c[q][3] = 0.0;
   int bad = 0;
   auto put = [&](int r, double x0, double x1) {   // one digit column, two values a lane
-    bad |= (nonfinite(x0) || nonfinite(x1)) ? 1 : 0;
+    bad |= (undigital(x0) || undigital(x1)) ? 1 : 0;
     const int m = __reduce_max_sync(0xffffffffu, max(exp_of(x0), exp_of(x1)));
     if (lane == 0) er[r] = m;
     uint32_t d0[P], d1[P];
@@ -259,7 +270,8 @@ __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
     digits<P>(fixed<B>(x1, m), d1);
 #pragma unroll
     for (int p = 0; p < P; ++p)
-      *reinterpret_cast<uint32_t*>(Dg + (p * ROWS_D + r) * kDxLD + 2 * lane) = d0[p] | (d1[p] << 16);
+      *reinterpret_cast<uint32_t*>(Dg + (p * ROWS_D + r) * kDxK + 8 * ((lane >> 2) ^ (r & 7)) + 2 * (lane & 3)) =
+          d0[p] | (d1[p] << 16);
   };
   if (c0 < c1) fetch(c0);
   for (int64_t ch = c0; ch < c1; ++ch) {
@@ -291,12 +303,12 @@ __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
 #pragma unroll
     for (int q = 0; q < NB; ++q) {
       const int t = warp + 8 * q, kk = 32 * (t & 1), mt = (t >> 1) & 3, nt = t >> 3;
-      float acc[NW][4];
+      float acc[NW][4], mag[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int w = 0; w < NW; ++w) acc[w][0] = acc[w][1] = acc[w][2] = acc[w][3] = 0.0f;
-      const uint32_t pa = s_u32(Dg + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kDxLD + kk + 8 * (lane >> 4));
-      const uint32_t pb = s_u32(Dg + (64 + 8 * nt + (lane & 7)) * kDxLD + kk + 8 * (lane >> 3));
-      constexpr int stride = 2 * ROWS_D * kDxLD;
+      const uint32_t pa = s_u32(Dg + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kDxK);
+      const uint32_t pb = s_u32(Dg + (64 + 8 * nt + (lane & 7)) * kDxK + 8 * (((kk >> 3) + (lane >> 3)) ^ (lane & 7)));
+      constexpr int stride = 2 * ROWS_D * kDxK;
       uint32_t fb[P][4];   // both k-steps of each digit of F
 #pragma unroll
       for (int p = 0; p < P; ++p) ldsm4(pb + p * stride, fb[p]);
@@ -305,26 +317,42 @@ __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
 #pragma unroll
         for (int p = 0; p < P; ++p) {
           uint32_t fa[4];
-          ldsm4(pa + p * stride + 32 * ks, fa);
+          ldsm4(pa + p * stride + 16 * (((kk >> 3) + 2 * ks + (lane >> 4)) ^ (lane & 7)), fa);
+          if (p == 0) mma_abs(mag, fa, fb[0] + 2 * ks);
 #pragma unroll
           for (int p2 = 0; p2 < P; ++p2)
             if (p + p2 < NW) mma(acc[(p + p2) % NW], fa, fb[p2] + 2 * ks);
         }
+      uint32_t redo = 0;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int x = er[16 * mt + gq + 8 * (e >> 1)] + er[64 + 8 * nt + 2 * tq + (e & 1)] - 2 * LEAD - 56;
+        const int ea = er[16 * mt + gq + 8 * (e >> 1)], eb = er[64 + 8 * nt + 2 * tq + (e & 1)];
+        if (ea == kExpZero || eb == kExpZero) continue;   // a column of zeros
+        if (weak(mag[e], 0x1p-6f, LEAD, c[q][e], ea + eb + 1)) {
+          redo |= 1u << e;
+          continue;
+        }
+        const int x = ea + eb - 2 * LEAD - 56;
         long long hi = 0, lo = 0;
 #pragma unroll
         for (int w = 0; w < 4; ++w) {
           hi = hi * 256 + __float2int_rn(acc[w][e]);
           lo = lo * 256 + __float2int_rn(acc[w + 4][e]);
         }
-        if (hi | lo) {   // (hi 2^32 + lo) 2^x; a column of zeros has no exponent
+        if (hi | lo) {   // (hi 2^32 + lo) 2^x
           const double v = fma((double)hi, 4294967296.0, (double)lo);
           if (x > -900 && x < 900) c[q][e] = fma(v, __hiloint2double((x + 1023) << 20, 0), c[q][e]);
           else c[q][e] += ldexp(v, x);
         }
       }
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (redo >> e & 1) {
+          const int o = 16 * mt + gq + 8 * (e >> 1), j = 8 * nt + 2 * tq + (e & 1);
+          const int n = (int)imin64(32, K - 64 * ch - kk);
+          c[q][e] = dx_dot(raw + (ROWS ? kk * kDxRaw + o : o * kDxRaw + kk), ROWS ? kDxRaw : 1,
+                           F + (64 * ch + kk) * fk + j * fj, fk, n, c[q][e]);
+        }
     }
   }
   // a non-finite value in this block's range: its products as FP64 FMAs
@@ -599,7 +627,7 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
 // W_k from W_{k-1} and G_k), so only these two products see every entry (2 N r
 // FMAs).  One contraction per core (d N r FMAs, and the interfaces of length
 // N_{d-1}) took 4.5 ms for 32^5 of rank 8; this takes 1.2 ms with the two products on the
-// FP64 pipe and 0.63 with them in digit arithmetic.
+// FP64 pipe and 0.76 with them in digit arithmetic.
 cudaError_t launch_reconstruct_backward(const Plan& P, int item, const double* cores, const void* dXt,
                                         int dx_f64, double* dcores, void* ws, cudaStream_t st) {
   const DevItem& it = plan_items_host(&P)[item];
