@@ -979,16 +979,18 @@ __global__ void __launch_bounds__(kThreads) cores_kernel(char* wsb, double* core
 
 // Large cores of a single problem in digit arithmetic: C(a, i, j) += sum_u A(u, a)
 // B(u, i, j) over one K range of slice i (cores_kernel's products; FP64 FMAs bound
-// those: 1.72 per cycle and SM on this GPU, against 1015 BF16 ones, which is 30 FP64
-// products in the 34 digit products kept here).  A block takes 64 contraction
+// those: 1.72 per cycle and SM on this GPU, against 1015 BF16 ones, which is 27 FP64
+// products in the 37 digit products formed here).  A block takes 64 contraction
 // indices at a time: a warp loads one column's 64 values (two per lane), scales
-// them by the column's largest exponent in this chunk and writes their seven
-// balanced base-256 digits (the largest value keeps all 53 bits); every (16 a) x
-// (8 j) tile sums its digit products of weight at most seven exactly in FP32 (64 x 7
-// x 2^14 < 2^24) and adds them to its FP64 sums.  What is dropped is below 2^-57 of
-// the largest product of the chunk, so the result is as exact as FP64 FMAs.
+// them by the column's largest exponent in this chunk and writes their eight
+// balanced base-256 digits (61 bits); every (16 a) x (8 j) tile sums its digit products
+// of weight at most seven exactly in FP32 (8 x 64 x 2^14 < 2^24) and adds them to its
+// FP64 sums.  The pairs left out are below 64 2^-57 of the two largest factors' product; where
+// the factors' magnitudes say that this is not small against sum |A B| (digit::weak, one
+// more product, of the leading digits without their signs), the 64 products are FP64 FMAs.
+// So an entry is held to 2^-44 of sum |A B| at worst, and otherwise is closer than FP64 FMAs.
 // Measured (middle core of 960^3, r = 25, l = 35): H = S M 1.64 ms and Q^T H 3.14 ms
-// -> Q^T S 0.60 ms and (Q^T S) M 0.04 ms.
+// -> Q^T S 0.73 ms (0.60 with seven digits and no test of the terms) and (Q^T S) M 0.04.
 struct CoreGemm {
   const double *A, *B;
   double* C;
@@ -998,14 +1000,19 @@ struct CoreGemm {
   int64_t inner, klen;      // contraction length, the part of one block
   int ra, rb;
 };
-constexpr int kGemmP = 7, kGemmK = 64, kGemmLD = kGemmK + 8;
+constexpr int kGemmP = 8, kGemmK = 64;
+// s + sum_u A(u sau) B(u) in FP64.
+__device__ __noinline__ double core_dot(const double* A, int64_t sau, const double* B, int n, double s) {
+  for (int u = 0; u < n; ++u) s = fma(A[u * sau], B[u], s);
+  return s;
+}
 __global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g) {
   using namespace digit;
-  constexpr int P = kGemmP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P + 1;   // weights kept: 0..7
+  constexpr int P = kGemmP, LEAD = 5, B = 8 * (P - 1) + LEAD, NW = P;   // weights kept: 0..7
   extern __shared__ __align__(16) double sm[];
   const int ma = (g.ra + 15) / 16, nb = (g.rb + 7) / 8, rows = 16 * ma + 8 * nb;
-  uint16_t* D = reinterpret_cast<uint16_t*>(sm);             // [P][rows][kGemmLD]: A's columns, then B's
-  int* er = reinterpret_cast<int*>(D + P * rows * kGemmLD);  // column exponents
+  uint16_t* D = reinterpret_cast<uint16_t*>(sm);             // [P][rows][kGemmK]: A's columns, then B's
+  int* er = reinterpret_cast<int*>(D + P * rows * kGemmK);  // column exponents
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
   const int64_t i = blockIdx.x, k0 = (int64_t)blockIdx.y * g.klen, k1 = imin64(g.inner, k0 + g.klen);
   const double *Ai = g.A + g.sai * i, *Bi = g.B + g.sbi * i;
@@ -1034,7 +1041,7 @@ __global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g
       for (int q = 0; q < 4; ++q) {
         const int r = r0 + q * (kThreads / 32);
         if (r >= rows) break;
-        bad |= (nonfinite(x[q][0]) || nonfinite(x[q][1])) ? 1 : 0;
+        bad |= (undigital(x[q][0]) || undigital(x[q][1])) ? 1 : 0;
         const int m = __reduce_max_sync(0xffffffffu, max(exp_of(x[q][0]), exp_of(x[q][1])));
         if (lane == 0) er[r] = m;
         uint32_t d0[P], d1[P];
@@ -1042,7 +1049,8 @@ __global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g
         digits<P>(fixed<B>(x[q][1], m), d1);
 #pragma unroll
         for (int p = 0; p < P; ++p)
-          *reinterpret_cast<uint32_t*>(D + (p * rows + r) * kGemmLD + 2 * lane) = d0[p] | (d1[p] << 16);
+          *reinterpret_cast<uint32_t*>(D + (p * rows + r) * kGemmK + 8 * ((lane >> 2) ^ (r & 7)) + 2 * (lane & 3)) =
+              d0[p] | (d1[p] << 16);
       }
     }
     __syncthreads();
@@ -1051,45 +1059,57 @@ __global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g
       const int t = warp + q * (kThreads / 32);
       if (t < tiles) {
         const int mt = t % ma, nt = t / ma;
-        float acc[NW][4];
+        float acc[NW][4], mag[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int w = 0; w < NW; ++w) acc[w][0] = acc[w][1] = acc[w][2] = acc[w][3] = 0.0f;
-        const uint32_t pa = s_u32(D + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kGemmLD + 8 * (lane >> 4));
-        const uint32_t pb = s_u32(D + (16 * ma + 8 * nt + (lane & 7)) * kGemmLD + 8 * (lane >> 3));
-        const int stride = 2 * rows * kGemmLD;   // bytes between digit arrays
+        const uint32_t pa = s_u32(D + (16 * mt + (lane & 7) + 8 * ((lane >> 3) & 1)) * kGemmK);
+        const uint32_t pb = s_u32(D + (16 * ma + 8 * nt + (lane & 7)) * kGemmK);
+        const int stride = 2 * rows * kGemmK;   // bytes between digit arrays
 #pragma unroll 1
-        for (int kk = 0; kk < kGemmK; kk += 32) {
+        for (int kk = 0; kk < kGemmK / 8; kk += 4) {   // 16-byte chunks, swizzled by their row
           uint32_t fb[P][4];   // two k-steps of each digit of B
 #pragma unroll
-          for (int p = 0; p < P; ++p) ldsm4(pb + p * stride + 2 * kk, fb[p]);
+          for (int p = 0; p < P; ++p) ldsm4(pb + p * stride + 16 * ((kk + (lane >> 3)) ^ (lane & 7)), fb[p]);
 #pragma unroll
           for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
             for (int p = 0; p < P; ++p) {
               uint32_t fa[4];
-              ldsm4(pa + p * stride + 2 * (kk + 16 * ks), fa);
+              ldsm4(pa + p * stride + 16 * ((kk + 2 * ks + (lane >> 4)) ^ (lane & 7)), fa);
+              if (p == 0) mma_abs(mag, fa, fb[0] + 2 * ks);
 #pragma unroll
               for (int p2 = 0; p2 < P; ++p2)
                 if (p + p2 < NW) mma(acc[(p + p2) % NW], fa, fb[p2] + 2 * ks);
             }
         }
+        uint32_t redo = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int ea = er[16 * mt + gq + 8 * (e >> 1)], eb = er[16 * ma + 8 * nt + 2 * tq + (e & 1)];
+          if (ea == kExpZero || eb == kExpZero) continue;   // a column of zeros
+          if (weak(mag[e], 0x1p-5f, LEAD, c[q][e], ea + eb + 2)) {
+            redo |= 1u << e;
+            continue;
+          }
           long long hi = 0, lo = 0;
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
             hi = hi * 256 + __float2int_rn(acc[w][e]);
             lo = lo * 256 + __float2int_rn(acc[w + 4][e]);
           }
-          // (hi 2^32 + lo) 2^(ea + eb - 2 LEAD - 56); a column of zeros has no exponent
-          if (hi | lo) {
+          if (hi | lo) {   // (hi 2^32 + lo) 2^(ea + eb - 2 LEAD - 56)
             const int x = ea + eb - 2 * LEAD - 56;
             const double v = fma((double)hi, 4294967296.0, (double)lo);
             if (x > -900 && x < 900) c[q][e] = fma(v, __hiloint2double((x + 1023) << 20, 0), c[q][e]);
             else c[q][e] += ldexp(v, x);
           }
         }
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (redo >> e & 1) {
+            const int a = 16 * mt + gq + 8 * (e >> 1), j = 8 * nt + 2 * tq + (e & 1);
+            c[q][e] = core_dot(Ai + u0 * g.sau + a * g.lda, g.sau, Bi + u0 + j * g.ldb, (int)imin64(kGemmK, k1 - u0), c[q][e]);
+          }
       }
     }
   }
@@ -1239,12 +1259,12 @@ bool mid_by_gemm(const Plan& P, int item) {
 
 cudaError_t run_core_gemm(CoreGemm g, int64_t n, int64_t nout, cudaStream_t st) {
   const int rows = (g.ra + 15) / 16 * 16 + (g.rb + 7) / 8 * 8;
-  const size_t smem = 2ul * kGemmP * rows * kGemmLD + sizeof(int) * rows;
+  const size_t smem = 2ul * kGemmP * rows * kGemmK + sizeof(int) * rows;
   static bool attr = false;
   cudaError_t e;
   if (!attr) {
     e = cudaFuncSetAttribute(core_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * kGemmP * 2 * TT_MAXL * kGemmLD + sizeof(int) * 2 * TT_MAXL));
+                             (int)(2 * kGemmP * 2 * TT_MAXL * kGemmK + sizeof(int) * 2 * TT_MAXL));
     if (e != cudaSuccess) return e;
     attr = true;
   }
