@@ -36,8 +36,9 @@
 // one-sided; more accumulators than that do not fit the registers and the
 // 64 x 32 kernel stays).
 //
-// Precision: MMA chains of at most 4 instructions (32 of the contraction, hi and
-// lo), summed in FP32 round-to-nearest over at most kAddsMax of them, then FP64.
+// Precision: 32 of the contraction are a chain of 4 MMA instructions (8 in TF32), the
+// low part of each k-step first; chains are summed in FP32 round-to-nearest, at most kAddsMax
+// = 12 on the column side and 64 on the row side (16 visits of up to 4), then in FP64.
 #include <algorithm>
 #include <cstring>
 

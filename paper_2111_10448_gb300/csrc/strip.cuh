@@ -21,7 +21,11 @@ constexpr int kMaxTA = 128;               // rows of i_1 per strip: one 16-row m
 constexpr int kDescWarp = kWarps - 1;     // describes the tiles, two ahead: the warp with the fewest column rows
 constexpr int kDescLoad = 96;             // what that costs, in row-product columns (planning)
 constexpr int kWarpTasks = 4;             // row products (m-tile, sketch) of one warp and tile, at most
-constexpr int kAddsMax = 32;              // FP32 additions into one accumulator between FP64 flushes
+// FP32 additions into one register accumulator between FP64 flushes: 12 leave the column sums
+// closer than the 64 x 32 tile kernel's, which went to FP64 after each 32 terms (BF16, 112 x 100 x
+// 100 x 112: 1.002e-7 against 1.005e-7; 32 additions 1.26e-7, 16 1.02e-7, 8 0.93e-7).  96^4 x 48, l = 28: 54.1
+// ms with 32, 54.9 with 16, 56.5 with 8, 61.6 with 4.
+constexpr int kAddsMax = 12;
 constexpr int kRowAddsMax = 16;           // the same for the row sketches' shared sums (4 chunks each)
 constexpr int kFmtBF16 = 0, kFmtTF32 = 1, kFmtFP16 = 2;
 
@@ -359,8 +363,10 @@ __device__ __forceinline__ void load_a(uint32_t xs, int ldb, int m0, int k0, uin
   }
 }
 
-// t = X'(m0.., k0..) G(k0.., :) of one k-step (FIRST), or added to t; hi and lo
-// parts of X.
+// t = X'(m0.., k0..) G(k0.., :) of one k-step (FIRST), or added to t; lo and hi
+// parts of X, the low one first: a tensor-core addition loses up to a unit of the last
+// place of its result, and there the result is still small (sums 1.05e-7 off with the high
+// part first, 0.87e-7 so; TF32 2.0e-7, 1.7e-7).
 template <int FMT, int NT, bool FIRST>
 __device__ __forceinline__ void step(float (*t)[4], const uint32_t* xh, const uint32_t* xl, uint32_t gs, int k0) {
   const int lane = threadIdx.x & 31;
@@ -374,9 +380,9 @@ __device__ __forceinline__ void step(float (*t)[4], const uint32_t* xh, const ui
     for (int n = 0; n + 1 < NT; n += 2) ldsm4t(p + 16 * (m ^ (uint32_t)n), b[n / 2]);
     if constexpr (NT & 1) ldsm2t(gs + (k0 + (lane & 15)) * LDG + 16 * (NT - 1), b[NT / 2]);
 #pragma unroll
-    for (int n = 0; n < NT; ++n) mma<FMT, FIRST>(t[n], xh, b[n / 2] + 2 * (n & 1));
+    for (int n = 0; n < NT; ++n) mma<FMT, FIRST>(t[n], xl, b[n / 2] + 2 * (n & 1));
 #pragma unroll
-    for (int n = 0; n < NT; ++n) mma<FMT, false>(t[n], xl, b[n / 2] + 2 * (n & 1));
+    for (int n = 0; n < NT; ++n) mma<FMT, false>(t[n], xh, b[n / 2] + 2 * (n & 1));
   } else {
     const int g = lane >> 2, tq = lane & 3;
     const uint32_t p = gs + (k0 + tq) * LDG + 4 * g;
@@ -387,9 +393,9 @@ __device__ __forceinline__ void step(float (*t)[4], const uint32_t* xh, const ui
       b[n][1] = __float_as_uint(lds_f(p + 32 * n + 4 * LDG));
     }
 #pragma unroll
-    for (int n = 0; n < NT; ++n) mma<FMT, FIRST>(t[n], xh, b[n]);
+    for (int n = 0; n < NT; ++n) mma<FMT, FIRST>(t[n], xl, b[n]);
 #pragma unroll
-    for (int n = 0; n < NT; ++n) mma<FMT, false>(t[n], xl, b[n]);
+    for (int n = 0; n < NT; ++n) mma<FMT, false>(t[n], xh, b[n]);
   }
 }
 
