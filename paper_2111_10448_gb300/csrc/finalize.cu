@@ -20,6 +20,7 @@
 #include "digits.cuh"
 #include "internal.cuh"
 #include "philox.cuh"
+#include "reflector.cuh"
 #include "testmat.cuh"
 
 namespace tts {
@@ -106,43 +107,6 @@ __device__ __forceinline__ double group_sum(double v) {
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
-}
-
-// Reflector of a column with squared norm g over rows i.. and head x0: v = (x0 - alpha,
-// rest), R(i, i) = alpha, beta = 2 / (v^T v) = 1 / (g + |x0| sqrt(g)) (0 for a zero
-// column).  One lane's serial chain in every QR step, so the root and the quotient
-// are Newton iterations from the 20-bit approximate instructions (two each, error
-// 2^-20 -> 2^-40 -> below rounding; five dependent FMAs, where the library's root and
-// division took about 690 and 670 cycles).
-__device__ __forceinline__ void reflector(double g, double x0, double& alpha, double& b, double& v0) {
-  alpha = 0.0, b = 0.0, v0 = 0.0;
-  if (!(g > 0.0)) {
-    if (g == 0.0) return;
-    alpha = v0 = b = g;   // NaN
-    return;
-  }
-  const int e = (__double2hiint(g) >> 20) & 0x7ff;
-  double nx;
-  if (e > 40 && e < 2000) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(g));
-    double s = g * y, h = 0.5 * y;
-    double r = fma(-s, h, 0.5);
-    s = fma(s, r, s);
-    h = fma(h, r, h);
-    r = fma(-s, h, 0.5);
-    nx = fma(s, r, s);
-    const double d = fma(fabs(x0), nx, g);
-    double q;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(d));
-    q = fma(q, fma(-d, q, 1.0), q);
-    b = fma(q, fma(-d, q, 1.0), q);
-  } else {
-    nx = sqrt(g);
-    b = 1.0 / fma(fabs(x0), nx, g);
-  }
-  alpha = -copysign(nx, x0);
-  v0 = x0 - alpha;
 }
 
 // Rows per iteration of a group and the first row of step i.
