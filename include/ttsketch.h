@@ -322,15 +322,17 @@ tt_status tt_pstt2_batched(tt_plan_t plan, const void* const* X_ptrs, void* ws, 
  * values mean 4); chunk = tiles (blocks) a CTA takes from the work counter at
  * a time (>= 1), ctas_per_sm = persistent CTAs per SM (1..32; the small-plane
  * kernel always runs one).  A batch of such items with at most three
- * sketches a side is one launch of the strip kernel, whose split follows from
- * the shapes: the values are kept and have no effect there.  Host only. */
+ * sketches a side is one launch of the strip kernel, which cuts the tensors into
+ * units of 2048 ta chunk entries (ta in {1, 2, 4, 8}; at most 2^17), or with ta = 32 or
+ * 64 (the default) into about four units per CTA slot of the device; ctas_per_sm has
+ * no effect there.  Host only. */
 tt_status tt_plan_batch_config(tt_plan_t plan, int ta, int chunk, int ctas_per_sm);
 
 /* Autotuner of the batched sketch (not in the paper): runs the batched
  * decomposition of X_ptrs once, times the batched sketch launch for every
  * candidate shape (ta in {32, 64} for FP64 plans, chunk in {1, 4, 16},
- * ctas_per_sm in {2, 4, 8}; small-plane batches: ta in {1, 2, 4, 8}, chunk
- * in {1, 4, 8}; CUDA events on `stream`, the second of two runs
+ * ctas_per_sm in {2, 4, 8}; strip and small-plane batches: ta in {1, 2, 4, 8}, chunk
+ * in {1, 4, 8}, of which the strip kernel is timed once per product; CUDA events on `stream`, the second of two runs
  * each) and keeps the fastest in the plan, then runs the decomposition once
  * more with it so that cores and ranks hold a valid result.  Synchronises;
  * refused during stream capture (TT_ERR_STATE).  best_out (host, 3 ints, may

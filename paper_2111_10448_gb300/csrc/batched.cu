@@ -75,9 +75,8 @@ cudaError_t launch_sketch_batched(const Plan& P, const void* const* X, const Bat
   const int nitems = plan_num_items(&P);
   if (nitems > kMaxBatchItems) return cudaErrorNotSupported;
   const StripBatchPlan* sb;
-  int64_t off_args, off_prefix;
-  if (plan_strip_batch(P, &sb, &off_args, &off_prefix))
-    return launch_sketch_strip_batched(P, *sb, off_args, off_prefix, X, ws, st);
+  int64_t off_args;
+  if (plan_strip_batch(P, &sb, &off_args)) return launch_sketch_strip_batched(P, *sb, off_args, cfg, X, ws, st);
   const int t3max = (cfg.ta == 1 || cfg.ta == 2 || cfg.ta == 4 || cfg.ta == 8) ? cfg.ta : 4;
   if (plan_items_host(&P)[0].prec != TT_PREC_FP64 && sp_batched_eligible(P, nullptr, nullptr, t3max))
     return launch_sketch_sp_batched(P, X, cfg, ws, st);

@@ -199,7 +199,7 @@ struct BatchLaunch {
 };
 // Launch shape of the batched sketch (chosen by tt_plan_autotune).
 struct BatchCfg {
-  int ta;            // tile rows along i_1: 32 or 64
+  int ta;            // tile rows along i_1: 32 or 64; 1, 2, 4 or 8: see tt_plan_batch_config
   int chunk;         // tiles per counter grab
   int ctas_per_sm;   // persistent CTAs per SM
 };
@@ -250,18 +250,23 @@ __host__ __device__ constexpr int strip_row_bytes(bool tf32, int nt) {
 __host__ __device__ constexpr int strip_swizzle(int chunks, int r) {
   return (chunks & 1) ? 0 : (chunks & 2) ? (r >> 2) & 1 : chunks == 4 ? (r >> 1) & 3 : r & 7;
 }
-// Batched strip launch: every tensor's arguments and first unit, in the visiting
-// order of the plan (uploaded with the plan tables).
+// Batched strip launch: every tensor's arguments (uploaded with the plan tables) and
+// what its split into units follows from, in the visiting order of the plan.
+struct StripBatchItem {
+  int64_t entries;
+  uint32_t base, npos;   // units are base x ranges of the npos positions
+};
 struct StripBatchPlan {
   std::vector<unsigned char> args;
-  std::vector<uint32_t> prefix;
+  std::vector<StripBatchItem> items;
+  int64_t entries = 0;
   int nt = 2;
   size_t smem = 0;
 };
 bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatchPlan* out);
-cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, int64_t off_prefix,
+cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, const BatchCfg& cfg,
                                         const void* const* X, void* ws, cudaStream_t st);
-bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args, int64_t* off_prefix);
+bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args);
 // The staged rows (st_tab) of every item of a batched plan, lpad elements a row.
 cudaError_t launch_rows_table_batched(char* wsb, int nitems, int lpad, cudaStream_t st);
 bool use_strip_kernel(const Plan& P, int item, int64_t count);

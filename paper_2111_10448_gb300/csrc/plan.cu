@@ -43,7 +43,7 @@ struct Plan {
   BatchCfg bcfg{64, 4, 4};  // batched sketch launch shape (tt_plan_autotune)
   StripBatchPlan strip;              // batched strip launch (strip_ok)
   bool strip_ok = false;
-  int64_t off_strip_args = 0, off_strip_prefix = 0;  // byte offsets of its tables in the workspace
+  int64_t off_strip_args = 0;        // byte offset of its arguments in the workspace
 };
 
 static constexpr int64_t kTableOff = 256;  // bytes
@@ -552,8 +552,6 @@ static void build_blob(Plan& P) {
   if (P.strip_ok) {
     P.off_strip_args = off;
     off += align_up((int64_t)P.strip.args.size(), 64);
-    P.off_strip_prefix = off;
-    off += align_up((int64_t)(sizeof(uint32_t) * P.strip.prefix.size()), 64);
   }
   P.blob.assign((size_t)(off - kTableOff), 0);
   auto put = [&](int64_t at, const void* src, size_t n) {
@@ -564,10 +562,7 @@ static void build_blob(Plan& P) {
   put(t.off_sketches, P.sketches.data(), sizeof(DevSketch) * P.sketches.size());
   for (int L = 0; L < kMaxLev; ++L) put(t.off_tasks[L], P.tasks[L].data(), sizeof(Task) * P.tasks[L].size());
   put(t.off_border, order.data(), sizeof(int) * order.size());
-  if (P.strip_ok) {
-    put(P.off_strip_args, P.strip.args.data(), P.strip.args.size());
-    put(P.off_strip_prefix, P.strip.prefix.data(), sizeof(uint32_t) * P.strip.prefix.size());
-  }
+  if (P.strip_ok) put(P.off_strip_args, P.strip.args.data(), P.strip.args.size());
 }
 
 static tt_status build_all(Plan& P, const tt_problem* probs, int count, int64_t base_doubles) {
@@ -692,10 +687,9 @@ int device_sm_count() {
 // The staged tables of the slab kernel that do not depend on the slab are
 // generated by the first accumulate of a decomposition and reused by the
 // others (begin / tt_pstt2 clear the flag).
-bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args, int64_t* off_prefix) {
+bool plan_strip_batch(const Plan& P, const StripBatchPlan** bp, int64_t* off_args) {
   *bp = &P.strip;
   *off_args = P.off_strip_args;
-  *off_prefix = P.off_strip_prefix;
   return P.strip_ok;
 }
 bool& plan_stream_tables(Plan& P) { return P.stream_tables; }
@@ -1126,11 +1120,12 @@ tt_status tt_plan_autotune(tt_plan_t plan, const void* const* X_ptrs, void* ws, 
   if (s != TT_OK) return s;
   const bool f64 = P->items[0].prec == TT_PREC_FP64;
   std::vector<BatchCfg> cands;
-  if (!f64 && sp_batched_eligible(*P, nullptr, nullptr)) {
-    // small-plane batched kernel (one CTA per SM): the block shape (ta = the
-    // largest number of kR values in a 16-plane block) and the units per grab
+  if (!f64 && (P->strip_ok || sp_batched_eligible(*P, nullptr, nullptr))) {
+    // strip kernel: units of 2048 ta chunk entries; small-plane batched kernel (one CTA
+    // per SM): the block shape (ta = the largest number of kR values in a 16-plane
+    // block) and the units per grab
     for (int t3 : {1, 2, 4, 8})
-      if (sp_batched_eligible(*P, nullptr, nullptr, t3))
+      if (P->strip_ok || sp_batched_eligible(*P, nullptr, nullptr, t3))
         for (int chunk : {1, 4, 8}) cands.push_back(BatchCfg{t3, chunk, 1});
   } else {
     for (int ta : {32, 64}) {
@@ -1168,6 +1163,11 @@ tt_status tt_plan_autotune(tt_plan_t plan, const void* const* X_ptrs, void* ws, 
   int best_i = -1;
   for (size_t c = 0; c < cands.size() && s == TT_OK; ++c) {
     float acc = 0.0f;
+    if (P->strip_ok) {   // the product alone counts
+      bool seen = false;
+      for (size_t b = 0; b < c; ++b) seen = seen || cands[b].ta * cands[b].chunk == cands[c].ta * cands[c].chunk;
+      if (seen) continue;
+    }
     for (int rep = 0; rep < 2 && s == TT_OK; ++rep) {
       s = cuda_status(launch_batch_zero(*P, ws, st));
       if (s == TT_OK) s = cuda_status(cudaEventRecord(e0, st));

@@ -57,7 +57,12 @@ constexpr int kSmemOne = 224 * 1024;   // one per SM
 // with every shared row staged -> with this: 16^4 47 -> 40 us, 9^6 TF32 172 -> 161, 4 x 30 x 30 x
 // 30 x 5 106 -> 92, 512 x 512 45 -> 39; 24^6 and 960^3 stage as before.
 constexpr int64_t kTableQuads = 1 << 19;
-constexpr int64_t kBatchUnit = 1 << 17;  // entries of a batched unit, about
+// Entries of a batched unit: the whole batch over about four units per CTA slot, at least
+// kUnitMin (the row sums of a unit are an FP64 atomic each) and at most kUnitMax.  A batch
+// whose tensors were cut into units of 2^17 whatever their number left most of the slots
+// without one.  Calls of 2 tensors of 10^5 entries, 8 of 10^6, 64 of 10^5, 512 of 10^6 (BF16): 511, 639,
+// 623, 10540 us so, now 154, 318, 402, 10628; the small-plane kernel, tuned, 187, 579, 659, 32300.
+constexpr int64_t kUnitMin = 1 << 11, kUnitMax = 1 << 17, kUnitStep = 1 << 11;
 
 int strip_octets(const Plan& P, int item) {
   const DevItem& it = plan_items_host(&P)[item];
@@ -68,8 +73,8 @@ int strip_octets(const Plan& P, int item) {
 }
 
 // Fills the launch arguments when the kernel serves this call.
-// nt_batch: column octets of a batched launch (0: a launch of its own), whose
-// units are sized by entries, since other tensors fill the SMs beside it.
+// nt_batch: column octets of a batched launch (0: a launch of its own), whose units are
+// sized when it is launched (*units: the least number of them).
 bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt_out, int* nt_out, size_t* smem,
                 int64_t* units, int nt_batch = 0) {
   const DevItem& it = plan_items_host(&P)[item];
@@ -221,7 +226,7 @@ bool plan_strip(const Plan& P, int item, int64_t count, StripArgs* out, int* fmt
   g.nGS = (int)((g.ngt + g.NG - 1) / g.NG);
   // position ranges: about four units per CTA slot
   const int64_t base = (int64_t)g.nA * g.nGS;
-  const int64_t goal = nt_batch ? (it.N[it.d] + kBatchUnit - 1) / kBatchUnit : 4LL * slots;
+  const int64_t goal = nt_batch ? base : 4LL * slots;
   const int64_t want = std::max<int64_t>(1, std::min<int64_t>(g.npos, (goal + base - 1) / base));
   g.CL = (uint32_t)((g.npos + want - 1) / want);
   *units = base * ((g.npos + g.CL - 1) / g.CL);
@@ -304,10 +309,23 @@ cudaError_t launch_sketch_strip(const Plan& P, int item, const void* X, int64_t 
   return cudaGetLastError();
 }
 
+namespace {
+// Units of one tensor of a batch, of about `unit` entries each: base x equal ranges of its
+// positions (sketch_strip_batched_kernel takes the ranges' length from this count).
+int64_t units_of(const StripBatchItem& it, int64_t unit) {
+  const int64_t goal = (it.entries + unit - 1) / unit;
+  const int64_t want = std::max<int64_t>(1, std::min<int64_t>(it.npos, (goal + it.base - 1) / it.base));
+  const int64_t len = (it.npos + want - 1) / want;
+  return it.base * ((it.npos + len - 1) / len);
+}
+}  // namespace
+
 bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatchPlan* out) {
+  int64_t units = 0;
   const int n = plan_num_items(&P);
   out->args.clear();
-  out->prefix.assign(1, 0u);
+  out->items.clear();
+  out->entries = 0;
   out->nt = 2;
   out->smem = 0;
   if (n < 2 || n > kMaxBatchItems) return false;
@@ -318,7 +336,6 @@ bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatch
   }
   if (out->nt > 4) return false;
   out->args.resize((size_t)n * sizeof(strip::StripArgs));
-  int64_t units = 0;
   for (int pos = 0; pos < n; ++pos) {
     strip::StripArgs g;
     int fmt, nt;
@@ -332,14 +349,16 @@ bool strip_plan_batched(const Plan& P, const std::vector<int>& order, StripBatch
     g.total = g.Nd1 * g.cnt;
     std::memcpy(out->args.data() + (size_t)pos * sizeof(g), &g, sizeof(g));
     out->smem = std::max(out->smem, smem);
-    units += u;
-    if (units >= (1LL << 31)) return false;
-    out->prefix.push_back((uint32_t)units);
+    out->items.push_back(StripBatchItem{it.N[it.d], (uint32_t)u, g.npos});
+    out->entries += it.N[it.d];
+    // the finest split of every tensor has to fit a launch
+    if (units_of(out->items.back(), strip::kUnitMin) + units >= (1LL << 31)) return false;
+    units += units_of(out->items.back(), strip::kUnitMin);
   }
   return true;
 }
 
-cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, int64_t off_prefix,
+cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp, int64_t off_args, const BatchCfg& cfg,
                                         const void* const* X, void* ws, cudaStream_t st) {
   const int n = plan_num_items(&P);
   const int prec = plan_items_host(&P)[0].prec;
@@ -352,8 +371,13 @@ cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp,
   strip::StripBatch b;
   b.wsb = (char*)ws;
   b.off_args = off_args;
-  b.off_prefix = off_prefix;
   b.nitems = n;
+  // a shape set by hand or by the tuner, else from the batch
+  const int64_t unit = cfg.ta <= 8 ? strip::kUnitStep * std::min<int64_t>(64, (int64_t)cfg.ta * cfg.chunk)
+                                   : std::min<int64_t>(strip::kUnitMax, std::max<int64_t>(
+                                         strip::kUnitMin, bp.entries / (8LL * device_sm_count())));
+  b.prefix[0] = 0;
+  for (int i = 0; i < n; ++i) b.prefix[i + 1] = b.prefix[i] + (uint32_t)units_of(bp.items[(size_t)i], unit);
   std::memcpy(b.X, X, sizeof(void*) * (size_t)n);
   const strip::BatchFn k = fmt == strip::kFmtTF32   ? strip::batched_tf32(bp.nt)
                            : fmt == strip::kFmtFP16 ? strip::batched_fp16(bp.nt)
@@ -365,7 +389,7 @@ cudaError_t launch_sketch_strip_batched(const Plan& P, const StripBatchPlan& bp,
     attr_set[fmt][bp.nt] = true;
   }
   count_launch();
-  k<<<bp.prefix.back(), strip::kThreads, bp.smem, st>>>(b);
+  k<<<b.prefix[n], strip::kThreads, bp.smem, st>>>(b);
   return cudaGetLastError();
 }
 

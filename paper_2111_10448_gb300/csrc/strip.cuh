@@ -791,12 +791,13 @@ __global__ void __launch_bounds__(kThreads, NCOL * NT <= 12 ? 2 : 1)
 
 // Batched form: one launch over the units of every tensor of a plan, largest
 // tensors first (prefix[] = first unit of each); the arguments of each tensor lie
-// in the workspace, the tensor pointers come by value (a captured launch needs
-// nothing uploaded).
+// in the workspace, the split and the tensor pointers come by value (a captured launch
+// needs nothing uploaded).
 struct StripBatch {
   char* wsb;
-  int64_t off_args, off_prefix;   // byte offsets from wsb
+  int64_t off_args;   // byte offset from wsb
   int nitems;
+  uint32_t prefix[kMaxBatchItems + 1];
   const void* X[kMaxBatchItems];
 };
 template <int FMT, int NT>
@@ -807,11 +808,10 @@ __global__ void __launch_bounds__(kThreads, 2) sketch_strip_batched_kernel(const
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
   __shared__ __align__(16) StripArgs a;
-  const uint32_t* prefix = reinterpret_cast<const uint32_t*>(b.wsb + b.off_prefix);
   int lo = 0, hi = b.nitems - 1;   // position of the tensor of this unit (last prefix <= unit)
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (prefix[mid] <= blockIdx.x) lo = mid;
+    if (b.prefix[mid] <= blockIdx.x) lo = mid;
     else hi = mid - 1;
   }
   const uint32_t* src = reinterpret_cast<const uint32_t*>(b.wsb + b.off_args + (int64_t)lo * sizeof(StripArgs));
@@ -826,9 +826,11 @@ __global__ void __launch_bounds__(kThreads, 2) sketch_strip_batched_kernel(const
     a.wsb = b.wsb;
     a.X = reinterpret_cast<const float*>(b.X[a.item]);
     a.vec = a.vec && ((uintptr_t)a.X & 15) == 0;
+    const uint32_t ranges = (b.prefix[lo + 1] - b.prefix[lo]) / (uint32_t)(a.nA * a.nGS);
+    a.CL = (a.npos + ranges - 1) / ranges;
   }
   __syncthreads();
-  strip_unit<FMT, NT, kMaxCol, false>(a, blockIdx.x - prefix[lo], sm, td, us, &bar, &abort_flag);
+  strip_unit<FMT, NT, kMaxCol, false>(a, blockIdx.x - b.prefix[lo], sm, td, us, &bar, &abort_flag);
 }
 
 using KernelFn = void (*)(const StripArgs);
