@@ -397,7 +397,7 @@ def run_precision(a, dev, P, stream):
         err = err.cpu().numpy()
         r = {"value": X.numel() / (ms * 1e-3), "unit": "entries/s", "ms_per_step": ms,
              "rel_err_vs_X": float((err[0] / err[1]) ** 0.5), "ranks": t.status(stream)[1],
-             "kernel": ["FP64 SIMT", "mma.sync tile", "tcgen05 plane", "small-plane mma.sync"][t.kernel_kind()]}
+             "kernel": t.kernel_name()}
         if form == "fp64":
             ref = t.reconstruct(torch.float32, stream=stream)
         elif ref is not None and not drm:
@@ -527,7 +527,7 @@ def run_second(a, dev, P, stream):
             r.update({"value": ntot / (ms * 1e-3), "unit": "entries/s", "ms_per_step": ms, "ms_runs": runs,
                       "hbm_frac_of_measured": ntot * 4 / (ms * 1e-3) / 1e9 / measured_peaks()[0],
                       "rel_err_vs_X": float((err[0] / err[1]) ** 0.5), "ranks": ranks, "status": st,
-                      "kernel": ["FP64 SIMT", "mma.sync tile", "tcgen05 plane", "small-plane mma.sync"][t.kernel_kind()],
+                      "kernel": t.kernel_name(),
                       "mode": {k: v for k, v in kw.items()}})
             stream.synchronize()
             del t
@@ -579,8 +579,7 @@ def run_onesided(a, dev, P, stream):
                 r[label] = {"value": ntot / (ms * 1e-3), "unit": "entries/s", "ms_per_step": ms, "ms_runs": runs,
                             "rel_err_vs_X": float((err[0] / err[1]) ** 0.5), "ranks": t.status(stream)[1],
                             "sketch_MB": sum(S.numel() for _, _, S in t.sketches(0)) * 8 / 1e6,
-                            "kernel": ["FP64 SIMT", "mma.sync tile", "tcgen05 plane", "small-plane mma.sync"][
-                                t.kernel_kind()]}
+                            "kernel": t.kernel_name()}
                 stream.synchronize()
                 del t
         except Exception as ex:  # reported in the line, the rest of the bench goes on
@@ -629,7 +628,7 @@ def run_tucker(a, dev, P, stream):
         out.update({"tt2tucker_ms": f0.elapsed_time(f1), "tt2tucker_tucker_ranks": [int(A.shape[1]) for A in As]})
         out.update({"ms": e0.elapsed_time(e1), "rel_err_vs_X": float((err[0] / err[1]) ** 0.5),
                     "ranks": t.status(stream)[1], "x_entries_not_formed": n ** 4, "core_entries": G.numel(),
-                    "kernel": ["FP64 SIMT", "mma.sync tile", "tcgen05 plane", "small-plane mma.sync"][t.kernel_kind()]})
+                    "kernel": t.kernel_name()})
         stream.synchronize()
         del t, cores
     except Exception as ex:  # reported in the line, the rest of the bench goes on
@@ -931,9 +930,9 @@ def run_gpu(a):
     normals = sum((ntot // rows) * w for rows, w in shapes)
     tpeak, tkind = measured_tensor_peak(a.prec)
     tflops = ntot * flops_pe / (sketch_ms * 1e-3) / 1e12
-    kind = t.kernel_kind(slab)
-    kname = {2: "sketch_slab_kernel" if slab < 128 else "sketch_tc_kernel", 3: "sketch_sp_kernel",
-             1: "sketch_mma_kernel", 0: "sketch_f64_kernel"}[kind]
+    kname = {"slab": "sketch_slab_kernel", "plane": "sketch_tc_kernel", "strip": "sketch_strip_kernel",
+             "small-plane": "sketch_sp_kernel", "tile": "sketch_mma_kernel", "fp64": "sketch_f64_kernel"}[
+                 t.kernel_name(slab)]
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic_record(f"{kname}_{a.prec}_{a.drm}_{n}x{m}x{m}x{slab}"),
                 "peak_kind": f"{peak_kind} hbm_gbs", "kernel": kname,

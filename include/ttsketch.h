@@ -227,6 +227,12 @@ tt_status tt_plan_sketch_info(tt_plan_t plan, int item, int index, int* type, in
  * takes these shapes, several planes a tile).  Host only. */
 int tt_sketch_kernel_kind(tt_plan_t plan, int64_t count_last);
 
+/* The kernel itself, as static text: "fp64", "plane", "slab", "strip",
+ * "small-plane" or "tile" (64 x 32); for a plan of several problems the one that
+ * the batched sketch launches (count_last is not read).  "" without a plan.
+ * Host only. */
+const char* tt_sketch_kernel_name(tt_plan_t plan, int64_t count_last);
+
 /* Problem of item `item` as stored by the plan (ranks clamped). */
 tt_status tt_plan_problem(tt_plan_t plan, int item, tt_problem* out);
 

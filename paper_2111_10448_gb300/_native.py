@@ -66,6 +66,7 @@ _SIGS = {
     "tt_plan_sketch_info": (C.c_int, [_P, C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_int),
                                       C.POINTER(C.c_int64), C.POINTER(C.c_int), C.POINTER(C.c_int64)]),
     "tt_sketch_kernel_kind": (C.c_int, [_P, C.c_int64]),
+    "tt_sketch_kernel_name": (C.c_char_p, [_P, C.c_int64]),
     "tt_pstt2": (C.c_int, [_P, _P, _P, _P, _P, _P]),
     "tt_pstt2_noalloc": (C.c_int, [_P, _P, _P, _P, _P, _P]),
     "tt_plan_batch_config": (C.c_int, [_P, C.c_int, C.c_int, C.c_int]),

@@ -200,6 +200,12 @@ class TTSketch:
         c = self.dims[-1] if count_last is None else count_last
         return N.lib().tt_sketch_kernel_kind(self.plan, int(c))
 
+    def kernel_name(self, count_last=None):
+        """The sketch kernel itself: 'fp64', 'plane', 'slab', 'strip', 'small-plane' or 'tile' (of a
+        batch: the one that its launch uses)."""
+        c = self.dims[-1] if count_last is None else count_last
+        return N.lib().tt_sketch_kernel_name(self.plan, int(c)).decode()
+
     # ---------------------------------------------------------------- status
     def status(self, stream=None):
         st = C.c_int()

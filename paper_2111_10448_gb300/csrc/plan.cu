@@ -803,6 +803,19 @@ int tt_sketch_kernel_kind(tt_plan_t plan, int64_t count_last) {
   return use_sp_kernel(*P, 0, count_last) ? 3 : 1;
 }
 
+const char* tt_sketch_kernel_name(tt_plan_t plan, int64_t count_last) {
+  Plan* P = as_plan(plan);
+  if (!P || P->items.empty()) return "";
+  if (P->items[0].prec == TT_PREC_FP64) return "fp64";
+  if (P->items.size() > 1)
+    return P->strip_ok ? "strip" : sp_batched_eligible(*P, nullptr, nullptr) ? "small-plane" : "tile";
+  if (use_tc_kernel(*P, 0, count_last)) return "plane";
+  if (use_slab_kernel(*P, 0, count_last)) return "slab";
+  const bool sp = use_sp_kernel(*P, 0, count_last);
+  if (sp && P->sketches[P->items[0].sk0].kr_nm) return "small-plane";
+  return use_strip_kernel(*P, 0, count_last) ? "strip" : sp ? "small-plane" : "tile";
+}
+
 tt_status tt_plan_problem(tt_plan_t plan, int item, tt_problem* out) {
   Plan* P = as_plan(plan);
   if (!P || !out || item < 0 || item >= (int)P->probs.size()) return TT_ERR_INVALID_ARG;
@@ -842,10 +855,8 @@ tt_status tt_pstt2_accumulate(tt_plan_t plan, const void* slab, int64_t first_la
   for (int64_t i = first_last; i < first_last + count_last; ++i)
     if (P->slab_seen[(size_t)i]) return TT_ERR_STATE;
   if (log_on()) {
-    static const char* kKind[] = {"FP64 SIMT", "generic mma.sync tile", "tcgen05", "small-plane mma.sync"};
-    const int kind = tt_sketch_kernel_kind(plan, count_last);
     TT_LOGF("plan %llu accumulate slices [%lld, %lld): %s kernel", (unsigned long long)P->id, (long long)first_last,
-            (long long)(first_last + count_last), kKind[kind & 3]);
+            (long long)(first_last + count_last), tt_sketch_kernel_name(plan, count_last));
   }
   tt_status s = accumulate(*P, 0, slab, first_last, count_last, ws, (cudaStream_t)stream);
   if (s != TT_OK) return s;
