@@ -582,15 +582,19 @@ cudaError_t launch_reconstruct(const Plan& P, int item, const double* cores, voi
   const int ds = it.ds;
   const int64_t Nm = it.N[ds], Mm = it.N[it.d] / it.N[ds];
   // Digit arithmetic (expand.cuh) for FP32 data from 3 2^18 entries on, with both
-  // interfaces at least as long as a staging step.  Measured (whole call, us, FP64
-  // kernel -> digit kernel): below the line 64^3 rank 2: 8 -> 11, 9^6 rank 8: 23 ->
-  // 26; above it 1000 x 1000 rank 3: 12.8 -> 12.2, 100^3 rank 10: 28 -> 17, 128^3
-  // rank 10: 50 -> 18, 200^3 rank 24: 376 -> 94, 256^4 rank 6: 51300 -> 8880 (4770
-  // with five digits, which left entries far below their row's and column's scale without
-  // correct bits; 16 warps an SM wait on their own chains, half of the issue slots used);
-  // error sums 24^6 rank 10: 4590 -> 1117 (923 with seven digits and residuals in FP32
-  // pairs, which were further off than FP64 ones).
-  if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && Nm * Mm >= (3 << 18)) {
+  // interfaces at least as long as a staging step and enough FP64 products to spare, entries x
+  // rank: 3 2^21 for the output, 3 2^20 for the error sums.  Measured (whole call, us, FP64
+  // kernel -> digit kernel): output, below the line 900 x 900 rank 3 18.5 -> 22.8, 1000 x 1000 rank 3
+  // 19.9 -> 23.3, 93^3 rank 2 20.7 -> 27.1; above it 900 x 900 rank 8 24.8 -> 22.8, 30^4 rank 8 33.0 ->
+  // 31.1, 128^3 rank 10 58 -> 33, 200^3 rank 2 62 -> 42, rank 24 385 -> 131, 256^4 rank 6 51300 -> 8880
+  // (4770 with five digits, which left entries far below their row's and column's scale without
+  // correct bits; 16 warps an SM wait on their own chains, half of the issue slots used).
+  // Error sums, below 900 x 900 rank 1 35.1 -> 36.1, 93^3 rank 2 39.4 -> 40.1; above 64 x 12500 rank 4
+  // 39.1 -> 32.6, 30^4 rank 8 52 -> 44, 200^3 rank 2 117 -> 74, 24^6 rank 10 4590 -> 1117 (923 with
+  // seven digits and residuals in FP32 pairs, which were further off than FP64 ones).
+  const int64_t entries = Nm * Mm;
+  if ((Xt ? !x_f64 : !cmp_f64) && Nm >= 64 && Mm >= 64 && entries >= (3 << 18) &&
+      entries * it.rpad[ds] >= (Xt ? 3 << 21 : 3 << 20)) {
     expand::ExpandArgs a;
     a.L = W + it.off_L[ds];
     a.Rt = W + it.off_Rt[ds + 1];
