@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kThreads) dense_kernel(const double* L, const 
   }
 }
 
-// Y(row, c) += sum_v dX(row + Nk v) Rt(c, v)   (Rt: rp x Mk, ld rp; Rt = null: 1).
+// Y(row, c) += sum_v dX(row + Nk v) Rt(c, v)   (Rt: rp x Mk, ld rp).
 // A job is 32 consecutive rows (the lanes) x vc consecutive v; the four warps
 // of a block take consecutive jobs of the same rows, add their partial sums in
 // shared memory and the block adds them into Y (FP64 atomics).  RP >= rp is a
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(128) ygram_kernel(const void* dX, int dx_f64, 
         const double x = dx_f64 ? __ldg((const double*)dX + idx) : (double)__ldg((const float*)dX + idx);
 #pragma unroll
         for (int c = 0; c < RP; ++c)
-          if (c < rp) acc[c] += x * (Rt ? __ldg(Rt + c + (int64_t)rp * v) : 1.0);
+          if (c < rp) acc[c] += x * __ldg(Rt + c + (int64_t)rp * v);
       }
     }
     __syncthreads();

@@ -1501,7 +1501,8 @@ cudaError_t launch_sketch_mixed(const Plan& P, int item, const void* X, int64_t 
   // Khatri-Rao sketch does not allow (it is scaled per plane)
   if (plan_sketches_host(&P)[plan_items_host(&P)[item].sk0].kr_nm && use_sp_kernel(P, item, count))
     return launch_sketch_sp(P, item, X, first, count, ws, st);
-  if (use_strip_kernel(P, item, count)) return launch_sketch_strip(P, item, X, first, count, ws, st);
+  const cudaError_t e = launch_sketch_strip(P, item, X, first, count, ws, st);
+  if (e != cudaErrorNotSupported) return e;
   if (use_sp_kernel(P, item, count)) return launch_sketch_sp(P, item, X, first, count, ws, st);
   return launch_sketch_mma(P, item, X, first, count, ws, st);
 }

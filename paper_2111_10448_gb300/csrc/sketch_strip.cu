@@ -1,6 +1,6 @@
 // Strip kernel (strip.cuh): host side.
 //
-// The fused multi-sketch for shapes outside the tcgen05 and small-plane
+// The fused multi-sketch for shapes outside the tcgen05
 // kernels: X = stack of planes X(:, w, :), w = kL + WL kR, every entry of X
 // read once and fed to every sketch (internal.cuh states the products).
 //
@@ -19,7 +19,7 @@
 // (cp.async) while this one is multiplied; two CTAs per SM overlap one's staging
 // with the other's products.
 //
-// What bounds it: issue slots, of which 53-60 % are used (16 warps an SM leave
+// What bounds it: issue slots, of which 54 % are used (96^4 x 6; 16 warps an SM leave
 // barriers and dependent chains uncovered).  At 96^4 x 48, l = 28, leaving one part out
 // saved: the normals 7.6 of 32.7 ms (5.3 since they take fewer slots), the rest of the
 // staging 5, conversion 4, copies of X 2, column products 2.2, row products 3.7.
@@ -27,14 +27,15 @@
 // entry) is busy 15 %.
 //
 // Measured (one accumulate, BF16 unless named; the 64 x 32 tile kernel that served
-// these shapes before in brackets): 960^3, l = 35: 3.28 ms (13.0); 64^5, l = 28:
-// 7.4 ms (26); 300^3, l = 60: 0.375 ms (0.79), TF32 0.53 (0.87); 200 x 128 x 100 x
-// 80, l = 16, FP16 Khatri-Rao: 1.03 ms (4.33); 16 x 300 x 300: 0.072 ms (0.150).
-// 24^6, l = 26: 2.68 ms (small-plane kernel: 10.7).
+// these shapes before in brackets): 960^3, l = 35: 3.32 ms (13.0); 64^5, l = 28:
+// 7.5 ms (26); 300^3, l = 60: 0.362 ms (0.79), TF32 0.51 (0.87); 200 x 128 x 100 x
+// 80, l = 16, FP16 Khatri-Rao: 1.03 ms (4.33); 16 x 300 x 300: 0.048 ms (0.150).
+// 24^6, l = 26: 2.70 ms (small-plane kernel: 10.7); 96^4 x 48, l = 28: 30.0.
 // No shape tried was slower, down to 8^3, 9 x 9 x 1000 and 2 x 1000 x 1000, so every
-// call with at most three sketches a side takes it (d <= 6 two-sided, d <= 4
+// call with one to three sketches a side takes it (d <= 6 two-sided, d <= 4
 // one-sided; more accumulators than that do not fit the registers and the
-// 64 x 32 kernel stays).
+// small-plane and 64 x 32 kernels stay, as for plans with no sketch on one side:
+// one-sided two-pass and d = 2 two-pass; and for Khatri-Rao small planes).
 //
 // Precision: 32 of the contraction are a chain of 4 MMA instructions (8 in TF32), the
 // low part of each k-step first; chains are summed in FP32 round-to-nearest, at most kAddsMax

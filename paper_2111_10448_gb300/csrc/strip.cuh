@@ -2,8 +2,9 @@
 // sketch_strip_<format>.cu instantiate it, sketch_strip.cu plans the launch.
 //
 // The fused multi-sketch (BF16, FP16 or TF32 tensor cores, X split into hi +
-// lo) for every shape that neither the tcgen05 kernels nor the small-plane
-// kernel take.  See sketch_strip.cu for the split of the work.
+// lo) for the shapes that the tcgen05 kernels do not take, with one to three sketches
+// a side (of small planes, n_1 and n_d <= 32: dense test matrices).  See sketch_strip.cu
+// for the split of the work.
 #pragma once
 #include <cstdint>
 
@@ -19,7 +20,9 @@ constexpr int kThreads = 256, kWarps = 8;
 constexpr int kMaxCol = 3, kMaxRow = 3;   // sketches a side
 constexpr int kMaxTA = 128;               // rows of i_1 per strip: one 16-row m-tile per warp
 constexpr int kDescWarp = kWarps - 1;     // describes the tiles, two ahead: the warp with the fewest column rows
-constexpr int kDescLoad = 96;             // what that costs, in row-product columns (planning)
+// What that costs, in row-product columns (planning): 200 changed nothing at 960^3, 24^6, 96^4 x 48 and
+// 61 x 53 x 67 x 47, so it only has to be of a row product's size.
+constexpr int kDescLoad = 96;
 constexpr int kWarpTasks = 4;             // row products (m-tile, sketch) of one warp and tile, at most
 // FP32 additions into one register accumulator between FP64 flushes: 12 leave the column sums
 // closer than the 64 x 32 tile kernel's, which went to FP64 after each 32 terms (BF16, 112 x 100 x
@@ -149,12 +152,6 @@ struct TileDesc {
   uint32_t fwlo[kMaxCol];            // ... to the rows of this w mod wdiv
 };
 
-// Asynchronous copies of one tile of X into the raw buffer: row (q, b) holds the
-// entries of plane row q at i_d = b0 + b, nl runs of n_1 (consecutive kL: one
-// contiguous run).  Rows that do not start on 16 bytes (a.vec = 0) are copied from
-// the 16-byte boundary below, so entry i of a row lies at word (start word mod 4) +
-// i; no copy leaves the slab.  (One bulk copy per row, 256 to 512 bytes each, was
-// slower: 960^3 5.2 ms against 3.4.)
 // Per CTA and unit: the cursor over the tiles (kDescWarp's) and every warp's row products.
 struct UnitState {
   uint32_t i2, i3, rg, rlo;
@@ -172,6 +169,12 @@ struct LaneMap {   // chunk (four words) and first item of this lane, items per 
   __device__ __forceinline__ int i0() const { return (v >> 8) & 255; }
   __device__ __forceinline__ int np() const { return v >> 16; }
 };
+// Asynchronous copies of one tile of X into the raw buffer: row (q, b) holds the
+// entries of plane row q at i_d = b0 + b, nl runs of n_1 (consecutive kL: one
+// contiguous run).  Rows that do not start on 16 bytes (a.vec = 0) are copied from
+// the 16-byte boundary below, so entry i of a row lies at word (start word mod 4) +
+// i; no copy leaves the slab.  (One bulk copy per row, 256 to 512 bytes each, was
+// slower: 960^3 5.2 ms against 3.4.)
 __device__ __forceinline__ void issue_x(const StripArgs& a, const TileDesc& d, float* raw, const LaneMap& m) {
   const int run = a.PL > 1 ? d.nl * (int)a.n1 : d.ta, nrow = d.nr * d.tb;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -202,19 +205,10 @@ __device__ __forceinline__ void issue_x(const StripArgs& a, const TileDesc& d, f
   }
 }
 
-template <int FMT>
-__device__ __forceinline__ void put_split2(const StripArgs& a, float x0, float x1, char* h, char* l) {
-  if constexpr (FMT == kFmtTF32) {
-    const float2 hi = make_float2(round_tf32(x0), round_tf32(x1));
-    *reinterpret_cast<float2*>(h) = hi;
-    *reinterpret_cast<float2*>(l) = make_float2(round_tf32(__fsub_rn(x0, hi.x)), round_tf32(__fsub_rn(x1, hi.y)));
-  } else {
-    if constexpr (FMT == kFmtFP16) {
-      x0 = __fmul_rn(x0, a.xscale);
-      x1 = __fmul_rn(x1, a.xscale);
-    }
-    tc::split_hi_lo<FMT == kFmtFP16>(x0, x1, *reinterpret_cast<uint32_t*>(h), *reinterpret_cast<uint32_t*>(l));
-  }
+__device__ __forceinline__ void put_split2_tf32(float x0, float x1, char* h, char* l) {
+  const float2 hi = make_float2(round_tf32(x0), round_tf32(x1));
+  *reinterpret_cast<float2*>(h) = hi;
+  *reinterpret_cast<float2*>(l) = make_float2(round_tf32(__fsub_rn(x0, hi.x)), round_tf32(__fsub_rn(x1, hi.y)));
 }
 
 // The raw tile into hi and lo parts [b][a].  Everything inside the valid planes'
@@ -251,8 +245,8 @@ __device__ __forceinline__ void convert_x(const StripArgs& a, const TileDesc& d,
         }
         const int o = drow + E * (p * a.n1p + 4 * q0);
         if constexpr (FMT == kFmtTF32) {
-          put_split2<FMT>(a, v.x, v.y, xh + o, xl + o);
-          put_split2<FMT>(a, v.z, v.w, xh + o + 8, xl + o + 8);
+          put_split2_tf32(v.x, v.y, xh + o, xl + o);
+          put_split2_tf32(v.z, v.w, xh + o + 8, xl + o + 8);
         } else {
           if constexpr (FMT == kFmtFP16) {
             v.x = __fmul_rn(v.x, a.xscale);
