@@ -5,7 +5,7 @@ namespace tts {
 
 // Reflector of a column with squared norm g over rows i.. and head x0: v = (x0 - alpha,
 // rest), R(i, i) = alpha, beta = 2 / (v^T v) = 1 / (g + |x0| sqrt(g)) (0 for a zero
-// column).  One lane's serial chain in every QR step, so the root and the quotient
+// column and for one with a NaN).  One lane's serial chain in every QR step, so the root and the quotient
 // are Newton iterations from the 20-bit approximate instructions (two each: five dependent
 // FMAs, where the library's root and division took about 690 and 670 cycles).  The last
 // step of each adds the correction from the residual, g - s^2 and 1 - d q, to the iterate
@@ -15,11 +15,7 @@ namespace tts {
 // the roots one unit off.)
 __device__ __forceinline__ void reflector(double g, double x0, double& alpha, double& b, double& v0) {
   alpha = 0.0, b = 0.0, v0 = 0.0;
-  if (!(g > 0.0)) {
-    if (g == 0.0) return;
-    alpha = v0 = b = g;   // NaN
-    return;
-  }
+  if (!(g > 0.0)) return;
   const int e = (__double2hiint(g) >> 20) & 0x7ff;
   double nx;
   if (e > 40 && e < 2000) {
