@@ -80,7 +80,9 @@ __device__ __forceinline__ void mma_abs(float* c, const uint32_t* a, const uint3
 // of the leading digits, full scale 2^LEAD each; a digit that is not zero is at most twice its
 // value, so the terms' magnitudes add up to at least mag 2^(-2 LEAD) / 4 of the two largest factors'
 // product.  Below `part` of that they may be as small as what the digits drop; then the
-// digits still serve if they are exact below the last bit of the sum so far, |sum| >= 2^e.
+// digits still serve if that, K 2^-57 of the factors' product for K terms, is no more than K
+// FP64 additions may lose of the sum so far, K 2^-53 |sum|: |sum| >= 2^e, e four below the
+// factors' exponents.
 __device__ __forceinline__ bool weak(float mag, float part, int lead, double sum, int e) {
   return mag < part * (float)(1 << (2 * lead)) && exp_of(sum) <= e;
 }

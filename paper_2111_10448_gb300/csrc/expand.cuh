@@ -26,7 +26,8 @@
 // half-ulp of the FP64 sum rounded once, however far it lies below its row's and column's
 // scale -- localised components that are large in different places, cancellation.
 // For random factors one entry in 10^4 is summed again; where all are (components that
-// nowhere meet) the call costs what the FP64 form did and the digits besides.
+// nowhere meet) the call costs what the FP64 form did and the digits besides (4000 x 4000,
+// rank 16: 86 us for random factors, 625 for such, 467 in FP64 throughout).
 //
 // Error sums: a residual is x minus the three-word sum of the weights, squares and sums are
 // held in words of their own (below), so that neither the residuals nor the sums are further

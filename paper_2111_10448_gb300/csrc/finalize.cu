@@ -967,6 +967,7 @@ struct CoreGemm {
 constexpr int kGemmP = 8, kGemmK = 64;
 // s + sum_u A(u sau) B(u) in FP64.
 __device__ __noinline__ double core_dot(const double* A, int64_t sau, const double* B, int n, double s) {
+#pragma unroll 8
   for (int u = 0; u < n; ++u) s = fma(A[u * sau], B[u], s);
   return s;
 }
@@ -1051,7 +1052,7 @@ __global__ void __launch_bounds__(kThreads, 2) core_gemm_kernel(const CoreGemm g
         for (int e = 0; e < 4; ++e) {
           const int ea = er[16 * mt + gq + 8 * (e >> 1)], eb = er[16 * ma + 8 * nt + 2 * tq + (e & 1)];
           if (ea == kExpZero || eb == kExpZero) continue;   // a column of zeros
-          if (weak(mag[e], 0x1p-5f, LEAD, c[q][e], ea + eb + 2)) {
+          if (weak(mag[e], 0x1p-5f, LEAD, c[q][e], ea + eb - 4)) {
             redo |= 1u << e;
             continue;
           }

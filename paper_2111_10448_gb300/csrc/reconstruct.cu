@@ -216,7 +216,9 @@ __global__ void __launch_bounds__(128) wgram_kernel(const void* dX, int dx_f64, 
 // row instead of padded: two CTAs an SM up to NB = 4.)
 // Measured (the whole adjoint, FP64 products and these): 32^5 of rank 8 1.22 -> 0.76 ms,
 // 64^4 of rank 16 1.15 -> 0.57, 48^4 of rank 40 1.30 -> 0.57, 32^4 of rank 8 120 -> 87 us (0.62, 0.47,
-// 0.50 ms and 83 us with seven digits and no test of the terms).
+// 0.50 ms and 83 us with seven digits and no test of the terms; where every sum
+// is formed in FP64 after all, 4000 x 4000 takes 0.80 ms at rank 6, 1.39 at 16, 3.6 at 40, FP64 throughout 0.93,
+// 1.49, 3.0).
 // Entries from which they serve (FP32 dX, both sides at least one tile wide): 512 x 512 of
 // rank 8 72 -> 47 us, 256 x 256 74 -> 47, of rank 32 109 -> 67.
 constexpr int64_t kDxMin = 1 << 16;
@@ -232,6 +234,7 @@ __device__ __forceinline__ double widen(float x) {
 }
 // s + sum_k x(k) F(k) in FP64.
 __device__ __noinline__ double dx_dot(const float* x, int sx, const double* F, int64_t fk, int n, double s) {
+#pragma unroll 8
   for (int k = 0; k < n; ++k) s = fma((double)x[k * sx], __ldg(F + k * fk), s);
   return s;
 }
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(256, NB <= 4 ? 2 : 1)
       for (int e = 0; e < 4; ++e) {
         const int ea = er[16 * mt + gq + 8 * (e >> 1)], eb = er[64 + 8 * nt + 2 * tq + (e & 1)];
         if (ea == kExpZero || eb == kExpZero) continue;   // a column of zeros
-        if (weak(mag[e], 0x1p-6f, LEAD, c[q][e], ea + eb + 1)) {
+        if (weak(mag[e], 0x1p-6f, LEAD, c[q][e], ea + eb - 4)) {
           redo |= 1u << e;
           continue;
         }
