@@ -211,7 +211,7 @@ tt_status tt_plan_sketch_info(tt_plan_t plan, int item, int index, int* type, in
 
 /* Which sketch kernel an accumulate of `count_last` last-mode slices runs for
  * item 0: 0 = FP64 SIMT kernel, 1 = generic tensor-core kernel (mma.sync,
- * any shape: the strip kernel where there are at most three sketches a side,
+ * any shape: the strip kernel where there are one to three sketches a side,
  * else 64 x 32 tiles; test-matrix rows that several tiles read are staged once
  * per call where they find room in scratch), 2 = a tcgen05
  * kernel: the plane kernel (n_1 and count_last in {128, 256}, d in {3, 4},

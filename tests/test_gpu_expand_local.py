@@ -75,6 +75,22 @@ def test_fp32_output_cancellation(r):
     assert np.median(np.abs(ref)) < 2.0 ** -18
 
 
+@pytest.mark.parametrize("r", [8, 16, 40, 60])
+@pytest.mark.parametrize("e", [6, 14, 22])
+def test_fp32_output_coherent_digits(r, e):
+    """Every digit of half the factors +127 (what is dropped adds up), cancelled down to 2^-e by factors
+    whose digits end after the third."""
+    n, m = 1030, 801
+    rng = np.random.default_rng(e)
+    a = sum(127.0 * 256.0 ** -i for i in range(1, 7))
+    L = np.full((n, r), a) * 2.0 ** rng.integers(0, 2, (n, 1))
+    R = np.full((r, m), a)
+    b = np.round(a * a * 2 ** 20) / 2 ** 20
+    L[:, r // 2:] = np.sign(L[:, r // 2:]) * 0.5 * L[:, :1] / a
+    R[r // 2:] = -2.0 * b * (1 - 2.0 ** -e * rng.integers(1, 4, (1, m)))
+    _check(_plan(n, m, r), L, R)
+
+
 @pytest.mark.parametrize("scale", [-140, -120, 120])
 def test_fp32_output_ends_of_the_range(scale):
     n, m, r = 1100, 1000, 6
